@@ -14,47 +14,33 @@
 namespace ceedbp {
 cudaError_t launch_elem_bp1(const DeviceMesh& m, const ElemArgs& a, cudaStream_t s);
 cudaError_t launch_elem_bp3(const DeviceMesh& m, const ElemArgs& a, cudaStream_t s);
-cudaError_t launch_elem_bp5(const DeviceMesh& m, const ElemArgs& a, cudaStream_t s);
-cudaError_t launch_elem_bp6(const DeviceMesh& m, const ElemArgs& a, cudaStream_t s);
 int elem_blocks_bp1(const DeviceMesh& m);
 cudaError_t launch_elem_bp2(const DeviceMesh& m, const ElemArgs& a, cudaStream_t s);
 cudaError_t launch_elem_bp4(const DeviceMesh& m, const ElemArgs& a, cudaStream_t s);
 int elem_blocks_bp4(const DeviceMesh& m);
 int elem_blocks_bp3(const DeviceMesh& m);
-int elem_blocks_bp5(const DeviceMesh& m);
-int elem_blocks_bp6(const DeviceMesh& m);
 
+// batched BP5 solves: even-odd kernel at odd orders, column kernel at even ones
 cudaError_t launch_elem_eo(const DeviceMesh& m, const ElemArgs& a, cudaStream_t s);
-int elem_eo_blocks(const DeviceMesh& m);
-bool elem_eo_available(const DeviceMesh& m);
-
-// Collocated FP64 stiffness with even p1 (odd order) uses the even-odd kernel
-// when its shape is resident on an SM (large p1 with three components is not).
-static bool use_even_odd(const DeviceMesh& m) { return m.colloc && (m.p1 % 2 == 0) && elem_eo_available(m); }
+cudaError_t launch_elem_bp5(const DeviceMesh& m, const ElemArgs& a, cudaStream_t s);
+int elem_eo_per_block_rt(const DeviceMesh& m);
+int elem_per_block_bp5(const DeviceMesh& m);
 
 cudaError_t launch_elem(const DeviceMesh& m, int kind, const ElemArgs& a, cudaStream_t s) {
   if (kind == kStiff && m.X != nullptr) return launch_elem_rc(m, a, s);
-  if (kind == kStiff && use_even_odd(m)) return launch_elem_eo(m, a, s);
-  if (m.colloc && kind == kStiff) return m.ncomp == 3 ? launch_elem_bp6(m, a, s) : launch_elem_bp5(m, a, s);
+  if (a.blk_prob != nullptr) return m.p1 % 2 == 0 ? launch_elem_eo(m, a, s) : launch_elem_bp5(m, a, s);
+  if (m.colloc && kind == kStiff) return launch_elem_fx(m, a, s);
   if (!m.colloc && kind == kStiff) return m.ncomp == 3 ? launch_elem_bp4(m, a, s) : launch_elem_bp3(m, a, s);
   if (!m.colloc && kind == kMass) return m.ncomp == 3 ? launch_elem_bp2(m, a, s) : launch_elem_bp1(m, a, s);
   return cudaErrorInvalidValue;
 }
 
-int elem_eo_per_block_rt(const DeviceMesh& m);
-int elem_per_block_bp5(const DeviceMesh& m);
-
-int elem_stiff_per_block(const DeviceMesh& m) {
-  if (m.X != nullptr) return 0;
-  if (use_even_odd(m)) return elem_eo_per_block_rt(m);
-  return m.colloc && m.ncomp == 1 ? elem_per_block_bp5(m) : 0;
-}
+int elem_batch_per_block(const DeviceMesh& m) { return m.p1 % 2 == 0 ? elem_eo_per_block_rt(m) : elem_per_block_bp5(m); }
 
 int elem_blocks(const DeviceMesh& m) {
   // stiffness and mass instantiations of one (p1, q) share the block shape
   if (m.X != nullptr) return elem_rc_blocks(m);
-  if (use_even_odd(m)) return std::max(elem_eo_blocks(m), m.ncomp == 3 ? elem_blocks_bp6(m) : elem_blocks_bp5(m));
-  if (m.colloc) return m.ncomp == 3 ? elem_blocks_bp6(m) : elem_blocks_bp5(m);
+  if (m.colloc) return elem_fx_blocks(m);
   return m.ncomp == 3 ? elem_blocks_bp4(m) : elem_blocks_bp3(m);
 }
 }  // namespace ceedbp
@@ -72,7 +58,7 @@ thread_local std::string g_setup_error;
 // only the direct schedules take.
 int pair_shape_candidates(const ceedbp_ctx* c, const DeviceMesh& m, int* eb, int* st, int* ns, int cap) {
   int n = elem_df_tile_candidates(m, eb, st, ns, cap, true);
-  if (!c->pipelined_only) {
+  if (!c->batch_group) {
     const int k = elem_dfeo_candidates(m, eb + n, ns + n, cap - n);
     for (int q = 0; q < k; ++q) st[n + q] = 3;
     n += k;
@@ -108,7 +94,7 @@ void release(ceedbp_ctx* c) {
   void* ptrs[] = {c->d_l2g, c->d_off, c->d_slots, c->d_basis, c->d_G, c->d_Mq, c->d_dinv, c->d_mdiag,
                   c->d_wl, c->d_r, c->d_p, c->d_ax, c->d_part_apply, c->d_part_vec, c->d_state,
                   c->d_Gdf, c->d_Ddf, c->d_dinvdf, c->d_G32, c->d_Gbf, c->d_dinv32, c->d_xin,
-                  c->d_rin, c->d_pin, c->d_outer, c->d_Ghat, c->d_scal, c->d_X, c->d_l2g_id};
+                  c->d_rin, c->d_pin, c->d_outer, c->d_Ghat, c->d_scal, c->d_X, c->d_l2g_id, c->d_Gfx, c->d_gexp};
   for (void* p : ptrs)
     if (p) cudaFree(p);
   if (c->h_outer) cudaFreeHost(c->h_outer);
@@ -118,6 +104,29 @@ void release(ceedbp_ctx* c) {
   if (c->ev1) cudaEventDestroy(c->ev1);
   for (cudaEvent_t e : c->prof) cudaEventDestroy(e);
   c->prof.clear();
+}
+
+// Fixed-point copy of the stiffness factors for the FP64 element kernel (elem_fx.cuh): as large as
+// the factors themselves, so it is kept only while it takes at most a quarter of the free memory;
+// without it the kernel runs in FP64.
+ceedbp_status prepare_fx(ceedbp_ctx* c) {
+  DeviceMesh& m = c->mesh;
+  const size_t q3 = size_t(c->q) * c->q * c->q, bytes = sizeof(int4) * 3 * size_t(m.nelem) * q3;
+  if (!c->d_Gfx) {
+    size_t free_b = 0, total_b = 0;
+    CK(c, cudaMemGetInfo(&free_b, &total_b));
+    if (bytes > free_b / 4) return CEEDBP_OK;
+    if (dalloc(&c->d_Gfx, bytes / sizeof(int4)) != cudaSuccess || dalloc(&c->d_gexp, size_t(m.nelem)) != cudaSuccess) {
+      cudaGetLastError();
+      if (c->d_Gfx) cudaFree(c->d_Gfx);
+      c->d_Gfx = nullptr;
+      return CEEDBP_OK;
+    }
+  }
+  CK(c, launch_fx_factors(m, kStiff, c->d_G, c->d_Gfx, c->d_gexp, c->stream));
+  m.Gfx = c->d_Gfx;
+  m.gexp = c->d_gexp;
+  return CEEDBP_OK;
 }
 
 ceedbp_status setup_impl(ceedbp_ctx* c, const double* coords, const int64_t* l2g, const uint8_t* dirichlet,
@@ -220,6 +229,8 @@ ceedbp_status setup_impl(ceedbp_ctx* c, const double* coords, const int64_t* l2g
   m.off = c->d_off;
   m.slots = c->d_slots;
   m.basis = c->d_basis;
+  build_fx_tables(basis, &c->fx);
+  m.fx = &c->fx;
 
   int nb_apply = elem_blocks(m);
   if (c->colloc) nb_apply = std::max(nb_apply, std::max(int(P.nelem), elem_lp_blocks(m)));
@@ -257,6 +268,10 @@ ceedbp_status setup_impl(ceedbp_ctx* c, const double* coords, const int64_t* l2g
     cudaFree(d_scratch);
     if (d_kappa) cudaFree(d_kappa);
     if (e != cudaSuccess) return cuda_fail(c, e, "geometric factors");
+  }
+  if (c->colloc && c->arith == CEEDBP_ARITH_FP64 && !recompute && !c->batch_group) {
+    const ceedbp_status st = prepare_fx(c);
+    if (st != CEEDBP_OK) return st;
   }
   // ---- Jacobi diagonal: local diag(A^e) (or diag(B^e)), summed by Q^T, inverted
   CK(c, launch_local_diag(m, c->op_kind, c->d_G, c->d_Mq, c->d_wl, s));
@@ -366,7 +381,7 @@ ceedbp_status setup_impl(ceedbp_ctx* c, const double* coords, const int64_t* l2g
     // autotuner: elements per block and G staging of the pair kernel, timed on this mesh
     int cand_eb[32], cand_st[32], cand_ns[32];
     int ncand = pair_shape_candidates(c, m, cand_eb, cand_st, cand_ns, 32);
-    if (c->pipelined_only) {  // keep the pipelined shapes when there are any
+    if (c->batch_group) {  // keep the pipelined shapes when there are any
       int np = 0;
       for (int k = 0; k < ncand; ++k)
         if (cand_st[k] == 2) {
@@ -900,6 +915,7 @@ ceedbp_status ceedbp_set_kappa(ceedbp_ctx* c, const double* kappa) {
   }
   CK(c, launch_scale_factors(c->d_Ghat, kappa, c->d_G, c->prm.nelem, int(q3), s));
   const DeviceMesh& m = c->mesh;
+  if (m.Gfx) CK(c, launch_fx_factors(m, kStiff, c->d_G, c->d_Gfx, c->d_gexp, s));
   CK(c, launch_local_diag(m, kStiff, c->d_G, c->d_Mq, c->d_wl, s));
   DeviceMesh m1 = m;
   m1.ncomp = 1;

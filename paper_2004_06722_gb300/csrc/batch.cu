@@ -441,7 +441,7 @@ ceedbp_status ceedbp_batch_setup(int nprob, const ceedbp_params* params, const d
     if (!g.ctx) return fail_out(bfail(nullptr, CEEDBP_ENOMEM, "host allocation failed"));
     g.ctx->prm = ceedbp_params{5, N, 0, E, ng, b->arith, CEEDBP_GEOM_STORED};
     g.ctx->stream = b->stream;
-    g.ctx->pipelined_only = true;  // pair arithmetic on large concatenated meshes: the pipelined schedule wins
+    g.ctx->batch_group = true;  // pair arithmetic on large concatenated meshes: the pipelined schedule wins
     ceedbp_status st = setup_context(g.ctx, cc.data(), ll.data(), dd.data(), nullptr);
     if (st != CEEDBP_OK) {
       const std::string msg = g.ctx->err;
@@ -452,7 +452,7 @@ ceedbp_status ceedbp_batch_setup(int nprob, const ceedbp_params* params, const d
     // kernel at this order (elements per block, times the sequence length of the pipelined schedule)
     int eb = 0;
     if (b->arith == CEEDBP_ARITH_FP64) {
-      eb = elem_stiff_per_block(g.ctx->mesh);
+      eb = elem_batch_per_block(g.ctx->mesh);
       if (eb < 1) {
         b->groups.push_back(g);
         return fail_out(bfail(nullptr, CEEDBP_EUNSUPPORTED, "no FP64 batched element kernel at this order"));

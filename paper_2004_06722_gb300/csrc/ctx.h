@@ -27,6 +27,9 @@ struct ceedbp_ctx {
   int* d_slots = nullptr;
   double* d_basis = nullptr;
   double* d_G = nullptr;
+  ceedbp::FxTables fx;               // host tables of the fixed-point kernels
+  int4* d_Gfx = nullptr;     // fixed-point factors and the exponent of each element (prepare_fx)
+  int* d_gexp = nullptr;
   double* d_X = nullptr;  // [E][3][p1^3] coordinates when the factors are recomputed
   int* d_l2g_id = nullptr;  // identity gather map of ceedbp_bk_apply (allocated on its first call)
   double* d_Mq = nullptr;
@@ -40,7 +43,7 @@ struct ceedbp_ctx {
   // Jacobi inverse; the CG pair vectors reuse d_r, d_p, d_ax and the local
   // scratch d_wl (a pair has the size of a double).
   int arith = 0;
-  bool pipelined_only = false;  // batched groups: tune among the pipelined pair-kernel shapes only
+  bool batch_group = false;  // of a batched solve: pipelined pair-kernel shapes only, no fixed-point factors
   double beta = 0.0;  // Helmholtz coefficient of Eq. (17) (ceedbp_set_helmholtz)
   ceedbp::dfloat* d_Gdf = nullptr;
   ceedbp::dfloat* d_Ddf = nullptr;

@@ -1,8 +1,7 @@
 // Element operator kernels (the column kernel): w^e = A^e u^e or B^e u^e for
-// every element, the unassembled product A_L Q u of Eq. (21).  It serves BK5/BK6
-// at even orders, BK2/BK4, and BK3 at order 14; BK1/BK3 otherwise run the
-// even-odd kernel of elem_gl.cuh, and BK5/BK6 at odd orders that of elem_eo.cuh.
-// The even-odd tables and products (EoTab, eo_build, eo_mul) defined here are
+// every element, the unassembled product A_L Q u of Eq. (21).  It serves BK2/BK4,
+// BK3 at order 14 and BK5 of batched solves at even orders; BK1/BK3 otherwise run the even-odd kernel of elem_gl.cuh, and
+// BK5/BK6 the fixed-point kernel of elem_fx.cuh.  The even-odd tables and products (EoTab, eo_build, eo_mul) defined here are
 // shared by those kernels.
 //
 // Stiffness, Eq. (22): w^e = sum_{m,m'} D_m^T G_mm' D_m' u^e with the
@@ -426,13 +425,8 @@ cudaError_t launch_elem_b(const DeviceMesh& m, const ElemArgs& a, cudaStream_t s
   return cudaGetLastError();
 }
 
-// Launch one instantiation (batched solves take the block-table variant: collocated stiffness,
-// one component).
 template <int P1, int Q, bool COLLOC, int KIND, int NC>
 cudaError_t launch_elem_t(const DeviceMesh& m, const ElemArgs& a, cudaStream_t s) {
-  if constexpr (COLLOC && KIND == kStiff && NC == 1) {
-    if (a.blk_prob != nullptr) return launch_elem_b<P1, Q, COLLOC, KIND, NC, true>(m, a, s);
-  }
   return launch_elem_b<P1, Q, COLLOC, KIND, NC, false>(m, a, s);
 }
 

@@ -1,6 +1,5 @@
 // FP32-pair BK5 element kernel with the even-odd decomposition of the 1D
-// contractions (the centro-antisymmetry of Eq. (37), as in the FP64 kernel of
-// elem_eo.cuh): every 1D pair product y = D x of a line becomes, for each
+// contractions (the centro-antisymmetry of Eq. (37)): every 1D pair product y = D x of a line becomes, for each
 // mirror pair of outputs (i, p1-1-i), two half-length sums
 //   S_E = sum_n E_in x+_n,  S_O = sum_n O_in x-_n,  y_i = S_E + S_O,  y_{p1-1-i} = S_O - S_E,
 // so a pair-arithmetic line costs p1^2/2 pair products instead of p1^2.
@@ -17,8 +16,7 @@
 // splitter of the direct kernel (dnorm_row max|x|) bounds both half sums.
 //
 // Thread mapping: one thread per mirror octet of nodes (i, j, k < p1/2), so
-// both outputs of every folded line product belong to the same thread (the
-// layout of elem_eo.cuh).  Schedule: each slot of p1^3/8 threads works through
+// both outputs of every folded line product belong to the same thread.  Schedule: each slot of p1^3/8 threads works through
 // a sequence of elements and fetches the next element's l2g and u by
 // asynchronous copies while it computes the current one (the dependent
 // l2g -> u gather is off the critical path); the next element's G is

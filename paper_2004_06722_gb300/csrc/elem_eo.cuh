@@ -1,5 +1,10 @@
-// FP64 BK5/BK6 element kernel with the even-odd decomposition of the 1D
+// FP64 BK5 element kernel of batched solves at odd orders, with the even-odd decomposition of the 1D
 // contractions (the symmetry of Eq. (37); Solomonoff 1992, Kopriva 2009).
+//
+// Batched solves keep this FP64 arithmetic although the fixed-point kernel of single solves
+// (elem_fx.cuh) is faster (32 problems of up to 12^3 elements: 50.8 against 88.1 ms): a batch stops each
+// problem at its residual tolerance after up to 400 iterations, where CG has lost orthogonality and
+// carries any other rounding of A p to 1e-9 of the solution at tolerance 1e-8.
 //
 // The GLL derivative matrix D and its transpose are centro-antisymmetric:
 // D[p1-1-i][p1-1-j] = -D[i][j].  With h = p1/2 (even p1), x+_j = x_j + x_{p1-1-j},
@@ -27,17 +32,17 @@ struct EoShape {
   static constexpr int TILE = 6 * HALF;     // r+, r-, s+, s-, t+, t- (doubles)
 };
 
-template <int P1, int NC>
+template <int P1>
 inline int elem_eo_per_block() {
   constexpr int H3 = EoShape<P1>::H3;
-  int eb = 128 / (H3 * NC);
+  const int eb = 128 / H3;
   return eb < 1 ? 1 : eb;
 }
 
-template <int P1, int NC>
+template <int P1>
 inline size_t elem_eo_smem_bytes(int eb) {
   using S = EoShape<P1>;
-  return sizeof(double) * (4 * S::H * S::H + 32 * NC + size_t(eb) * NC * S::TILE);
+  return sizeof(double) * (4 * S::H * S::H + 32 + size_t(eb) * S::TILE);
 }
 
 // node index of octet corner (bi, bj, bk) in {0,1}^3 of octet (i, j, k)
@@ -63,34 +68,27 @@ __device__ __forceinline__ void eo_pair(const double* E, const double* O, const 
   y1 = __fma_rn(-2.0, se, s);
 }
 
-// HELM: the Helmholtz term beta B u of Eq. (17) is compiled in only for beta != 0, so the plain
-// stiffness kernel carries no extra registers or branches.  BATCH: the block tables and per-problem
-// reductions of batched solves (one component), likewise compiled in only where used.
-template <int P1, int NC, bool HELM, bool BATCH = false>
-__global__ void elem_eo_kernel(const DeviceMesh m, const ElemArgs a, const int eb) {
+// Block tables (a.blk_*) give each block elements of one problem.
+template <int P1>
+__global__ void elem_eo_kernel(const DeviceMesh m, const ElemArgs a) {
+  constexpr int NC = 1;
   using S = EoShape<P1>;
   constexpr int H = S::H, H3 = S::H3, P3 = S::P3, HALF = S::HALF;
   extern __shared__ double smem_eo[];
-  if (a.state != nullptr && a.state->stop) return;
   double* sE = smem_eo;          // [H][H] even part of D (gradient)
   double* sO = sE + H * H;       // [H][H] odd part of D
   double* sEt = sO + H * H;      // [H][H] even part of D^T (transpose)
   double* sOt = sEt + H * H;     // [H][H] odd part of D^T
-  double* red = sOt + H * H;     // 32 * NC
-  double* tiles = red + 32 * NC;
+  double* red = sOt + H * H;     // 32
+  double* tiles = red + 32;
 
   const int tid = threadIdx.x;
   const int slot = tid / H3, o = tid - slot * H3;
   const int i = o % H, j = (o / H) % H, k = o / (H * H);
-  int64_t e0 = int64_t(blockIdx.x) * eb;
-  int nact = m.nelem - e0 < eb ? int(m.nelem - e0) : eb;
-  int prob = 0;
-  if constexpr (BATCH) {  // batched: this block holds elements of one problem
-    prob = a.blk_prob[blockIdx.x];
-    if (!a.bst[prob].c.active) return;
-    e0 = a.blk_e0[blockIdx.x];
-    nact = a.blk_n[blockIdx.x];
-  }
+  const int prob = a.blk_prob[blockIdx.x];
+  if (!a.bst[prob].c.active) return;
+  const int64_t e0 = a.blk_e0[blockIdx.x];
+  const int nact = a.blk_n[blockIdx.x];
   const int64_t e = e0 + slot;
   const bool active = slot < nact;
 
@@ -289,91 +287,26 @@ __global__ void elem_eo_kernel(const DeviceMesh m, const ElemArgs a, const int e
 #pragma unroll
       for (int c8 = 0; c8 < 8; ++c8) {
         const int node = eo_node<P1>(i, j, k, c8 & 1, (c8 >> 1) & 1, c8 >> 2);
-        if constexpr (HELM) w[c8] += a.beta * __ldg(a.Mq + e * P3 + node) * u[c][c8];  // Eq. (17)
         if (!(a.skip_dirichlet_out && ((dmask >> c8) & 1))) wl[size_t(node) * NC + c] = w[c8];
         dot[c] += w[c8] * u[c][c8];
       }
     }
   }
 
-  if constexpr (BATCH && NC == 1) {  // per-problem alpha from a segmented last-block reduction
-    batch_alpha(dot, a.partials, a.prob_blk0, a.prob_nblk, a.bst, prob, red);
-    return;
-  }
-  if (a.partials != nullptr) {
-    if (grid_sum_last<NC>(dot, a.partials, gridDim.x, blockIdx.x, &a.state->ticket[kTicketApply], red)) {
-      if (threadIdx.x == 0) {
-        SolveState* st = a.state;
-        int any = 0;
-#pragma unroll
-        for (int c = 0; c < NC; ++c) {
-          CompScalars& cs = st->c[c];
-          if (!cs.active) continue;
-          const double pAp = dot[c];
-          cs.pAp = pAp;
-          if (!(pAp > 0.0) || !isfinite(pAp) || !isfinite(cs.rz)) {
-            cs.status = CEEDBP_EBREAKDOWN;
-            cs.alpha = 0.0;
-            if (!st->fixed) cs.active = 0;
-          } else {
-            cs.alpha = cs.rz / pAp;
-          }
-          any |= cs.active;
-        }
-        if (!any) st->stop = 1;
-      }
-    }
-  }
+  // per-problem alpha from a segmented last-block reduction
+  batch_alpha(dot, a.partials, a.prob_blk0, a.prob_nblk, a.bst, prob, red);
 }
 
-template <int P1, int NC, bool HELM, bool BATCH = false>
-cudaError_t launch_elem_eo_h(const DeviceMesh& m, const ElemArgs& a, cudaStream_t s) {
-  const int eb = elem_eo_per_block<P1, NC>();
+template <int P1>
+cudaError_t launch_elem_eo_t(const DeviceMesh& m, const ElemArgs& a, cudaStream_t s) {
+  const int eb = elem_eo_per_block<P1>();
   const int nthreads = ((eb * EoShape<P1>::H3 + 31) / 32) * 32;
-  const size_t smem = elem_eo_smem_bytes<P1, NC>(eb);
-  auto kern = elem_eo_kernel<P1, NC, HELM, BATCH>;
+  const size_t smem = elem_eo_smem_bytes<P1>(eb);
+  auto kern = elem_eo_kernel<P1>;
   static const cudaError_t attr = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
   if (attr != cudaSuccess) return attr;
-  const int64_t blocks = BATCH ? int64_t(a.batch_blocks) : (m.nelem + eb - 1) / eb;
-  kern<<<unsigned(blocks), nthreads, smem, s>>>(m, a, eb);
+  kern<<<unsigned(a.batch_blocks), nthreads, smem, s>>>(m, a);
   return cudaGetLastError();
-}
-
-template <int P1, int NC>
-cudaError_t launch_elem_eo_t(const DeviceMesh& m, const ElemArgs& a, cudaStream_t s) {
-  if constexpr (NC == 1) {
-    if (a.blk_prob != nullptr) return launch_elem_eo_h<P1, 1, false, true>(m, a, s);
-  }
-  return a.beta != 0.0 ? launch_elem_eo_h<P1, NC, true>(m, a, s) : launch_elem_eo_h<P1, NC, false>(m, a, s);
-}
-
-// whether the kernel can be resident (its registers and threads fit an SM)
-template <int P1, int NC>
-inline bool elem_eo_launchable() {
-  static const bool ok = [] {
-    const int eb = elem_eo_per_block<P1, NC>();
-    const int nthreads = ((eb * EoShape<P1>::H3 + 31) / 32) * 32;
-    const size_t smem = elem_eo_smem_bytes<P1, NC>(eb);
-    int nb0 = 0, nb1 = 0;
-    if (cudaFuncSetAttribute(elem_eo_kernel<P1, NC, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             int(smem)) != cudaSuccess ||
-        cudaFuncSetAttribute(elem_eo_kernel<P1, NC, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             int(smem)) != cudaSuccess)
-      return false;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb0, elem_eo_kernel<P1, NC, false>, nthreads, smem) !=
-            cudaSuccess ||
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb1, elem_eo_kernel<P1, NC, true>, nthreads, smem) !=
-            cudaSuccess)
-      return false;
-    return nb0 >= 1 && nb1 >= 1;
-  }();
-  return ok;
-}
-
-template <int P1, int NC>
-inline int elem_eo_blocks_t(int64_t nelem) {
-  const int eb = elem_eo_per_block<P1, NC>();
-  return int((nelem + eb - 1) / eb);
 }
 
 }  // namespace ceedbp

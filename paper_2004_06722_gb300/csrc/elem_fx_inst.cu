@@ -1,0 +1,36 @@
+// Dispatch of the fixed-point BK5/BK6 kernel (elem_fx.cuh) by order; instantiated in elem_fx_[a-e].cu.
+#include "elem_fx.cuh"
+
+namespace ceedbp {
+
+#define CEEDBP_FX_P1(X) \
+  X(2) X(3) X(4) X(5) X(6) X(7) X(8) X(9) X(10) X(11) X(12) X(13) X(14) X(15) X(16)
+
+#define X(P)                                                                                    \
+  extern template cudaError_t launch_elem_fx_t<P>(const DeviceMesh&, const ElemArgs&, cudaStream_t); \
+  extern template int elem_fx_blocks_t<P, 1>(int64_t);                                          \
+  extern template int elem_fx_blocks_t<P, 3>(int64_t);
+CEEDBP_FX_P1(X)
+#undef X
+
+cudaError_t launch_elem_fx(const DeviceMesh& m, const ElemArgs& a, cudaStream_t s) {
+  switch (m.p1) {
+#define X(P) \
+  case P: return launch_elem_fx_t<P>(m, a, s);
+    CEEDBP_FX_P1(X)
+#undef X
+    default: return cudaErrorInvalidValue;
+  }
+}
+
+int elem_fx_blocks(const DeviceMesh& m) {
+  switch (m.p1) {
+#define X(P) \
+  case P: return m.ncomp == 3 ? elem_fx_blocks_t<P, 3>(m.nelem) : elem_fx_blocks_t<P, 1>(m.nelem);
+    CEEDBP_FX_P1(X)
+#undef X
+    default: return 0;
+  }
+}
+
+}  // namespace ceedbp

@@ -1,0 +1,199 @@
+// Block fixed-point arithmetic of the FP64 element kernels.
+//
+// GB300 issues 2 FP64 FMAs per clock per SM but 64 widening integer
+// multiply-adds (32 x 32 + 64 -> 64 bits; measured 64.4 per clock per SM), so an
+// FP64 contraction is cheaper in integers: every value of an element is an
+// integer on one power-of-two grid, 60 bits below the element's largest value,
+// and a 1D product costs three widening multiply-adds per term instead of one
+// FP64 FMA at 1/32 of their rate.
+//
+// Values.  x = h 2^31 + l with -2^30 <= l < 2^30 (two 32-bit limbs, "limbs" below) and |x| < 2^60.
+// Matrix entries are M = h 2^31 + l likewise, scaled so that the largest absolute row sum is 2^62.
+// A line product is
+//   y = sum_j M_j x_j / 2^62 = HH + MM / 2^31,  HH = sum h_M h_x,  MM = sum (h_M l_x + l_M h_x)
+// (the l l terms stay below one unit), so |y| < 2^60 again and the next stage starts without
+// renormalisation.  MM / 2^31 is applied as twice MM's rounded upper word (one more multiply-add).
+// The sums are integer sums: exact, and independent of their order; a sum of zeros is zero.
+//
+// Accuracy.  One unit is 2^-60 of an a-priori bound of a stage's values, against FP64's 2^-53 of each
+// partial sum.  The bound of a derivative (the largest row sum of |D|) can exceed the actual values by
+// 2^8; the gradient keeps enough bits for that, but the fluxes G grad u are moved up to 2^60 again by
+// the element's actual maximum before the transposes, so that the two derivatives' slack does not add
+// up (fx_limbs_up).  With that the error of one application, against quad-precision references, stays
+// at or below that of the FP64 kernels this arithmetic replaces.  Values a grid cannot hold
+// (infinities, NaN, elements whose factors spread over more than 2^7, exponents near the ends of the
+// FP64 range) take the FP64 form of the same kernel (the double overloads below).
+#pragma once
+
+#include "common.cuh"
+#include "df.cuh"
+
+namespace ceedbp {
+
+// Even-odd form of a centro-(anti)symmetric NO x NI matrix (Eq. (37)): e, o hold
+// (M_ij + M_ij')/2 and (M_ij - M_ij')/2 for the first NO/2 rows (j' = NI-1-j; the middle column of
+// an odd NI is held whole in e), m the middle row of an odd NO (over x+ or, antisymmetric, x-).
+template <int NI, int NO, typename T>
+struct EoMat {
+  static constexpr int H = NI / 2, HC = (NI + 1) / 2, R = NO / 2;
+  T e[R][HC];
+  T o[R][H];
+  T m[NO % 2 ? HC : 1];
+};
+
+constexpr long long kFxHalf = 1ll << 30;   // half a unit of h: limbs are taken from y + kFxHalf
+constexpr long long kFxRound = 1ll << 31;  // MM starts here: its upper word is rounded to nearest, zeros stay zero
+
+__device__ __forceinline__ long long fx_mad(int a, int b, long long c) { return (long long)a * b + c; }
+
+// limbs of y, given y + kFxHalf
+__device__ __forceinline__ int2 fx_limbs(long long yb) {
+  return make_int2(int(yb >> 31), (int(yb) & 0x7fffffff) - int(kFxHalf));
+}
+
+// limbs of y 2^s, 0 <= s <= 30, |y 2^s| < 2^60, given y + (kFxHalf >> s)
+__device__ __forceinline__ int2 fx_limbs_up(long long yb, int s) {
+  return make_int2(int(__funnelshift_r(unsigned(yb), unsigned(yb >> 32), 31 - s)),
+                   (int(unsigned(yb) << s) & 0x7fffffff) - int(kFxHalf));
+}
+
+// HH + MM / 2^31, MM started from kFxRound
+__device__ __forceinline__ long long fx_join(long long hh, long long mm) { return fx_mad(int(mm >> 32), 2, hh); }
+
+// limbs of v 2^(1082 - eb), below 2^60 in an element whose largest magnitude has the biased exponent eb
+__device__ __forceinline__ int2 fx_from_double(double v, int eb) {
+  const int hi = __double2hiint(v), lo = __double2loint(v);
+  const int ev = (hi >> 20) & 0x7ff;
+  const int d = min(eb - ev, 63);  // zeros and subnormals (ev = 0) shift out: eb is at least 500 here
+  const unsigned long long mant =
+      ((unsigned long long)(unsigned((hi & 0xfffff) | 0x100000)) << 32 | unsigned(lo)) << 7;
+  const long long f = (long long)(mant >> d);
+  return fx_limbs((hi < 0 ? -f : f) + kFxHalf);
+}
+
+// y = M x for one line, even-odd; emit(i, y_i), in limbs' arithmetic y_i + BIAS (int2 overload).
+template <long long BIAS, int NI, int NO, bool ANTI, class Emit>
+__device__ __forceinline__ void eo_line(const EoMat<NI, NO, int2>& M, const int2 (&x)[NI], Emit&& emit) {
+  constexpr int H = NI / 2, HC = (NI + 1) / 2, R = NO / 2;
+  int2 p[HC], q[H];
+#pragma unroll
+  for (int j = 0; j < H; ++j) {
+    p[j] = make_int2(x[j].x + x[NI - 1 - j].x, x[j].y + x[NI - 1 - j].y);
+    q[j] = make_int2(x[j].x - x[NI - 1 - j].x, x[j].y - x[NI - 1 - j].y);
+  }
+  if constexpr (HC > H) p[H] = x[H];
+#pragma unroll
+  for (int i = 0; i < R; ++i) {
+    long long he = BIAS, me = kFxRound, ho = 0, mo = kFxRound;
+#pragma unroll
+    for (int j = 0; j < HC; ++j) {
+      he = fx_mad(M.e[i][j].x, p[j].x, he);
+      me = fx_mad(M.e[i][j].x, p[j].y, me);
+      me = fx_mad(M.e[i][j].y, p[j].x, me);
+    }
+#pragma unroll
+    for (int j = 0; j < H; ++j) {
+      ho = fx_mad(M.o[i][j].x, q[j].x, ho);
+      mo = fx_mad(M.o[i][j].x, q[j].y, mo);
+      mo = fx_mad(M.o[i][j].y, q[j].x, mo);
+    }
+    const long long se = fx_join(he, me), so = fx_join(ho, mo);
+    emit(i, se + so);
+    emit(NO - 1 - i, ANTI ? so - se + 2 * BIAS : se - so);
+  }
+  if constexpr (NO % 2) {
+    long long hh = BIAS, mm = kFxRound;
+#pragma unroll
+    for (int j = 0; j < (ANTI ? H : HC); ++j) {
+      const int2 v = ANTI ? q[j < H ? j : 0] : p[j];
+      hh = fx_mad(M.m[j].x, v.x, hh);
+      mm = fx_mad(M.m[j].x, v.y, mm);
+      mm = fx_mad(M.m[j].y, v.x, mm);
+    }
+    emit(R, fx_join(hh, mm));
+  }
+}
+
+template <long long BIAS, int NI, int NO, bool ANTI, class Emit>
+__device__ __forceinline__ void eo_line(const EoMat<NI, NO, double>& M, const double (&x)[NI], Emit&& emit) {
+  constexpr int H = NI / 2, HC = (NI + 1) / 2, R = NO / 2;
+  double p[HC], q[H];
+#pragma unroll
+  for (int j = 0; j < H; ++j) {
+    p[j] = x[j] + x[NI - 1 - j];
+    q[j] = x[j] - x[NI - 1 - j];
+  }
+  if constexpr (HC > H) p[H] = x[H];
+#pragma unroll
+  for (int i = 0; i < R; ++i) {
+    // the odd half-sum on top of the even one: y_i comes out of the chain, its mirror is one more fma
+    double se = __dmul_rn(M.e[i][0], p[0]);
+#pragma unroll
+    for (int j = 1; j < HC; ++j) se = __fma_rn(M.e[i][j], p[j], se);
+    double s = se;
+#pragma unroll
+    for (int j = 0; j < H; ++j) s = __fma_rn(M.o[i][j], q[j], s);
+    emit(i, s);
+    emit(NO - 1 - i, ANTI ? __fma_rn(-2.0, se, s) : __fma_rn(2.0, se, -s));
+  }
+  if constexpr (NO % 2) {
+    double s = 0.0;
+#pragma unroll
+    for (int j = 0; j < (ANTI ? H : HC); ++j) s = __fma_rn(M.m[j], ANTI ? q[j < H ? j : 0] : p[j], s);
+    emit(R, s);
+  }
+}
+
+// One row of the geometric factors times the gradient at a point.
+__device__ __forceinline__ long long fx_dot3(int2 a, int2 x, int2 b, int2 y, int2 c, int2 z) {
+  long long hh = fx_mad(a.x, x.x, 0), mm = fx_mad(a.x, x.y, kFxRound);
+  mm = fx_mad(a.y, x.x, mm);
+  hh = fx_mad(b.x, y.x, hh);
+  mm = fx_mad(b.x, y.y, mm);
+  mm = fx_mad(b.y, y.x, mm);
+  hh = fx_mad(c.x, z.x, hh);
+  mm = fx_mad(c.x, z.y, mm);
+  mm = fx_mad(c.y, z.x, mm);
+  return fx_join(hh, mm);
+}
+
+// Largest magnitude of a set of values by their upper words, and the shift that moves it up to 2^60.
+struct FxRange {
+  int hi = 0, lo = 0;
+  __device__ __forceinline__ void add(long long y) {
+    const int w = int(y >> 32);
+    hi = max(hi, w);
+    lo = min(lo, w);
+  }
+  __device__ __forceinline__ unsigned top() const { return unsigned(max(hi, ~lo)); }
+};
+__device__ __forceinline__ int fx_shift(unsigned top) { return min(max(__clz(int(top)) - 4, 0), 30); }
+
+// The two arithmetics of the element kernels: L a stage's input, Raw its output.
+struct FxArith {
+  using L = int2;
+  using Raw = long long;
+  static constexpr long long kBias = kFxHalf;
+  FxRange range;
+  int shift = 0;
+  long long bias = 0;  // kFxHalf on the unshifted grid
+  __device__ __forceinline__ static L limbs(long long yb) { return fx_limbs(yb); }  // of a biased output
+  __device__ __forceinline__ L load(Raw y) const { return fx_limbs_up(y + bias, shift); }
+  __device__ __forceinline__ void see(Raw y) { range.add(y); }
+  __device__ __forceinline__ void set_shift(unsigned top) {
+    shift = fx_shift(top);
+    bias = kFxHalf >> shift;
+  }
+};
+struct F64Arith {
+  using L = double;
+  using Raw = double;
+  static constexpr long long kBias = 0;
+  __device__ __forceinline__ static L limbs(double y) { return y; }
+  __device__ __forceinline__ L load(Raw y) const { return y; }
+  __device__ __forceinline__ void see(Raw) {}
+};
+
+__device__ __forceinline__ void l2_prefetch(const void* p) { asm volatile("prefetch.global.L2 [%0];" ::"l"(p)); }
+
+}  // namespace ceedbp

@@ -32,6 +32,24 @@ struct Basis1D {
 // Device table layout (doubles): J [q*p1] | Dh [q*p1] | Dq [q*q] | w [q]
 inline size_t basis_doubles(int p1, int q) { return size_t(2) * q * p1 + size_t(q) * q + q; }
 
+// Even-odd tables of the block fixed-point kernels (fx.cuh), flattened in the order of EoMat: limb
+// pairs, and the FP64 forms. A scale is the true value of a stage's result over its fixed-point value;
+// chain and mchain are the products over all tables of a stiffness and a mass operator.
+struct FxTables {
+  std::vector<int> D, DT, J, JT;
+  std::vector<double> D64, DT64, J64, JT64;
+  std::vector<double> w;  // GLL weights
+  long double chain = 1.0L, mchain = 1.0L;
+};
+
+// Exponent of an element whose factors do not fit the fixed-point grid.
+constexpr int kFxNoGrid = -(1 << 30);
+struct Basis1D;
+void build_fx_tables(const Basis1D& b, FxTables* t);
+
+// Longest element sequence of a slot of the fixed-point kernels.
+constexpr int kFxMaxSeq = 16;
+
 bool build_basis(int order, int q, bool gll_quad, Basis1D* out, std::string* err);
 
 // Per-component CG scalars kept on the device.
@@ -81,6 +99,11 @@ struct DeviceMesh {
   int tune_stage;       // pair kernel schedule (autotuner): 0 G ring by cp.async, 1 G staged by a bulk
                         // copy, 2 software-pipelined element sequences (elem_dfp_kernel)
   int tune_ns;          // elements per slot sequence of the pipelined schedule
+  const FxTables* fx;   // host: tables of the fixed-point kernels
+  const int4* Gfx;      // fixed-point stiffness factors [E][q][3][q^2], or nullptr (FP64 form)
+  const int* gexp;      // [E] exponent of the element's fixed-point result (kFxNoGrid: it runs in FP64)
+  const int2* Mfx;      // fixed-point mass factors [E][q^3] of Gauss quadrature, or nullptr
+  const int* mexp;      // [E] as gexp
   const double* X;      // [E][3][p1^3] nodal coordinates when the factors are recomputed, else nullptr
 };
 
@@ -124,8 +147,8 @@ struct ElemArgs {
   int batch_blocks;      // grid size of a batched launch
 };
 int elem_blocks(const DeviceMesh& m);
-// Elements per block of the FP64 stiffness kernel launch_elem uses (block tables of batched solves).
-int elem_stiff_per_block(const DeviceMesh& m);
+// Elements per block of the FP64 kernel of batched BP5 solves (block tables).
+int elem_batch_per_block(const DeviceMesh& m);
 cudaError_t launch_elem(const DeviceMesh& m, int kind, const ElemArgs& a, cudaStream_t s);
 // Stiffness element kernel recomputing G from m.X (collocated, FP64).
 cudaError_t launch_elem_rc(const DeviceMesh& m, const ElemArgs& a, cudaStream_t s);
@@ -133,6 +156,12 @@ int elem_rc_blocks(const DeviceMesh& m);
 bool elem_rc_supported(int p1, int ncomp);
 // coords [E][p1^3][3] -> X [E][3][p1^3]
 cudaError_t launch_coords_soa(const double* coords, double* X, int64_t nelem, int p3, cudaStream_t s);
+
+// Fixed-point copy of the stiffness (kStiff) or mass (kMass) factors, without quadrature weights, and
+// the exponent of each element's result.
+cudaError_t launch_fx_factors(const DeviceMesh& m, int kind, const double* G, void* out, int* gexp, cudaStream_t s);
+cudaError_t launch_elem_fx(const DeviceMesh& m, const ElemArgs& a, cudaStream_t s);
+int elem_fx_blocks(const DeviceMesh& m);
 
 // Gather-scatter sum w[g] = sum_slots wl (masked on Dirichlet nodes if mask_out).
 cudaError_t launch_gs(const DeviceMesh& m, const double* wl, double* w, int mask_out, cudaStream_t s);
