@@ -12,36 +12,24 @@
 #include "internal.h"
 
 namespace ceedbp {
-cudaError_t launch_elem_bp1(const DeviceMesh& m, const ElemArgs& a, cudaStream_t s);
-cudaError_t launch_elem_bp3(const DeviceMesh& m, const ElemArgs& a, cudaStream_t s);
-int elem_blocks_bp1(const DeviceMesh& m);
-cudaError_t launch_elem_bp2(const DeviceMesh& m, const ElemArgs& a, cudaStream_t s);
-cudaError_t launch_elem_bp4(const DeviceMesh& m, const ElemArgs& a, cudaStream_t s);
-int elem_blocks_bp4(const DeviceMesh& m);
-int elem_blocks_bp3(const DeviceMesh& m);
-
 // batched BP5 solves: even-odd kernel at odd orders, column kernel at even ones
 cudaError_t launch_elem_eo(const DeviceMesh& m, const ElemArgs& a, cudaStream_t s);
-cudaError_t launch_elem_bp5(const DeviceMesh& m, const ElemArgs& a, cudaStream_t s);
+cudaError_t launch_elem_col(const DeviceMesh& m, const ElemArgs& a, cudaStream_t s);
 int elem_eo_per_block_rt(const DeviceMesh& m);
-int elem_per_block_bp5(const DeviceMesh& m);
+int elem_col_per_block_rt(const DeviceMesh& m);
 
 cudaError_t launch_elem(const DeviceMesh& m, int kind, const ElemArgs& a, cudaStream_t s) {
   if (kind == kStiff && m.X != nullptr) return launch_elem_rc(m, a, s);
-  if (a.blk_prob != nullptr) return m.p1 % 2 == 0 ? launch_elem_eo(m, a, s) : launch_elem_bp5(m, a, s);
+  if (a.blk_prob != nullptr) return m.p1 % 2 == 0 ? launch_elem_eo(m, a, s) : launch_elem_col(m, a, s);
   if (m.colloc && kind == kStiff) return launch_elem_fx(m, a, s);
-  if (!m.colloc && kind == kStiff) return m.ncomp == 3 ? launch_elem_bp4(m, a, s) : launch_elem_bp3(m, a, s);
-  if (!m.colloc && kind == kMass) return m.ncomp == 3 ? launch_elem_bp2(m, a, s) : launch_elem_bp1(m, a, s);
-  return cudaErrorInvalidValue;
+  return m.colloc ? cudaErrorInvalidValue : launch_elem_fxgl(m, kind, a, s);
 }
 
-int elem_batch_per_block(const DeviceMesh& m) { return m.p1 % 2 == 0 ? elem_eo_per_block_rt(m) : elem_per_block_bp5(m); }
+int elem_batch_per_block(const DeviceMesh& m) { return m.p1 % 2 == 0 ? elem_eo_per_block_rt(m) : elem_col_per_block_rt(m); }
 
 int elem_blocks(const DeviceMesh& m) {
-  // stiffness and mass instantiations of one (p1, q) share the block shape
   if (m.X != nullptr) return elem_rc_blocks(m);
-  if (m.colloc) return elem_fx_blocks(m);
-  return m.ncomp == 3 ? elem_blocks_bp4(m) : elem_blocks_bp3(m);
+  return m.colloc ? elem_fx_blocks(m) : elem_fxgl_blocks(m);
 }
 }  // namespace ceedbp
 
@@ -94,7 +82,8 @@ void release(ceedbp_ctx* c) {
   void* ptrs[] = {c->d_l2g, c->d_off, c->d_slots, c->d_basis, c->d_G, c->d_Mq, c->d_dinv, c->d_mdiag,
                   c->d_wl, c->d_r, c->d_p, c->d_ax, c->d_part_apply, c->d_part_vec, c->d_state,
                   c->d_Gdf, c->d_Ddf, c->d_dinvdf, c->d_G32, c->d_Gbf, c->d_dinv32, c->d_xin,
-                  c->d_rin, c->d_pin, c->d_outer, c->d_Ghat, c->d_scal, c->d_X, c->d_l2g_id, c->d_Gfx, c->d_gexp};
+                  c->d_rin, c->d_pin, c->d_outer, c->d_Ghat, c->d_scal, c->d_X, c->d_l2g_id, c->d_Gfx, c->d_gexp, c->d_Mfx,
+                  c->d_mexp};
   for (void* p : ptrs)
     if (p) cudaFree(p);
   if (c->h_outer) cudaFreeHost(c->h_outer);
@@ -106,26 +95,35 @@ void release(ceedbp_ctx* c) {
   c->prof.clear();
 }
 
-// Fixed-point copy of the stiffness factors for the FP64 element kernel (elem_fx.cuh): as large as
-// the factors themselves, so it is kept only while it takes at most a quarter of the free memory;
-// without it the kernel runs in FP64.
+// Fixed-point copies of the stiffness factors and, with Gauss quadrature, the mass factors for the FP64
+// element kernels (elem_fx.cuh, elem_fxgl.cuh): as large as the factors themselves, so they are kept
+// only while they take at most a quarter of the free memory; without them the kernels run in FP64.
 ceedbp_status prepare_fx(ceedbp_ctx* c) {
   DeviceMesh& m = c->mesh;
-  const size_t q3 = size_t(c->q) * c->q * c->q, bytes = sizeof(int4) * 3 * size_t(m.nelem) * q3;
-  if (!c->d_Gfx) {
-    size_t free_b = 0, total_b = 0;
-    CK(c, cudaMemGetInfo(&free_b, &total_b));
-    if (bytes > free_b / 4) return CEEDBP_OK;
-    if (dalloc(&c->d_Gfx, bytes / sizeof(int4)) != cudaSuccess || dalloc(&c->d_gexp, size_t(m.nelem)) != cudaSuccess) {
-      cudaGetLastError();
-      if (c->d_Gfx) cudaFree(c->d_Gfx);
-      c->d_Gfx = nullptr;
-      return CEEDBP_OK;
-    }
+  const size_t nq = size_t(m.nelem) * c->q * c->q * c->q;
+  const bool stiff = c->op_kind == kStiff, mass = !c->colloc;
+  size_t free_b = 0, total_b = 0;
+  CK(c, cudaMemGetInfo(&free_b, &total_b));
+  if (nq * (stiff * 3 * sizeof(int4) + mass * sizeof(int2)) > free_b / 4) return CEEDBP_OK;
+  cudaError_t e = cudaSuccess;
+  if (stiff) e = dalloc(&c->d_Gfx, 3 * nq);
+  if (stiff && e == cudaSuccess) e = dalloc(&c->d_gexp, size_t(m.nelem));
+  if (mass && e == cudaSuccess) e = dalloc(&c->d_Mfx, nq);
+  if (mass && e == cudaSuccess) e = dalloc(&c->d_mexp, size_t(m.nelem));
+  if (e != cudaSuccess) {
+    cudaGetLastError();  // out of memory: run in FP64
+    return CEEDBP_OK;
   }
-  CK(c, launch_fx_factors(m, kStiff, c->d_G, c->d_Gfx, c->d_gexp, c->stream));
-  m.Gfx = c->d_Gfx;
-  m.gexp = c->d_gexp;
+  if (stiff) {
+    CK(c, launch_fx_factors(m, kStiff, c->d_G, c->d_Gfx, c->d_gexp, c->stream));
+    m.Gfx = c->d_Gfx;
+    m.gexp = c->d_gexp;
+  }
+  if (mass) {
+    CK(c, launch_fx_factors(m, kMass, c->d_Mq, c->d_Mfx, c->d_mexp, c->stream));
+    m.Mfx = c->d_Mfx;
+    m.mexp = c->d_mexp;
+  }
   return CEEDBP_OK;
 }
 
@@ -269,7 +267,7 @@ ceedbp_status setup_impl(ceedbp_ctx* c, const double* coords, const int64_t* l2g
     if (d_kappa) cudaFree(d_kappa);
     if (e != cudaSuccess) return cuda_fail(c, e, "geometric factors");
   }
-  if (c->colloc && c->arith == CEEDBP_ARITH_FP64 && !recompute && !c->batch_group) {
+  if (c->arith == CEEDBP_ARITH_FP64 && !recompute && !c->batch_group) {
     const ceedbp_status st = prepare_fx(c);
     if (st != CEEDBP_OK) return st;
   }

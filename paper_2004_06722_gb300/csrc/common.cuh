@@ -94,4 +94,29 @@ __device__ __forceinline__ void batch_alpha(double (&dot)[1], double* partials, 
   }
 }
 
+// (p, A p) of the NC components over the grid; the last block writes each component's alpha and
+// deactivates components that broke down.
+template <int NC>
+__device__ __forceinline__ void cg_alpha(double (&dot)[NC], double* partials, SolveState* st, double* red) {
+  if (!grid_sum_last<NC>(dot, partials, gridDim.x, blockIdx.x, &st->ticket[kTicketApply], red)) return;
+  if (threadIdx.x != 0) return;
+  int any = 0;
+#pragma unroll
+  for (int c = 0; c < NC; ++c) {
+    CompScalars& cs = st->c[c];
+    if (!cs.active) continue;
+    const double pAp = dot[c];
+    cs.pAp = pAp;
+    if (!(pAp > 0.0) || !isfinite(pAp) || !isfinite(cs.rz)) {
+      cs.status = CEEDBP_EBREAKDOWN;
+      cs.alpha = 0.0;
+      if (!st->fixed) cs.active = 0;
+    } else {
+      cs.alpha = cs.rz / pAp;
+    }
+    any |= cs.active;
+  }
+  if (!any) st->stop = 1;
+}
+
 }  // namespace ceedbp

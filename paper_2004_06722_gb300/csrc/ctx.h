@@ -30,6 +30,8 @@ struct ceedbp_ctx {
   ceedbp::FxTables fx;               // host tables of the fixed-point kernels
   int4* d_Gfx = nullptr;     // fixed-point factors and the exponent of each element (prepare_fx)
   int* d_gexp = nullptr;
+  int2* d_Mfx = nullptr;     // likewise the mass factors of Gauss quadrature
+  int* d_mexp = nullptr;
   double* d_X = nullptr;  // [E][3][p1^3] coordinates when the factors are recomputed
   int* d_l2g_id = nullptr;  // identity gather map of ceedbp_bk_apply (allocated on its first call)
   double* d_Mq = nullptr;

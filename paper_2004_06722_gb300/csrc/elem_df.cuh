@@ -1,6 +1,6 @@
 // FP64-accurate BK5/BK6 element kernel on the FP32 pipe (pairs of floats).
 //
-// Same operator as elem_kernel with GLL collocation (Eq. (22) with J = I):
+// The BK5/BK6 operator (Eq. (22) with J = I):
 //   u_r = D_1 u, u_s = D_2 u, u_t = D_3 u           (3 x p1 pair products per node)
 //   (w_r, w_s, w_t) = G (u_r, u_s, u_t)              (Eq. (23) factors, stored as pairs)
 //   w = D_1^T w_r + D_2^T w_s + D_3^T w_t            (3 x p1 pair products per node)

@@ -2,7 +2,7 @@
 // FP64-accurate arithmetic of df.cuh for the bake-off problems with
 // interpolation stages (Table 1: BP1 mass, BP3 Poisson; one component).
 //
-// Stages as in the FP64 kernel of elem_gl.cuh, one thread per line:
+// Stages, one thread per line:
 // interpolation J (q x p1) along x, y, z; for BK3 the GL derivative Dq along
 // the r and s lines and the t column, the factors G of Eq. (23) per point, the
 // transposes Dq^T, and for BK1 the mass factors of Eq. (34); then J^T back

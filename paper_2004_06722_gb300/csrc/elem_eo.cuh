@@ -18,7 +18,7 @@
 // x {k, p1-1-k} (i, j, k < h), so both outputs of every 1D pair product in all
 // three directions belong to the same thread.  The decomposed input lines are
 // exchanged through shared memory; G, the transpose and the output stay per
-// thread.  Same operator, layout and fused (u, w) dot as elem_kernel.
+// thread.  Fused (u, w) dot, deterministic.
 #pragma once
 
 #include "common.cuh"

@@ -75,11 +75,11 @@ struct FxCoElem {
 };
 
 // Contractions and factors of one element in arithmetic Ar (FxArith or F64Arith), u in tile A.
-// factors(k, gradient, flux) multiplies by G at point k of the own column; seen(ar) runs before and
-// scaled(ar) after the barrier that follows the factors; out(k, r, s, t) receives the three transposes.
-template <int P1, class Ar, class Tab, class Factors, class Mid, class Seen, class Scaled, class Out>
+// factors(k, gradient, flux) multiplies by G at point k of the own column; done(shift) comes with the
+// number of bits the fluxes were moved up; out(k, r, s, t) receives the three transposes.
+template <int P1, class Ar, class Tab, class Factors, class Mid, class Done, class Out>
 __device__ __forceinline__ void fx_co_stages(const FxCoElem<P1>& el, const Tab& D, const Tab& DT, bool live,
-                                             Factors&& factors, Mid&& mid, Seen&& seen, Scaled&& scaled, Out&& out) {
+                                             const FxNorm& norm, Factors&& factors, Mid&& mid, Done&& done, Out&& out) {
   using Sh = FxCoShape<P1>;
   using L = typename Ar::L;
   using Raw = typename Ar::Raw;
@@ -115,9 +115,10 @@ __device__ __forceinline__ void fx_co_stages(const FxCoElem<P1>& el, const Tab& 
       Ar_[own + k * PS] = ft;
     }
   }
-  seen(ar);
+  ar.publish(norm, 1);
   __syncthreads();
-  scaled(ar);
+  ar.take(norm, 1);
+  done(ar.total);
   if (live) {
 #pragma unroll Sh::UNROLL
     for (int dir = 0; dir < 3; ++dir) {
@@ -144,7 +145,7 @@ __global__ void __launch_bounds__(FxCoShape<P1>::NT, FxCoShape<P1>::MINB)
   extern __shared__ __align__(16) double smem_fx[];
   if (a.state != nullptr && a.state->stop) return;
   double* red = smem_fx;                                  // 32 * NC
-  unsigned* smax = reinterpret_cast<unsigned*>(red + 96);  // [2][EB] of u, then [2][EB] of the fluxes
+  unsigned* smax = reinterpret_cast<unsigned*>(red + 96);  // [u, fluxes][2][EB]
   const int tid = threadIdx.x;
   const int slot = tid / PP;
   const bool live = slot < EB;  // threads that pad the block to whole warps only take part in barriers
@@ -162,7 +163,7 @@ __global__ void __launch_bounds__(FxCoShape<P1>::NT, FxCoShape<P1>::MINB)
   // the slot's element of item `it` (a slot past the block's last element repeats that one, unstored)
   auto elem_of = [&](int it) { return e0 + min((it / NC) * EB + slot, nblk - 1); };
   const unsigned lanes = __match_any_sync(0xffffffffu, slot);  // the warp's lanes of this slot
-  const bool lead = (tid & 31) == __ffs(int(lanes)) - 1;
+  const bool lead = live && (tid & 31) == __ffs(int(lanes)) - 1;
 
   int g[P1];
   unsigned dnext = 0, dcur = 0;  // Dirichlet bits of the own column
@@ -216,9 +217,10 @@ __global__ void __launch_bounds__(FxCoShape<P1>::NT, FxCoShape<P1>::MINB)
     }
     mx = __reduce_max_sync(lanes, mx);
     const int ge = live && m.gexp != nullptr ? __ldg(m.gexp + e) : kFxNoGrid;
-    if (lead && live) atomicMax(smax + (it & 1) * EB + slot, mx);
+    const FxNorm norm{lanes, lead, smax + (it & 1) * EB + (live ? slot : 0), 2 * EB};
+    if (lead) atomicMax(norm.top, mx);
     __syncthreads();
-    int eb = live ? int(smax[(it & 1) * EB + slot] >> 20) : 1023;
+    int eb = live ? int(*norm.top >> 20) : 1023;
     const bool bad = live && (ge == kFxNoGrid || (eb != 0 && (eb < 500 || eb > 1500)));
     if (eb == 0) eb = 1023;  // every value is zero (or too small to matter to `bad` blocks): any exponent
     if (el.t == 0 && live) smax[(~it & 1) * EB + slot] = smax[(2 + (~it & 1)) * EB + slot] = 0u;
@@ -245,10 +247,9 @@ __global__ void __launch_bounds__(FxCoShape<P1>::NT, FxCoShape<P1>::MINB)
     }
     if (!__syncthreads_or(bad)) {
       const int4* G = m.Gfx + e * 3 * P3 + el.t;
-      unsigned* stop = smax + 2 * EB + (it & 1) * EB + slot;
       double sc = 0.0;
       fx_co_stages<P1, FxArith>(
-          el, tab.D, tab.DT, live,
+          el, tab.D, tab.DT, live, norm,
           [&](int k, int2 r, int2 s, int2 t, long long& fr, long long& fs, long long& ft) {
             const int4 g0 = __ldcs(G + (3 * k + 0) * PP), g1 = __ldcs(G + (3 * k + 1) * PP),
                        g2 = __ldcs(G + (3 * k + 2) * PP);
@@ -259,14 +260,7 @@ __global__ void __launch_bounds__(FxCoShape<P1>::NT, FxCoShape<P1>::MINB)
             ft = fx_dot3(g02, r, g12, s, g22, t);
           },
           mid,
-          [&](const FxArith& ar) {
-            const unsigned top = __reduce_max_sync(lanes, ar.range.top());
-            if (lead && live) atomicMax(stop, top);
-          },
-          [&](FxArith& ar) {
-            if (live) ar.set_shift(*stop);
-            sc = wij * __hiloint2double((eb + ge - ar.shift - (1082 - 1023)) << 20, 0);
-          },
+          [&](int shift) { sc = wij * __hiloint2double((eb + ge - shift - (1082 - 1023)) << 20, 0); },
           [&](int k, long long r, long long s, long long t) {
             finish(k, __ll2double_rn(r + s + t) * (tab.w[k] * sc));
           });
@@ -279,7 +273,7 @@ __global__ void __launch_bounds__(FxCoShape<P1>::NT, FxCoShape<P1>::MINB)
       __syncthreads();
       const double* G = a.G + e * 6 * P3 + el.t;
       fx_co_stages<P1, F64Arith>(
-          el, tab.D64, tab.DT64, live,
+          el, tab.D64, tab.DT64, live, norm,
           [&](int k, double r, double s, double t, double& fr, double& fs, double& ft) {
             const double* Gk = G + k * PP;
             const double g00 = __ldcs(Gk), g01 = __ldcs(Gk + P3), g02 = __ldcs(Gk + 2 * P3), g11 = __ldcs(Gk + 3 * P3),
@@ -288,7 +282,7 @@ __global__ void __launch_bounds__(FxCoShape<P1>::NT, FxCoShape<P1>::MINB)
             fs = g01 * r + g11 * s + g12 * t;
             ft = g02 * r + g12 * s + g22 * t;
           },
-          mid, [](const F64Arith&) {}, [](F64Arith&) {}, [&](int k, double r, double s, double t) { finish(k, r + s + t); });
+          mid, [](int) {}, [&](int k, double r, double s, double t) { finish(k, r + s + t); });
     }
     if (Sh::NU == 1 && live && it + 1 < nit) fetch_u(it + 1);  // the own column's values were read last above
 #pragma unroll
@@ -296,32 +290,8 @@ __global__ void __launch_bounds__(FxCoShape<P1>::NT, FxCoShape<P1>::MINB)
       if (q == c) dot[q] += acc;
   }
 
-  if (a.partials != nullptr) {
-    if (grid_sum_last<NC>(dot, a.partials, gridDim.x, blockIdx.x, &a.state->ticket[kTicketApply], red)) {
-      if (threadIdx.x == 0) {
-        SolveState* st = a.state;
-        int any = 0;
-#pragma unroll
-        for (int c = 0; c < NC; ++c) {
-          CompScalars& cs = st->c[c];
-          if (!cs.active) continue;
-          const double pAp = dot[c];
-          cs.pAp = pAp;
-          if (!(pAp > 0.0) || !isfinite(pAp) || !isfinite(cs.rz)) {
-            cs.status = CEEDBP_EBREAKDOWN;
-            cs.alpha = 0.0;
-            if (!st->fixed) cs.active = 0;
-          } else {
-            cs.alpha = cs.rz / pAp;
-          }
-          any |= cs.active;
-        }
-        if (!any) st->stop = 1;
-      }
-    }
-  }
+  if (a.partials != nullptr) cg_alpha<NC>(dot, a.partials, a.state, red);
 }
-
 
 template <int P1>
 FxCoTab<P1> elem_fx_tab(const DeviceMesh& m) {
@@ -339,26 +309,15 @@ FxCoTab<P1> elem_fx_tab(const DeviceMesh& m) {
 // attribute that lets it use its shared memory is set on the way.
 template <int P1, int NC, bool HELM>
 int elem_fx_resident() {
-  static const int n = [] {
-    auto kern = elem_fx_kernel<P1, NC, HELM>;
-    int dev = 0, sms = 0, nb = 0;
-    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, int(FxCoShape<P1>::SMEM)) !=
-            cudaSuccess ||
-        cudaGetDevice(&dev) != cudaSuccess ||
-        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, kern, FxCoShape<P1>::NT, FxCoShape<P1>::SMEM) != cudaSuccess)
-      return 0;
-    return nb * sms;
-  }();
+  using Sh = FxCoShape<P1>;
+  static const int n = fx_resident(reinterpret_cast<const void*>(elem_fx_kernel<P1, NC, HELM>), Sh::NT, Sh::SMEM);
   return n;
 }
 
 // Elements in a slot's sequence: one wave of resident blocks covers the mesh.
 template <int P1, int NC>
 int elem_fx_seq(int64_t nelem) {
-  const int res = std::max(1, elem_fx_resident<P1, NC, false>());
-  const int64_t full = (nelem + FxCoShape<P1>::EB - 1) / FxCoShape<P1>::EB;
-  return int(std::min<int64_t>(kFxMaxSeq, (full + res - 1) / res));
+  return fx_seq(nelem, FxCoShape<P1>::EB, elem_fx_resident<P1, NC, false>());
 }
 
 template <int P1, int NC>

@@ -1,5 +1,7 @@
-// Dispatch of the fixed-point BK5/BK6 kernel (elem_fx.cuh) by order; instantiated in elem_fx_[a-e].cu.
+// Dispatch of the fixed-point kernels by order: BK5/BK6 (elem_fx.cuh, instantiated in elem_fx_[a-e].cu) and
+// BK1..BK4 (elem_fxgl.cuh, instantiated in elem_fxgl_[a-h].cu).
 #include "elem_fx.cuh"
+#include "elem_fxgl.cuh"
 
 namespace ceedbp {
 
@@ -9,7 +11,9 @@ namespace ceedbp {
 #define X(P)                                                                                    \
   extern template cudaError_t launch_elem_fx_t<P>(const DeviceMesh&, const ElemArgs&, cudaStream_t); \
   extern template int elem_fx_blocks_t<P, 1>(int64_t);                                          \
-  extern template int elem_fx_blocks_t<P, 3>(int64_t);
+  extern template int elem_fx_blocks_t<P, 3>(int64_t); \
+  extern template cudaError_t launch_elem_fxgl_t<P>(const DeviceMesh&, int, const ElemArgs&, cudaStream_t); \
+  extern template int elem_fxgl_blocks_any<P>(const DeviceMesh&);
 CEEDBP_FX_P1(X)
 #undef X
 
@@ -27,6 +31,26 @@ int elem_fx_blocks(const DeviceMesh& m) {
   switch (m.p1) {
 #define X(P) \
   case P: return m.ncomp == 3 ? elem_fx_blocks_t<P, 3>(m.nelem) : elem_fx_blocks_t<P, 1>(m.nelem);
+    CEEDBP_FX_P1(X)
+#undef X
+    default: return 0;
+  }
+}
+
+cudaError_t launch_elem_fxgl(const DeviceMesh& m, int kind, const ElemArgs& a, cudaStream_t s) {
+  switch (m.p1) {
+#define X(P) \
+  case P: return launch_elem_fxgl_t<P>(m, kind, a, s);
+    CEEDBP_FX_P1(X)
+#undef X
+    default: return cudaErrorInvalidValue;
+  }
+}
+
+int elem_fxgl_blocks(const DeviceMesh& m) {
+  switch (m.p1) {
+#define X(P) \
+  case P: return elem_fxgl_blocks_any<P>(m);
     CEEDBP_FX_P1(X)
 #undef X
     default: return 0;

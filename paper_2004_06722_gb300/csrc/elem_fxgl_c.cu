@@ -1,0 +1,9 @@
+// Instantiations of the fixed-point BK1..BK4 kernel (elem_fxgl.cuh), p1 = 8, 9.
+#include "elem_fxgl.cuh"
+
+namespace ceedbp {
+template cudaError_t launch_elem_fxgl_t<8>(const DeviceMesh& m, int kind, const ElemArgs& a, cudaStream_t s);
+template int elem_fxgl_blocks_any<8>(const DeviceMesh& m);
+template cudaError_t launch_elem_fxgl_t<9>(const DeviceMesh& m, int kind, const ElemArgs& a, cudaStream_t s);
+template int elem_fxgl_blocks_any<9>(const DeviceMesh& m);
+}  // namespace ceedbp

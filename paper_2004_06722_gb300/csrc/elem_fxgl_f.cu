@@ -1,0 +1,9 @@
+// Instantiations of the fixed-point BK1..BK4 kernel (elem_fxgl.cuh), p1 = 13, 14.
+#include "elem_fxgl.cuh"
+
+namespace ceedbp {
+template cudaError_t launch_elem_fxgl_t<13>(const DeviceMesh& m, int kind, const ElemArgs& a, cudaStream_t s);
+template int elem_fxgl_blocks_any<13>(const DeviceMesh& m);
+template cudaError_t launch_elem_fxgl_t<14>(const DeviceMesh& m, int kind, const ElemArgs& a, cudaStream_t s);
+template int elem_fxgl_blocks_any<14>(const DeviceMesh& m);
+}  // namespace ceedbp

@@ -157,31 +157,40 @@ __device__ __forceinline__ long long fx_dot3(int2 a, int2 x, int2 b, int2 y, int
   return fx_join(hh, mm);
 }
 
-// Largest magnitude of a set of values by their upper words, and the shift that moves it up to 2^60.
-struct FxRange {
-  int hi = 0, lo = 0;
-  __device__ __forceinline__ void add(long long y) {
-    const int w = int(y >> 32);
-    hi = max(hi, w);
-    lo = min(lo, w);
-  }
-  __device__ __forceinline__ unsigned top() const { return unsigned(max(hi, ~lo)); }
+// Where the threads of an element exchange the largest magnitude of a stage's values: one word for each
+// stage, `step` words apart.
+struct FxNorm {
+  unsigned lanes;  // the warp's lanes of this element
+  bool lead;       // one of them in each warp (false for threads without an element)
+  unsigned* top;
+  int step;
 };
-__device__ __forceinline__ int fx_shift(unsigned top) { return min(max(__clz(int(top)) - 4, 0), 30); }
 
-// The two arithmetics of the element kernels: L a stage's input, Raw its output.
+// The two arithmetics of the element kernels: L a stage's input, Raw its output.  see() collects the
+// magnitudes (by upper words) of raw values that the next stage reads with load(); publish() before and
+// take() after a barrier turn the element's largest into the shift that moves it up to 2^60.
 struct FxArith {
   using L = int2;
   using Raw = long long;
   static constexpr long long kBias = kFxHalf;
-  FxRange range;
-  int shift = 0;
+  int hi = 0, lo = 0;
+  int shift = 0, total = 0;
   long long bias = 0;  // kFxHalf on the unshifted grid
   __device__ __forceinline__ static L limbs(long long yb) { return fx_limbs(yb); }  // of a biased output
   __device__ __forceinline__ L load(Raw y) const { return fx_limbs_up(y + bias, shift); }
-  __device__ __forceinline__ void see(Raw y) { range.add(y); }
-  __device__ __forceinline__ void set_shift(unsigned top) {
-    shift = fx_shift(top);
+  __device__ __forceinline__ void see(Raw y) {
+    const int w = int(y >> 32);
+    hi = max(hi, w);
+    lo = min(lo, w);
+  }
+  __device__ __forceinline__ void publish(const FxNorm& n, int stage) {
+    const unsigned t = __reduce_max_sync(n.lanes, unsigned(max(hi, ~lo)));
+    if (n.lead) atomicMax(n.top + stage * n.step, t);
+    hi = lo = 0;
+  }
+  __device__ __forceinline__ void take(const FxNorm& n, int stage) {
+    shift = min(max(__clz(int(n.top[stage * n.step])) - 4, 0), 30);
+    total += shift;
     bias = kFxHalf >> shift;
   }
 };
@@ -189,11 +198,33 @@ struct F64Arith {
   using L = double;
   using Raw = double;
   static constexpr long long kBias = 0;
+  int total = 0;
   __device__ __forceinline__ static L limbs(double y) { return y; }
   __device__ __forceinline__ L load(Raw y) const { return y; }
   __device__ __forceinline__ void see(Raw) {}
+  __device__ __forceinline__ void publish(const FxNorm&, int) {}
+  __device__ __forceinline__ void take(const FxNorm&, int) {}
 };
 
 __device__ __forceinline__ void l2_prefetch(const void* p) { asm volatile("prefetch.global.L2 [%0];" ::"l"(p)); }
+
+// Host: blocks of a kernel resident on the GPU (0: it does not fit), and the attribute that lets it use its
+// shared memory.
+inline int fx_resident(const void* kernel, int threads, size_t smem) {
+  int dev = 0, sms = 0, nb = 0;
+  if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem)) != cudaSuccess ||
+      cudaGetDevice(&dev) != cudaSuccess ||
+      cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
+      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, kernel, threads, smem) != cudaSuccess)
+    return 0;
+  return nb * sms;
+}
+
+// Host: elements in a slot's sequence such that one wave of resident blocks covers the mesh.
+inline int fx_seq(int64_t nelem, int per_block, int resident) {
+  const int64_t full = (nelem + per_block - 1) / per_block, res = resident < 1 ? 1 : resident;
+  const int64_t n = (full + res - 1) / res;
+  return int(n < kFxMaxSeq ? n : kFxMaxSeq);
+}
 
 }  // namespace ceedbp

@@ -143,8 +143,8 @@ cudaError_t launch_fx_factors(const DeviceMesh& m, int kind, const double* G, vo
   return cudaGetLastError();
 }
 
-// Even-odd tables of D and of the weighted transposes. With W the quadrature weights and v the GLL
-// weights: DT = W^-1 D^T W, JT = v^-1 J^T W, so that W (DT f) = D^T (W f) and v (JT f) = J^T (W f).
+// Even-odd tables of D and of the weighted transposes. With W the quadrature weights: DT = W^-1 D^T W and,
+// with s_i = sum_q |J_qi| w_q, JT = s^-1 J^T W, so that W (DT f) = D^T (W f) and s (JT f) = J^T (W f).
 void build_fx_tables(const Basis1D& b, FxTables* t) {
   const int p = b.p1, q = b.q;
   std::vector<long double> M(size_t(q) * q), MT(size_t(q) * q);
@@ -165,11 +165,15 @@ void build_fx_tables(const Basis1D& b, FxTables* t) {
   t->chain = d * dt;
   if (b.colloc) return;
   std::vector<long double> J(size_t(q) * p), JT(size_t(q) * p);
-  for (int i = 0; i < q; ++i)
-    for (int j = 0; j < p; ++j) {
+  for (int j = 0; j < p; ++j) {
+    long double sj = 0.0L;
+    for (int i = 0; i < q; ++i) sj += std::fabs((long double)b.J[size_t(i) * p + j]) * b.w[i];
+    t->w[j] = double(sj);
+    for (int i = 0; i < q; ++i) {
       J[size_t(i) * p + j] = b.J[size_t(i) * p + j];
-      JT[size_t(j) * q + i] = (long double)b.J[size_t(i) * p + j] * b.w[i] / b.rho[j];
+      JT[size_t(j) * q + i] = (long double)b.J[size_t(i) * p + j] * b.w[i] / t->w[j];
     }
+  }
   const long double js = eo_tables(q, p, false, J, 62, &t->J, &t->J64);
   const long double jt = eo_tables(p, q, false, JT, 62, &t->JT, &no_f64);
   for (int i = 0; i < q; ++i)

@@ -38,7 +38,7 @@ inline size_t basis_doubles(int p1, int q) { return size_t(2) * q * p1 + size_t(
 struct FxTables {
   std::vector<int> D, DT, J, JT;
   std::vector<double> D64, DT64, J64, JT64;
-  std::vector<double> w;  // GLL weights
+  std::vector<double> w;  // weights of the result: GLL, or s of the Gauss tables (elem_fxgl.cuh)
   long double chain = 1.0L, mchain = 1.0L;
 };
 
@@ -162,6 +162,8 @@ cudaError_t launch_coords_soa(const double* coords, double* X, int64_t nelem, in
 cudaError_t launch_fx_factors(const DeviceMesh& m, int kind, const double* G, void* out, int* gexp, cudaStream_t s);
 cudaError_t launch_elem_fx(const DeviceMesh& m, const ElemArgs& a, cudaStream_t s);
 int elem_fx_blocks(const DeviceMesh& m);
+cudaError_t launch_elem_fxgl(const DeviceMesh& m, int kind, const ElemArgs& a, cudaStream_t s);
+int elem_fxgl_blocks(const DeviceMesh& m);
 
 // Gather-scatter sum w[g] = sum_slots wl (masked on Dirichlet nodes if mask_out).
 cudaError_t launch_gs(const DeviceMesh& m, const double* wl, double* w, int mask_out, cudaStream_t s);

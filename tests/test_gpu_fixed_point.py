@@ -41,7 +41,10 @@ def _run(op, uL):
 
 # element counts around the elements per block (32, 14, 8, 5, 7 and 1 from order 1 up)
 CASES = [(5, 1, 31), (5, 1, 33), (5, 2, 15), (5, 3, 9), (5, 4, 6), (5, 5, 8), (5, 6, 3), (5, 8, 2), (5, 9, 2),
-         (5, 10, 1), (5, 11, 1), (5, 12, 1), (6, 1, 33), (6, 4, 6), (6, 6, 2), (6, 9, 1)]
+         (5, 10, 1), (5, 11, 1), (5, 12, 1), (6, 1, 33), (6, 4, 6), (6, 6, 2), (6, 9, 1),
+         (1, 1, 15), (1, 2, 9), (1, 3, 4), (1, 4, 8), (1, 5, 2), (1, 8, 2), (1, 12, 1), (2, 2, 9), (2, 6, 2), (2, 11, 1),
+         (3, 1, 15), (3, 2, 7), (3, 3, 6), (3, 4, 6), (3, 6, 3), (3, 8, 2), (3, 10, 1), (3, 11, 1), (3, 12, 1),
+         (4, 1, 15), (4, 3, 6), (4, 5, 2), (4, 9, 1)]
 
 
 @pytest.mark.parametrize("bp,N,E", CASES)
@@ -55,7 +58,7 @@ def test_element_operator(bp, N, E):
     assert np.linalg.norm(w - ref) < 1e-12 * np.linalg.norm(ref)
 
 
-@pytest.mark.parametrize("bp,N", [(5, 2), (5, 3), (5, 7), (6, 5)])
+@pytest.mark.parametrize("bp,N", [(5, 2), (5, 3), (5, 7), (6, 5), (1, 3), (2, 2), (3, 4), (3, 7), (4, 3)])
 def test_element_sequences_agree(bp, N):
     """Every copy of one element in a mesh long enough for element sequences gives the same bits."""
     E = 40000 if N < 6 else 9000
@@ -67,12 +70,13 @@ def test_element_sequences_agree(bp, N):
     assert bool((w == w[:1]).all())
 
 
-@pytest.mark.parametrize("N", [3, 6, 7, 15])
+@pytest.mark.parametrize("bp,N", [(5, 3), (5, 6), (5, 7), (5, 15), (1, 5), (3, 7), (3, 15), (4, 2)])
 @pytest.mark.parametrize("k", [-900, -400, 300, 700])
-def test_power_of_two_scaling(N, k):
+def test_power_of_two_scaling(bp, N, k):
     """2^k u: inside the grid's exponent range the same integers, outside it the FP64 form."""
-    op = pkg.Operator.box(5, 2, 1, 1, N)
-    uL = uniform_pm1(5, np.arange(2 * (N + 1) ** 3)).reshape(2, -1)
+    op = pkg.Operator.box(bp, 2, 1, 1, N)
+    shape = (2, (N + 1) ** 3) if op.ncomp == 1 else (2, (N + 1) ** 3, 3)
+    uL = uniform_pm1(5, np.arange(int(np.prod(shape)))).reshape(shape)
     w0, w1 = _run(op, uL), np.ldexp(_run(op, np.ldexp(uL, k)), -k)
     if abs(k) <= 400:
         np.testing.assert_array_equal(w0, w1)
@@ -98,6 +102,19 @@ def test_non_finite_values(N, bad):
     assert np.abs(w[[0, 2]] - clean[[0, 2]]).max() < 1e-12 * np.abs(clean).max()
 
 
+@pytest.mark.parametrize("bp,N", [(1, 3), (1, 7), (3, 4), (3, 7)])
+@pytest.mark.parametrize("bad", [np.nan, np.inf])
+def test_non_finite_values_gauss(bp, N, bad):
+    """Interpolation reaches every node of the element, and no other element."""
+    op = pkg.Operator.box(bp, 1, 3, 1, N)
+    uL = uniform_pm1(6, np.arange(3 * (N + 1) ** 3)).reshape(3, -1)
+    clean = _run(op, uL)
+    uL[1, 5] = bad
+    w = _run(op, uL)
+    assert not np.isfinite(w[1]).any()
+    assert np.abs(w[[0, 2]] - clean[[0, 2]]).max() < 1e-12 * np.abs(clean).max()
+
+
 @pytest.mark.parametrize("N,contrast", [(3, 30.0), (7, 100.0), (7, 1e6), (4, 1e9), (5, 0.0)])
 def test_coefficient_contrast(N, contrast):
     """kappa jumping inside an element: below 2^7 on the grid, above it (and with zeros) in FP64."""
@@ -114,7 +131,7 @@ def test_coefficient_contrast(N, contrast):
         assert np.linalg.norm(w[e] - ref[e]) < 1e-12 * np.linalg.norm(ref[e])
 
 
-@pytest.mark.parametrize("bp,N", [(5, 4), (6, 3)])
+@pytest.mark.parametrize("bp,N", [(5, 4), (6, 3), (1, 4), (3, 5)])
 def test_zero_and_sparse_elements(bp, N):
     op = pkg.Operator.box(bp, 3, 1, 1, N)
     p3 = (N + 1) ** 3
