@@ -79,7 +79,7 @@ cudaError_t dalloc(T** p, size_t count) {
 void release(ceedbp_ctx* c) {
   for (auto& g : c->graphs) cudaGraphExecDestroy(g.exec);
   c->graphs.clear();
-  void* ptrs[] = {c->d_l2g, c->d_off, c->d_slots, c->d_basis, c->d_G, c->d_Mq, c->d_dinv, c->d_mdiag,
+  void* ptrs[] = {c->d_l2g, c->d_off, c->d_slots, c->d_head, c->d_basis, c->d_G, c->d_Mq, c->d_dinv, c->d_mdiag,
                   c->d_wl, c->d_r, c->d_p, c->d_ax, c->d_part_apply, c->d_part_vec, c->d_state,
                   c->d_Gdf, c->d_Ddf, c->d_dinvdf, c->d_G32, c->d_Gbf, c->d_dinv32, c->d_xin,
                   c->d_rin, c->d_pin, c->d_outer, c->d_Ghat, c->d_scal, c->d_X, c->d_l2g_id, c->d_Gfx, c->d_gexp, c->d_Mfx,
@@ -192,7 +192,8 @@ ceedbp_status setup_impl(ceedbp_ctx* c, const double* coords, const int64_t* l2g
   const int64_t n = P.nglobal;
   CK(c, dalloc(&c->d_l2g, nloc));
   CK(c, dalloc(&c->d_off, n + 1));
-  CK(c, dalloc(&c->d_slots, nloc));
+  CK(c, dalloc(&c->d_slots, nloc + kSlotPad));
+  CK(c, dalloc(&c->d_head, n));
   CK(c, dalloc(&c->d_basis, hb.size()));
   if (c->op_kind == kStiff) CK(c, dalloc(&c->d_G, size_t(P.nelem) * 6 * Q3));
   CK(c, dalloc(&c->d_Mq, size_t(P.nelem) * Q3));
@@ -212,6 +213,8 @@ ceedbp_status setup_impl(ceedbp_ctx* c, const double* coords, const int64_t* l2g
   CK(c, cudaMemcpyAsync(c->d_l2g, hl2g.data(), sizeof(int) * nloc, cudaMemcpyHostToDevice, s));
   CK(c, cudaMemcpyAsync(c->d_off, hoff.data(), sizeof(int) * (n + 1), cudaMemcpyHostToDevice, s));
   CK(c, cudaMemcpyAsync(c->d_slots, hslots.data(), sizeof(int) * nloc, cudaMemcpyHostToDevice, s));
+  CK(c, cudaMemsetAsync(c->d_slots + nloc, 0, sizeof(int) * kSlotPad, s));
+  CK(c, launch_heads(c->d_off, c->d_slots, c->d_head, n, s));
   CK(c, cudaMemcpyAsync(c->d_basis, hb.data(), sizeof(double) * hb.size(), cudaMemcpyHostToDevice, s));
   CK(c, cudaMemsetAsync(c->d_state, 0, sizeof(SolveState), s));
 
@@ -226,6 +229,7 @@ ceedbp_status setup_impl(ceedbp_ctx* c, const double* coords, const int64_t* l2g
   m.l2g = c->d_l2g;
   m.off = c->d_off;
   m.slots = c->d_slots;
+  m.head = c->d_head;
   m.basis = c->d_basis;
   build_fx_tables(basis, &c->fx);
   m.fx = &c->fx;
@@ -498,13 +502,12 @@ void run_inner_iterations(ceedbp_ctx* c, int mode, int n) {
   for (int i = 0; i < n; ++i) {
     if (mode == CEEDBP_MIXED_FP32_TC) launch_elem_tc(m, a, c->stream);
     else launch_elem_lp(m, a, bf16, c->stream);
-    launch_inner_update(m, bf16, a.wl, c->d_xin, c->d_rin, c->d_pin, c->d_dinv32, c->d_part_vec, c->d_state,
-                        c->stream);
-    launch_inner_dir(m, bf16, c->d_rin, c->d_pin, c->d_dinv32, c->d_state, c->stream);
+    launch_inner_update(m, a.wl, c->d_rin, c->d_dinv32, c->d_part_vec, c->d_state, i, c->stream);
+    launch_inner_dir(m, bf16, c->d_rin, c->d_pin, c->d_xin, c->d_dinv32, c->d_state, i, c->stream);
   }
 }
 
-void run_iterations(ceedbp_ctx* c, double* x, int n, bool profile = false, bool capturing = false) {
+void run_iterations(ceedbp_ctx* c, int n, bool profile = false, bool capturing = false) {
   const DeviceMesh& m = c->mesh;
   ElemArgs a{};
   a.u = c->d_p;
@@ -530,11 +533,11 @@ void run_iterations(ceedbp_ctx* c, double* x, int n, bool profile = false, bool 
     if (df) launch_elem_df(m, da, c->stream);
     else launch_elem(m, c->op_kind, a, c->stream);
     if (profile) mark(c, 4 * i + 1, capturing);
-    if (df) launch_update_df(m, wd, xd, rd, pd, c->d_dinvdf, c->d_part_vec, c->d_state, c->stream);
-    else launch_pcg_update(m, c->d_wl, x, c->d_r, c->d_p, c->d_dinv, c->d_part_vec, c->d_state, c->stream);
+    if (df) launch_update_df(m, wd, rd, c->d_dinvdf, c->d_part_vec, c->d_state, i, c->stream);
+    else launch_pcg_update(m, c->d_wl, c->d_r, c->d_dinv, c->d_part_vec, c->d_state, i, c->stream);
     if (profile) mark(c, 4 * i + 2, capturing);
-    if (df) launch_dir_df(m, rd, pd, c->d_dinvdf, c->d_state, c->stream);
-    else launch_pcg_dir(m, c->d_r, c->d_p, c->d_dinv, c->d_state, c->stream);
+    if (df) launch_dir_df(m, rd, pd, xd, c->d_dinvdf, c->d_state, i, c->stream);
+    else launch_pcg_dir(m, c->d_r, c->d_p, c->d_dinv, c->d_state, i, c->stream);
     if (profile) mark(c, 4 * i + 3, capturing);
   }
 }
@@ -548,15 +551,15 @@ ceedbp_status ensure_prof_events(ceedbp_ctx* c, int n) {
   return CEEDBP_OK;
 }
 
-ceedbp_status graph_for(ceedbp_ctx* c, double* x, int n, int profile, cudaGraphExec_t* out, int mode = 0) {
+ceedbp_status graph_for(ceedbp_ctx* c, int n, int profile, cudaGraphExec_t* out, int mode = 0) {
   for (auto& g : c->graphs)
-    if (g.x == x && g.n == n && g.profile == profile && g.mode == mode) {
+    if (g.n == n && g.profile == profile && g.mode == mode) {
       *out = g.exec;
       return CEEDBP_OK;
     }
   cudaGraph_t graph = nullptr;
   CK(c, cudaStreamBeginCapture(c->stream, cudaStreamCaptureModeThreadLocal));
-  if (mode == 0) run_iterations(c, x, n, profile != 0, true);
+  if (mode == 0) run_iterations(c, n, profile != 0, true);
   else run_inner_iterations(c, mode, n);
   cudaError_t e = cudaStreamEndCapture(c->stream, &graph);
   if (e != cudaSuccess) return cuda_fail(c, e, "cudaStreamEndCapture");
@@ -568,7 +571,7 @@ ceedbp_status graph_for(ceedbp_ctx* c, double* x, int n, int profile, cudaGraphE
     cudaGraphExecDestroy(c->graphs.front().exec);
     c->graphs.erase(c->graphs.begin());
   }
-  c->graphs.push_back({x, n, profile, mode, exec});
+  c->graphs.push_back({n, profile, mode, exec});
   *out = exec;
   return CEEDBP_OK;
 }
@@ -636,7 +639,7 @@ ceedbp_status solve_mixed(ceedbp_ctx* c, const double* b, double* x, const ceedb
       const int k = std::min(o.chunk, inner_maxit - its);
       if (graphs) {
         cudaGraphExec_t exec = nullptr;
-        ceedbp_status st = graph_for(c, nullptr, k, 0, &exec, o.mixed);
+        ceedbp_status st = graph_for(c, k, 0, &exec, o.mixed);
         if (st != CEEDBP_OK) return st;
         CK(c, cudaGraphLaunch(exec, s));
       } else {
@@ -840,11 +843,11 @@ ceedbp_status ceedbp_solve(ceedbp_ctx* c, const double* b, double* x, const ceed
     const int k = std::min(o.chunk, limit - done);
     if (graphs) {
       cudaGraphExec_t exec = nullptr;
-      ceedbp_status st = graph_for(c, x, k, profile ? 1 : 0, &exec);
+      ceedbp_status st = graph_for(c, k, profile ? 1 : 0, &exec);
       if (st != CEEDBP_OK) return st;
       CK(c, cudaGraphLaunch(exec, s));
     } else {
-      run_iterations(c, x, k, profile, false);
+      run_iterations(c, k, profile, false);
       CK(c, cudaGetLastError());
     }
     CK(c, cudaEventRecord(c->ev1, s));

@@ -94,7 +94,7 @@ __global__ void batch_update_kernel(const int* __restrict__ off, const int* __re
     if (o0 < 0) continue;
     const int o1 = __ldg(off + g + 1) & 0x7fffffff;
     dfloat w{0.0f, 0.0f};
-    for (int k = o0; k < o1; ++k) w = dw_add(w, wl[__ldg(slots + k)]);
+    for (int k = o0; k < o1; ++k) w = dw_add(w, wl[__ldg(slots + k) & 0x7fffffff]);
     const dfloat rv = dw_add(r[g], dw_neg(dw_mul(alpha, w)));
     x[g] = dw_add(x[g], dw_mul(alpha, p[g]));
     r[g] = rv;
@@ -183,7 +183,7 @@ __global__ void batch_update64_kernel(const int* __restrict__ off, const int* __
     if (o0 < 0) continue;
     const int o1 = __ldg(off + g + 1) & 0x7fffffff;
     double w = 0.0;
-    for (int k = o0; k < o1; ++k) w += wl[__ldg(slots + k)];
+    for (int k = o0; k < o1; ++k) w += wl[__ldg(slots + k) & 0x7fffffff];
     const double rv = r[g] - alpha * w;
     x[g] += alpha * p[g];
     r[g] = rv;

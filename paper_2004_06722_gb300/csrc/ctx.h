@@ -9,7 +9,6 @@
 #include "kernel_args.h"
 
 struct GraphEntry {
-  double* x;
   int n;
   int profile;
   int mode;  // 0: FP64 / pair iteration, else the CEEDBP_MIXED_* precision of the inner iterations
@@ -25,6 +24,7 @@ struct ceedbp_ctx {
   int* d_l2g = nullptr;
   int* d_off = nullptr;
   int* d_slots = nullptr;
+  int* d_head = nullptr;
   double* d_basis = nullptr;
   double* d_G = nullptr;
   ceedbp::FxTables fx;               // host tables of the fixed-point kernels

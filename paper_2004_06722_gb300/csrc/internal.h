@@ -47,6 +47,9 @@ constexpr int kFxNoGrid = -(1 << 30);
 struct Basis1D;
 void build_fx_tables(const Basis1D& b, FxTables* t);
 
+// Entries behind the last list of `slots` that the gather may read (gather.cuh).
+constexpr int kSlotPad = 8;
+
 // Longest element sequence of a slot of the fixed-point kernels.
 constexpr int kFxMaxSeq = 16;
 
@@ -63,7 +66,7 @@ struct CompScalars {
   int iters;     // iterations performed
   int active;    // 1 while the component is iterating
   int status;    // CEEDBP_OK or CEEDBP_EBREAKDOWN
-  int pad;
+  int xstep;     // 1: the last update kernel took a step of this component (x += alpha p is the direction kernel's)
 };
 
 struct SolveState {
@@ -73,6 +76,8 @@ struct SolveState {
   int stop;      // 1: every component inactive; kernels return at once
   int fault;     // nonzero: a kernel gave up a bounded wait (its results are invalid)
   unsigned int ticket[4];  // last-block counters, one per reduction site
+  double* x;     // solution of the FP64 iteration (captured iterations take any x)
+  int step;      // iteration of the chunk whose update kernel ran last, -1 before the first
 };
 
 // Per-problem CG scalars of batched solves.
@@ -93,7 +98,8 @@ struct DeviceMesh {
   int64_t nelem, nglobal;
   const int* l2g;       // [E][p1^3]; Dirichlet nodes encoded as -(g+1)
   const int* off;       // [nglobal+1]; bit 31 of off[g] = Dirichlet flag of node g
-  const int* slots;     // [E p1^3] local slots sorted by node, then slot
+  const int* slots;     // [E p1^3] local slots sorted by node, then slot; bit 31 = last of its node
+  const int* head;      // [nglobal] way into slots, see gather.cuh
   const double* basis;  // device 1D tables (layout above)
   int tune_eb;          // elements per block of the FP32-pair kernel (0 = default; set by the autotuner)
   int tune_stage;       // pair kernel schedule (autotuner): 0 G ring by cp.async, 1 G staged by a bulk
@@ -172,13 +178,17 @@ cudaError_t launch_dinv(const int* off, const double* diag, double* dinv, int64_
 
 // PCG kernels.
 int vec_blocks(int64_t n);
+inline int gather_blocks(int64_t n) { return vec_blocks((n + 1) / 2); }  // two nodes a thread
 cudaError_t launch_pcg_init(const DeviceMesh& m, const double* b, const double* ax, double* x, double* r, double* p,
                             const double* dinv, double* partials, SolveState* st, double tol,
                             int fixed, cudaStream_t s);
-cudaError_t launch_pcg_update(const DeviceMesh& m, const double* wl, double* x, double* r, const double* p,
-                              const double* dinv, double* partials, SolveState* st, cudaStream_t s);
+// step: the iteration's index in its chunk; the direction kernel takes x += alpha p of the update that ran with it
+cudaError_t launch_pcg_update(const DeviceMesh& m, const double* wl, double* r, const double* dinv, double* partials,
+                              SolveState* st, int step, cudaStream_t s);
 cudaError_t launch_pcg_dir(const DeviceMesh& m, const double* r, double* p, const double* dinv,
-                           const SolveState* st, cudaStream_t s);
+                           const SolveState* st, int step, cudaStream_t s);
+// head[] of gather.cuh from the CSR offsets, and bit 31 of each node's last slot
+cudaError_t launch_heads(const int* off, int* slots, int* head, int64_t n, cudaStream_t s);
 
 // FP32-pair path (df.cuh, elem_df.cuh, pcg_df.cu).
 struct dfloat;
@@ -198,10 +208,10 @@ cudaError_t launch_elem_dfgl(const DeviceMesh& m, const ElemDfArgs& a, cudaStrea
 cudaError_t launch_init_df(const DeviceMesh& m, const double* b, const double* ax, double* x, dfloat* xd, dfloat* r,
                            dfloat* p, const dfloat* dinv, int x0, double* partials, SolveState* st, double tol,
                            int fixed, cudaStream_t s);
-cudaError_t launch_update_df(const DeviceMesh& m, const dfloat* wl, dfloat* x, dfloat* r, const dfloat* p,
-                             const dfloat* dinv, double* partials, SolveState* st, cudaStream_t s);
-cudaError_t launch_dir_df(const DeviceMesh& m, const dfloat* r, dfloat* p, const dfloat* dinv, const SolveState* st,
-                          cudaStream_t s);
+cudaError_t launch_update_df(const DeviceMesh& m, const dfloat* wl, dfloat* r, const dfloat* dinv, double* partials,
+                             SolveState* st, int step, cudaStream_t s);
+cudaError_t launch_dir_df(const DeviceMesh& m, const dfloat* r, dfloat* p, dfloat* x, const dfloat* dinv,
+                          const SolveState* st, int step, cudaStream_t s);
 cudaError_t launch_df_to_f64(const dfloat* src, double* dst, int64_t n, cudaStream_t s);
 cudaError_t launch_f64_to_df(const double* src, dfloat* dst, int64_t n, cudaStream_t s);
 cudaError_t launch_gs_df(const DeviceMesh& m, const dfloat* wl, double* w, int mask_out, cudaStream_t s);
@@ -226,10 +236,10 @@ cudaError_t launch_residual(const DeviceMesh& m, const double* b, const double* 
 cudaError_t launch_inner_init(const DeviceMesh& m, int bf16, const double* r64, const double* scale,
                               const float* dinv, float* x, float* r, void* p, double* partials, SolveState* st,
                               double tol, cudaStream_t s);
-cudaError_t launch_inner_update(const DeviceMesh& m, int bf16, const float* wl, float* x, float* r, const void* p,
-                                const float* dinv, double* partials, SolveState* st, cudaStream_t s);
-cudaError_t launch_inner_dir(const DeviceMesh& m, int bf16, const float* r, void* p, const float* dinv,
-                             const SolveState* st, cudaStream_t s);
+cudaError_t launch_inner_update(const DeviceMesh& m, const float* wl, float* r, const float* dinv, double* partials,
+                                SolveState* st, int step, cudaStream_t s);
+cudaError_t launch_inner_dir(const DeviceMesh& m, int bf16, const float* r, void* p, float* x, const float* dinv,
+                             const SolveState* st, int step, cudaStream_t s);
 cudaError_t launch_correct(const DeviceMesh& m, double* x, const float* d, const double* norm, cudaStream_t s);
 cudaError_t launch_narrow(const double* src, void* dst, int64_t n, int bf16, cudaStream_t s);
 

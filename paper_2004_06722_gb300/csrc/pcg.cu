@@ -6,11 +6,11 @@
 //            dot before the direct-stiffness sum: it needs no multiplicity
 //            weighting); the last block forms alpha = rz / pAp.
 //   update : w = Q^T w_L (deterministic gather-scatter, masked), then
-//            x += alpha p, r -= alpha w, z = dinv r, and the sums (r, z), (r, r);
+//            r -= alpha w, z = dinv r, and the sums (r, z), (r, r);
 //            the last block forms beta = rz_new / rz and tests ||r|| <= tol ||b||.
-//   dir    : p = dinv r + beta p.
+//   dir    : x += alpha p, p = dinv r + beta p (p is read once for both).
 // Independent components (BP6) carry their own scalars and stop separately.
-#include "common.cuh"
+#include "gather.cuh"
 
 namespace ceedbp {
 
@@ -22,7 +22,7 @@ __global__ void pcg_init_kernel(const int* __restrict__ off, const double* __res
                                 double* __restrict__ p,
                                 const double* __restrict__ dinv, int64_t n, double* partials, SolveState* st,
                                 double tol, int fixed) {
-  __shared__ double red[32 * 3 * NC];
+  __shared__ double red[256 * 3 * NC];
   double acc[3 * NC];
 #pragma unroll
   for (int k = 0; k < 3 * NC; ++k) acc[k] = 0.0;
@@ -42,11 +42,13 @@ __global__ void pcg_init_kernel(const int* __restrict__ off, const double* __res
       acc[2 * NC + c] += bv * bv;
     }
   }
-  if (grid_sum_last<3 * NC>(acc, partials, gridDim.x, blockIdx.x, &st->ticket[kTicketInit], red)) {
+  if (grid_sum_last_256<3 * NC>(acc, partials, &st->ticket[kTicketInit], red)) {
     if (threadIdx.x == 0) {
       int any = 0;
       st->ncomp = NC;
       st->fixed = fixed;
+      st->x = x;
+      st->step = -1;
 #pragma unroll
       for (int c = 0; c < NC; ++c) {
         CompScalars& cs = st->c[c];
@@ -68,12 +70,15 @@ __global__ void pcg_init_kernel(const int* __restrict__ off, const double* __res
 }
 
 template <int NC>
-__global__ void pcg_update_kernel(const int* __restrict__ off, const int* __restrict__ slots,
-                                  const double* __restrict__ wl, double* __restrict__ x, double* __restrict__ r,
-                                  const double* __restrict__ p, const double* __restrict__ dinv, int64_t n,
-                                  double* partials, SolveState* st) {
-  __shared__ double red[32 * 2 * NC];
-  if (st->stop) return;
+__global__ void __launch_bounds__(256) pcg_update_kernel(const int* __restrict__ head, const int* __restrict__ slots,
+                                                         const double* __restrict__ wl, double* __restrict__ r,
+                                                         const double* __restrict__ dinv, int64_t n,
+                                                         double* partials, SolveState* st, int step) {
+  __shared__ double red[256 * 2 * NC];
+  if (st->stop) {
+    if (blockIdx.x == 0 && threadIdx.x == 0) st->step = -1;  // nothing for this iteration's direction kernel
+    return;
+  }
   double alpha[NC];
   bool act[NC];
 #pragma unroll
@@ -84,53 +89,39 @@ __global__ void pcg_update_kernel(const int* __restrict__ off, const int* __rest
   double acc[2 * NC];
 #pragma unroll
   for (int k = 0; k < 2 * NC; ++k) acc[k] = 0.0;
-  for (int64_t g = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; g < n; g += int64_t(gridDim.x) * blockDim.x) {
-    const int o0 = __ldg(off + g);
-    if (o0 < 0) continue;  // Dirichlet node: x, r, p stay zero
-    const int o1 = __ldg(off + g + 1) & 0x7fffffff;
-    // start from the first slot (one FP64 add fewer per node); a node no element touches sums to 0
-    double w[NC];
+  const int64_t stride = int64_t(gridDim.x) * 256;
+  for (int64_t g0 = int64_t(blockIdx.x) * 256 + threadIdx.x; g0 < n; g0 += 2 * stride) {
+    int hd[2];
+    double w[2][NC], rv[2][NC], di[2];
 #pragma unroll
-    for (int c = 0; c < NC; ++c) w[c] = 0.0;
-    if (o0 < o1) {
-      const int sl = __ldg(slots + o0);
+    for (int h = 0; h < 2; ++h) {
+      const int64_t g = g0 + h * stride < n ? g0 + h * stride : g0;
+      di[h] = dinv[g];
 #pragma unroll
-      for (int c = 0; c < NC; ++c) w[c] = __ldcs(wl + size_t(sl) * NC + c);
+      for (int c = 0; c < NC; ++c) rv[h][c] = r[size_t(g) * NC + c];
     }
-    // the remaining slots two at a time (loads issued together, sums in slot order)
-    int k = o0 + 1;
-    for (; k + 1 < o1; k += 2) {
-      const int s0 = __ldg(slots + k), s1 = __ldg(slots + k + 1);
+    gather_nodes<2, NC>(head, slots, wl, g0, stride, n, hd, w);
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      if (hd[h] == kHeadDirichlet) continue;  // Dirichlet node: x, r, p stay zero
 #pragma unroll
       for (int c = 0; c < NC; ++c) {
-        const double v0 = __ldcs(wl + size_t(s0) * NC + c), v1 = __ldcs(wl + size_t(s1) * NC + c);
-        w[c] += v0;
-        w[c] += v1;
+        if (!act[c]) continue;
+        const double v = rv[h][c] - alpha[c] * w[h][c];
+        r[size_t(g0 + h * stride) * NC + c] = v;
+        acc[c] += v * (di[h] * v);
+        acc[NC + c] += v * v;
       }
     }
-    if (k < o1) {
-      const int s0 = __ldg(slots + k);
-#pragma unroll
-      for (int c = 0; c < NC; ++c) w[c] += __ldcs(wl + size_t(s0) * NC + c);
-    }
-    const double di = dinv[g];
-#pragma unroll
-    for (int c = 0; c < NC; ++c) {
-      if (!act[c]) continue;
-      const size_t i = size_t(g) * NC + c;
-      const double rv = r[i] - alpha[c] * w[c];
-      x[i] += alpha[c] * p[i];
-      r[i] = rv;
-      acc[c] += rv * (di * rv);
-      acc[NC + c] += rv * rv;
-    }
   }
-  if (grid_sum_last<2 * NC>(acc, partials, gridDim.x, blockIdx.x, &st->ticket[kTicketUpdate], red)) {
+  if (grid_sum_last_256<2 * NC>(acc, partials, &st->ticket[kTicketUpdate], red)) {
     if (threadIdx.x == 0) {
       int any = 0;
+      st->step = step;
 #pragma unroll
       for (int c = 0; c < NC; ++c) {
         CompScalars& cs = st->c[c];
+        cs.xstep = cs.active;
         if (!cs.active) continue;
         const double rz_new = acc[c];
         cs.beta = cs.rz != 0.0 ? rz_new / cs.rz : 0.0;
@@ -150,24 +141,29 @@ __global__ void pcg_update_kernel(const int* __restrict__ off, const int* __rest
 }
 
 template <int NC>
-__global__ void pcg_dir_kernel(const int* __restrict__ off, const double* __restrict__ r, double* __restrict__ p,
-                               const double* __restrict__ dinv, int64_t n, const SolveState* st) {
-  if (st->stop) return;
-  double beta[NC];
-  bool act[NC];
+__global__ void pcg_dir_kernel(const int* __restrict__ head, const double* __restrict__ r, double* __restrict__ p,
+                               const double* __restrict__ dinv, int64_t n, const SolveState* st, int step) {
+  if (st->step != step) return;  // no update ran in this iteration (the solve had stopped)
+  double* __restrict__ x = st->x;
+  double alpha[NC], beta[NC];
+  bool xs[NC], act[NC];
 #pragma unroll
   for (int c = 0; c < NC; ++c) {
+    xs[c] = st->c[c].xstep != 0;
     act[c] = st->c[c].active != 0;
+    alpha[c] = st->c[c].alpha;
     beta[c] = st->c[c].beta;
   }
   for (int64_t g = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; g < n; g += int64_t(gridDim.x) * blockDim.x) {
-    if (__ldg(off + g) < 0) continue;
+    if (__ldg(head + g) == kHeadDirichlet) continue;
     const double di = dinv[g];
 #pragma unroll
     for (int c = 0; c < NC; ++c) {
-      if (!act[c]) continue;
+      if (!xs[c]) continue;
       const size_t i = size_t(g) * NC + c;
-      p[i] = di * r[i] + beta[c] * p[i];
+      const double pv = p[i];
+      x[i] += alpha[c] * pv;
+      if (act[c]) p[i] = di * r[i] + beta[c] * pv;
     }
   }
 }
@@ -185,23 +181,23 @@ cudaError_t launch_pcg_init(const DeviceMesh& m, const double* b, const double* 
   return cudaGetLastError();
 }
 
-cudaError_t launch_pcg_update(const DeviceMesh& m, const double* wl, double* x, double* r, const double* p,
-                              const double* dinv, double* partials, SolveState* st, cudaStream_t s) {
-  const int nb = vec_blocks(m.nglobal);
+cudaError_t launch_pcg_update(const DeviceMesh& m, const double* wl, double* r, const double* dinv, double* partials,
+                              SolveState* st, int step, cudaStream_t s) {
+  const int nb = gather_blocks(m.nglobal);
   if (m.ncomp == 3)
-    pcg_update_kernel<3><<<nb, 256, 0, s>>>(m.off, m.slots, wl, x, r, p, dinv, m.nglobal, partials, st);
+    pcg_update_kernel<3><<<nb, 256, 0, s>>>(m.head, m.slots, wl, r, dinv, m.nglobal, partials, st, step);
   else
-    pcg_update_kernel<1><<<nb, 256, 0, s>>>(m.off, m.slots, wl, x, r, p, dinv, m.nglobal, partials, st);
+    pcg_update_kernel<1><<<nb, 256, 0, s>>>(m.head, m.slots, wl, r, dinv, m.nglobal, partials, st, step);
   return cudaGetLastError();
 }
 
 cudaError_t launch_pcg_dir(const DeviceMesh& m, const double* r, double* p, const double* dinv,
-                           const SolveState* st, cudaStream_t s) {
+                           const SolveState* st, int step, cudaStream_t s) {
   const int nb = vec_blocks(m.nglobal);
   if (m.ncomp == 3)
-    pcg_dir_kernel<3><<<nb, 256, 0, s>>>(m.off, r, p, dinv, m.nglobal, st);
+    pcg_dir_kernel<3><<<nb, 256, 0, s>>>(m.head, r, p, dinv, m.nglobal, st, step);
   else
-    pcg_dir_kernel<1><<<nb, 256, 0, s>>>(m.off, r, p, dinv, m.nglobal, st);
+    pcg_dir_kernel<1><<<nb, 256, 0, s>>>(m.head, r, p, dinv, m.nglobal, st, step);
   return cudaGetLastError();
 }
 

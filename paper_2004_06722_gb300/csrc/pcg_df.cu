@@ -6,8 +6,7 @@
 // Per-thread sums are accumulated as pairs and handed to the FP64 block and
 // grid reductions of common.cuh, so alpha and beta are formed in FP64 exactly
 // as in the FP64 kernels (pcg.cu).
-#include "common.cuh"
-#include "df.cuh"
+#include "gather.cuh"
 #include "internal.h"
 
 namespace ceedbp {
@@ -21,7 +20,7 @@ __global__ void init_df_kernel(const int* __restrict__ off, const double* __rest
                                const double* __restrict__ ax, double* __restrict__ x, dfloat* __restrict__ xd,
                                dfloat* __restrict__ r, dfloat* __restrict__ p, const dfloat* __restrict__ dinv,
                                int64_t n, int x0, double* partials, SolveState* st, double tol, int fixed) {
-  __shared__ double red[32 * 3 * NC];
+  __shared__ double red[256 * 3 * NC];
   double acc[3 * NC];
 #pragma unroll
   for (int k = 0; k < 3 * NC; ++k) acc[k] = 0.0;
@@ -44,11 +43,12 @@ __global__ void init_df_kernel(const int* __restrict__ off, const double* __rest
       acc[2 * NC + c] += bv * bv;
     }
   }
-  if (grid_sum_last<3 * NC>(acc, partials, gridDim.x, blockIdx.x, &st->ticket[kTicketInit], red)) {
+  if (grid_sum_last_256<3 * NC>(acc, partials, &st->ticket[kTicketInit], red)) {
     if (threadIdx.x == 0) {
       int any = 0;
       st->ncomp = NC;
       st->fixed = fixed;
+      st->step = -1;
 #pragma unroll
       for (int c = 0; c < NC; ++c) {
         CompScalars& cs = st->c[c];
@@ -70,12 +70,15 @@ __global__ void init_df_kernel(const int* __restrict__ off, const double* __rest
 }
 
 template <int NC>
-__global__ void update_df_kernel(const int* __restrict__ off, const int* __restrict__ slots,
-                                 const dfloat* __restrict__ wl, dfloat* __restrict__ x, dfloat* __restrict__ r,
-                                 const dfloat* __restrict__ p, const dfloat* __restrict__ dinv, int64_t n,
-                                 double* partials, SolveState* st) {
-  __shared__ double red[32 * 2 * NC];
-  if (st->stop) return;
+__global__ void __launch_bounds__(256) update_df_kernel(const int* __restrict__ head, const int* __restrict__ slots,
+                                                        const dfloat* __restrict__ wl, dfloat* __restrict__ r,
+                                                        const dfloat* __restrict__ dinv, int64_t n,
+                                                        double* partials, SolveState* st, int step) {
+  __shared__ double red[256 * 2 * NC];
+  if (st->stop) {
+    if (blockIdx.x == 0 && threadIdx.x == 0) st->step = -1;  // nothing for this iteration's direction kernel
+    return;
+  }
   dfloat alpha[NC];
   bool act[NC];
 #pragma unroll
@@ -86,53 +89,29 @@ __global__ void update_df_kernel(const int* __restrict__ off, const int* __restr
   dfloat rz[NC], rr[NC];
 #pragma unroll
   for (int c = 0; c < NC; ++c) rz[c] = rr[c] = dfloat{0.0f, 0.0f};
-  for (int64_t g = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; g < n; g += int64_t(gridDim.x) * blockDim.x) {
-    const int o0 = __ldg(off + g);
-    if (o0 < 0) continue;
-    const int o1 = __ldg(off + g + 1) & 0x7fffffff;
-    // start from the first slot (the local values are normalised pairs, so this equals adding
-    // them to zero); a node no element touches sums to 0
-    dfloat w[NC];
+  const int64_t stride = int64_t(gridDim.x) * 256;
+  for (int64_t g0 = int64_t(blockIdx.x) * 256 + threadIdx.x; g0 < n; g0 += 2 * stride) {
+    int hd[2];
+    dfloat w[2][NC], rv[2][NC], di[2];
 #pragma unroll
-    for (int c = 0; c < NC; ++c) w[c] = dfloat{0.0f, 0.0f};
-    if (o0 < o1) {
-      const int sl = __ldg(slots + o0);
+    for (int h = 0; h < 2; ++h) {
+      const int64_t g = g0 + h * stride < n ? g0 + h * stride : g0;
+      di[h] = dinv[g];
+#pragma unroll
+      for (int c = 0; c < NC; ++c) rv[h][c] = r[size_t(g) * NC + c];
+    }
+    gather_nodes<2, NC>(head, slots, wl, g0, stride, n, hd, w);
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      if (hd[h] == kHeadDirichlet) continue;
 #pragma unroll
       for (int c = 0; c < NC; ++c) {
-        const float2 v = __ldcs(reinterpret_cast<const float2*>(wl + size_t(sl) * NC + c));
-        w[c] = dfloat{v.x, v.y};
+        if (!act[c]) continue;
+        const dfloat v = dw_add(rv[h][c], dw_neg(dw_mul(alpha[c], w[h][c])));
+        r[size_t(g0 + h * stride) * NC + c] = v;
+        rz[c] = dw_add(rz[c], dw_mul(v, dw_mul(di[h], v)));
+        rr[c] = dw_add(rr[c], dw_mul(v, v));
       }
-    }
-    // the remaining slots two at a time (loads issued together, sums in slot order)
-    int k = o0 + 1;
-    for (; k + 1 < o1; k += 2) {
-      const int s0 = __ldg(slots + k), s1 = __ldg(slots + k + 1);
-#pragma unroll
-      for (int c = 0; c < NC; ++c) {
-        const float2 v0 = __ldcs(reinterpret_cast<const float2*>(wl + size_t(s0) * NC + c));
-        const float2 v1 = __ldcs(reinterpret_cast<const float2*>(wl + size_t(s1) * NC + c));
-        w[c] = dw_add(w[c], dfloat{v0.x, v0.y});
-        w[c] = dw_add(w[c], dfloat{v1.x, v1.y});
-      }
-    }
-    if (k < o1) {
-      const int s0 = __ldg(slots + k);
-#pragma unroll
-      for (int c = 0; c < NC; ++c) {
-        const float2 v = __ldcs(reinterpret_cast<const float2*>(wl + size_t(s0) * NC + c));
-        w[c] = dw_add(w[c], dfloat{v.x, v.y});
-      }
-    }
-    const dfloat di = dinv[g];
-#pragma unroll
-    for (int c = 0; c < NC; ++c) {
-      if (!act[c]) continue;
-      const size_t i = size_t(g) * NC + c;
-      const dfloat rv = dw_add(r[i], dw_neg(dw_mul(alpha[c], w[c])));
-      x[i] = dw_add(x[i], dw_mul(alpha[c], p[i]));
-      r[i] = rv;
-      rz[c] = dw_add(rz[c], dw_mul(rv, dw_mul(di, rv)));
-      rr[c] = dw_add(rr[c], dw_mul(rv, rv));
     }
   }
   double acc[2 * NC];
@@ -141,12 +120,14 @@ __global__ void update_df_kernel(const int* __restrict__ off, const int* __restr
     acc[c] = df_to_f64(rz[c]);
     acc[NC + c] = df_to_f64(rr[c]);
   }
-  if (grid_sum_last<2 * NC>(acc, partials, gridDim.x, blockIdx.x, &st->ticket[kTicketUpdate], red)) {
+  if (grid_sum_last_256<2 * NC>(acc, partials, &st->ticket[kTicketUpdate], red)) {
     if (threadIdx.x == 0) {
       int any = 0;
+      st->step = step;
 #pragma unroll
       for (int c = 0; c < NC; ++c) {
         CompScalars& cs = st->c[c];
+        cs.xstep = cs.active;
         if (!cs.active) continue;
         const double rz_new = acc[c];
         cs.beta = cs.rz != 0.0 ? rz_new / cs.rz : 0.0;
@@ -166,24 +147,29 @@ __global__ void update_df_kernel(const int* __restrict__ off, const int* __restr
 }
 
 template <int NC>
-__global__ void dir_df_kernel(const int* __restrict__ off, const dfloat* __restrict__ r, dfloat* __restrict__ p,
-                              const dfloat* __restrict__ dinv, int64_t n, const SolveState* st) {
-  if (st->stop) return;
-  dfloat beta[NC];
-  bool act[NC];
+__global__ void dir_df_kernel(const int* __restrict__ head, const dfloat* __restrict__ r, dfloat* __restrict__ p,
+                              dfloat* __restrict__ x, const dfloat* __restrict__ dinv, int64_t n, const SolveState* st,
+                              int step) {
+  if (st->step != step) return;  // no update ran in this iteration (the solve had stopped)
+  dfloat alpha[NC], beta[NC];
+  bool xs[NC], act[NC];
 #pragma unroll
   for (int c = 0; c < NC; ++c) {
+    xs[c] = st->c[c].xstep != 0;
     act[c] = st->c[c].active != 0;
+    alpha[c] = df_from_f64_scalar(st->c[c].alpha);
     beta[c] = df_from_f64_scalar(st->c[c].beta);
   }
   for (int64_t g = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; g < n; g += int64_t(gridDim.x) * blockDim.x) {
-    if (__ldg(off + g) < 0) continue;
+    if (__ldg(head + g) == kHeadDirichlet) continue;
     const dfloat di = dinv[g];
 #pragma unroll
     for (int c = 0; c < NC; ++c) {
-      if (!act[c]) continue;
+      if (!xs[c]) continue;
       const size_t i = size_t(g) * NC + c;
-      p[i] = dw_add(dw_mul(di, r[i]), dw_mul(beta[c], p[i]));
+      const dfloat pv = p[i];
+      x[i] = dw_add(x[i], dw_mul(alpha[c], pv));
+      if (act[c]) p[i] = dw_add(dw_mul(di, r[i]), dw_mul(beta[c], pv));
     }
   }
 }
@@ -198,23 +184,20 @@ __global__ void f64_to_df_kernel(const double* __restrict__ src, dfloat* __restr
     dst[i] = f64_to_df(src[i]);
 }
 
+// mask_out: Dirichlet rows are zero; their values are not read (the element kernels may skip them).
 template <int NC>
-__global__ void gs_df_kernel(const int* __restrict__ off, const int* __restrict__ slots, const dfloat* __restrict__ wl,
-                             double* __restrict__ w, int64_t n, int mask_out) {
-  for (int64_t g = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; g < n; g += int64_t(gridDim.x) * blockDim.x) {
-    const int o0 = __ldg(off + g), o1 = __ldg(off + g + 1) & 0x7fffffff;
-    dfloat s[NC];
+__global__ void __launch_bounds__(256) gs_df_kernel(const int* __restrict__ head, const int* __restrict__ slots,
+                                                    const dfloat* __restrict__ wl, double* __restrict__ w, int64_t n) {
+  const int64_t stride = int64_t(gridDim.x) * 256;
+  for (int64_t g0 = int64_t(blockIdx.x) * 256 + threadIdx.x; g0 < n; g0 += 2 * stride) {
+    int hd[2];
+    dfloat v[2][NC];
+    gather_nodes<2, NC>(head, slots, wl, g0, stride, n, hd, v);
 #pragma unroll
-    for (int c = 0; c < NC; ++c) s[c] = dfloat{0.0f, 0.0f};
-    if (!(o0 < 0 && mask_out)) {
-      for (int k = o0 & 0x7fffffff; k < o1; ++k) {
-        const int sl = __ldg(slots + k);
+    for (int h = 0; h < 2; ++h)
+      if (g0 + h * stride < n)
 #pragma unroll
-        for (int c = 0; c < NC; ++c) s[c] = dw_add(s[c], wl[size_t(sl) * NC + c]);
-      }
-    }
-#pragma unroll
-    for (int c = 0; c < NC; ++c) w[g * NC + c] = df_to_f64(s[c]);
+        for (int c = 0; c < NC; ++c) w[size_t(g0 + h * stride) * NC + c] = df_to_f64(v[h][c]);
   }
 }
 
@@ -231,23 +214,23 @@ cudaError_t launch_init_df(const DeviceMesh& m, const double* b, const double* a
   return cudaGetLastError();
 }
 
-cudaError_t launch_update_df(const DeviceMesh& m, const dfloat* wl, dfloat* x, dfloat* r, const dfloat* p,
-                             const dfloat* dinv, double* partials, SolveState* st, cudaStream_t s) {
-  const int nb = vec_blocks(m.nglobal);
+cudaError_t launch_update_df(const DeviceMesh& m, const dfloat* wl, dfloat* r, const dfloat* dinv, double* partials,
+                             SolveState* st, int step, cudaStream_t s) {
+  const int nb = gather_blocks(m.nglobal);
   if (m.ncomp == 3)
-    update_df_kernel<3><<<nb, 256, 0, s>>>(m.off, m.slots, wl, x, r, p, dinv, m.nglobal, partials, st);
+    update_df_kernel<3><<<nb, 256, 0, s>>>(m.head, m.slots, wl, r, dinv, m.nglobal, partials, st, step);
   else
-    update_df_kernel<1><<<nb, 256, 0, s>>>(m.off, m.slots, wl, x, r, p, dinv, m.nglobal, partials, st);
+    update_df_kernel<1><<<nb, 256, 0, s>>>(m.head, m.slots, wl, r, dinv, m.nglobal, partials, st, step);
   return cudaGetLastError();
 }
 
-cudaError_t launch_dir_df(const DeviceMesh& m, const dfloat* r, dfloat* p, const dfloat* dinv, const SolveState* st,
-                          cudaStream_t s) {
+cudaError_t launch_dir_df(const DeviceMesh& m, const dfloat* r, dfloat* p, dfloat* x, const dfloat* dinv,
+                          const SolveState* st, int step, cudaStream_t s) {
   const int nb = vec_blocks(m.nglobal);
   if (m.ncomp == 3)
-    dir_df_kernel<3><<<nb, 256, 0, s>>>(m.off, r, p, dinv, m.nglobal, st);
+    dir_df_kernel<3><<<nb, 256, 0, s>>>(m.head, r, p, x, dinv, m.nglobal, st, step);
   else
-    dir_df_kernel<1><<<nb, 256, 0, s>>>(m.off, r, p, dinv, m.nglobal, st);
+    dir_df_kernel<1><<<nb, 256, 0, s>>>(m.head, r, p, x, dinv, m.nglobal, st, step);
   return cudaGetLastError();
 }
 
@@ -262,10 +245,11 @@ cudaError_t launch_f64_to_df(const double* src, dfloat* dst, int64_t n, cudaStre
 }
 
 cudaError_t launch_gs_df(const DeviceMesh& m, const dfloat* wl, double* w, int mask_out, cudaStream_t s) {
+  if (!mask_out) return cudaErrorInvalidValue;  // the heads know no values of Dirichlet nodes
   if (m.ncomp == 3)
-    gs_df_kernel<3><<<vec_blocks(m.nglobal), 256, 0, s>>>(m.off, m.slots, wl, w, m.nglobal, mask_out);
+    gs_df_kernel<3><<<gather_blocks(m.nglobal), 256, 0, s>>>(m.head, m.slots, wl, w, m.nglobal);
   else
-    gs_df_kernel<1><<<vec_blocks(m.nglobal), 256, 0, s>>>(m.off, m.slots, wl, w, m.nglobal, mask_out);
+    gs_df_kernel<1><<<gather_blocks(m.nglobal), 256, 0, s>>>(m.head, m.slots, wl, w, m.nglobal);
   return cudaGetLastError();
 }
 

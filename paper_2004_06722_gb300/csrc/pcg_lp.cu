@@ -8,8 +8,7 @@
 // FP64).  The inner vectors x_in and r_in are FP32.
 #include <cuda_bf16.h>
 
-#include "common.cuh"
-#include "df.cuh"
+#include "gather.cuh"
 #include "internal.h"
 
 namespace ceedbp {
@@ -33,7 +32,7 @@ template <int NC>
 __global__ void residual_kernel(const int* __restrict__ off, const double* __restrict__ b,
                                 const double* __restrict__ ax, double* __restrict__ r, int64_t n, double* partials,
                                 unsigned* ticket, double* out) {
-  __shared__ double red[32 * NC];
+  __shared__ double red[256 * NC];
   double acc[NC];
 #pragma unroll
   for (int c = 0; c < NC; ++c) acc[c] = 0.0;
@@ -47,7 +46,7 @@ __global__ void residual_kernel(const int* __restrict__ off, const double* __res
       acc[c] += v * v;
     }
   }
-  if (grid_sum_last<NC>(acc, partials, gridDim.x, blockIdx.x, ticket, red)) {
+  if (grid_sum_last_256<NC>(acc, partials, ticket, red)) {
     if (threadIdx.x == 0)
 #pragma unroll
       for (int c = 0; c < NC; ++c) out[c] = acc[c];
@@ -62,7 +61,7 @@ template <int NC, typename TS>
 __global__ void inner_init_kernel(const int* __restrict__ off, const double* __restrict__ r64, Scale3 scale,
                                   const float* __restrict__ dinv, float* __restrict__ x, float* __restrict__ r,
                                   TS* __restrict__ p, int64_t n, double* partials, SolveState* st, double tol) {
-  __shared__ double red[32 * 2 * NC];
+  __shared__ double red[256 * 2 * NC];
   dfloat rz[NC], rr[NC];
 #pragma unroll
   for (int c = 0; c < NC; ++c) rz[c] = rr[c] = dfloat{0.0f, 0.0f};
@@ -87,11 +86,12 @@ __global__ void inner_init_kernel(const int* __restrict__ off, const double* __r
     acc[c] = df_to_f64(rz[c]);
     acc[NC + c] = df_to_f64(rr[c]);
   }
-  if (grid_sum_last<2 * NC>(acc, partials, gridDim.x, blockIdx.x, &st->ticket[kTicketInit], red)) {
+  if (grid_sum_last_256<2 * NC>(acc, partials, &st->ticket[kTicketInit], red)) {
     if (threadIdx.x == 0) {
       int any = 0;
       st->ncomp = NC;
       st->fixed = 0;
+      st->step = -1;
 #pragma unroll
       for (int c = 0; c < NC; ++c) {
         CompScalars& cs = st->c[c];
@@ -112,13 +112,16 @@ __global__ void inner_init_kernel(const int* __restrict__ off, const double* __r
   }
 }
 
-template <int NC, typename TS>
-__global__ void inner_update_kernel(const int* __restrict__ off, const int* __restrict__ slots,
-                                    const float* __restrict__ wl, float* __restrict__ x, float* __restrict__ r,
-                                    const TS* __restrict__ p, const float* __restrict__ dinv, int64_t n,
-                                    double* partials, SolveState* st) {
-  __shared__ double red[32 * 2 * NC];
-  if (st->stop) return;
+template <int NC>
+__global__ void __launch_bounds__(256) inner_update_kernel(const int* __restrict__ head, const int* __restrict__ slots,
+                                                           const float* __restrict__ wl, float* __restrict__ r,
+                                                           const float* __restrict__ dinv, int64_t n,
+                                                           double* partials, SolveState* st, int step) {
+  __shared__ double red[256 * 2 * NC];
+  if (st->stop) {
+    if (blockIdx.x == 0 && threadIdx.x == 0) st->step = -1;  // nothing for this iteration's direction kernel
+    return;
+  }
   float alpha[NC];
   bool act[NC];
 #pragma unroll
@@ -129,46 +132,28 @@ __global__ void inner_update_kernel(const int* __restrict__ off, const int* __re
   dfloat rz[NC], rr[NC];
 #pragma unroll
   for (int c = 0; c < NC; ++c) rz[c] = rr[c] = dfloat{0.0f, 0.0f};
-  // Two nodes per thread and step, g and g + stride: the offsets, the first local slot and its
-  // values of both nodes are loaded before either is used (most nodes -- element interiors --
-  // have exactly one slot), so two dependent load chains are in flight per thread.
-  const int64_t stride = int64_t(gridDim.x) * blockDim.x;
-  for (int64_t g0 = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; g0 < n; g0 += 2 * stride) {
-    int64_t gs[2] = {g0, g0 + stride};
-    int o0[2], o1[2];
-    float w[2][NC];
+  const int64_t stride = int64_t(gridDim.x) * 256;
+  for (int64_t g0 = int64_t(blockIdx.x) * 256 + threadIdx.x; g0 < n; g0 += 2 * stride) {
+    int hd[2];
+    float w[2][NC], rv[2][NC], di[2];
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
-      const bool in = gs[h] < n;
-      o0[h] = in ? __ldg(off + gs[h]) : -1;
-      o1[h] = in ? (__ldg(off + gs[h] + 1) & 0x7fffffff) : 0;
+      const int64_t g = g0 + h * stride < n ? g0 + h * stride : g0;
+      di[h] = dinv[g];
+#pragma unroll
+      for (int c = 0; c < NC; ++c) rv[h][c] = r[size_t(g) * NC + c];
     }
-    int sl[2];
-#pragma unroll
-    for (int h = 0; h < 2; ++h) sl[h] = (o0[h] >= 0 && o0[h] < o1[h]) ? __ldg(slots + o0[h]) : -1;
-#pragma unroll
-    for (int h = 0; h < 2; ++h)
-#pragma unroll
-      for (int c = 0; c < NC; ++c) w[h][c] = sl[h] >= 0 ? __ldcs(wl + size_t(sl[h]) * NC + c) : 0.0f;
+    gather_nodes<2, NC>(head, slots, wl, g0, stride, n, hd, w);
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
-      if (o0[h] < 0) continue;  // Dirichlet node (or past the end)
-      for (int k = o0[h] + 1; k < o1[h]; ++k) {
-        const int s = __ldg(slots + k);
-#pragma unroll
-        for (int c = 0; c < NC; ++c) w[h][c] += __ldcs(wl + size_t(s) * NC + c);
-      }
-      const int64_t g = gs[h];
-      const float di = dinv[g];
+      if (hd[h] == kHeadDirichlet) continue;
 #pragma unroll
       for (int c = 0; c < NC; ++c) {
         if (!act[c]) continue;
-        const size_t i = size_t(g) * NC + c;
-        const float rv = fmaf(-alpha[c], w[h][c], r[i]);
-        x[i] = fmaf(alpha[c], lp_get(p + i), x[i]);
-        r[i] = rv;
-        acc_prod(rz[c], rv, di * rv);
-        acc_prod(rr[c], rv, rv);
+        const float v = fmaf(-alpha[c], w[h][c], rv[h][c]);
+        r[size_t(g0 + h * stride) * NC + c] = v;
+        acc_prod(rz[c], v, di[h] * v);
+        acc_prod(rr[c], v, v);
       }
     }
   }
@@ -178,12 +163,14 @@ __global__ void inner_update_kernel(const int* __restrict__ off, const int* __re
     acc[c] = df_to_f64(rz[c]);
     acc[NC + c] = df_to_f64(rr[c]);
   }
-  if (grid_sum_last<2 * NC>(acc, partials, gridDim.x, blockIdx.x, &st->ticket[kTicketUpdate], red)) {
+  if (grid_sum_last_256<2 * NC>(acc, partials, &st->ticket[kTicketUpdate], red)) {
     if (threadIdx.x == 0) {
       int any = 0;
+      st->step = step;
 #pragma unroll
       for (int c = 0; c < NC; ++c) {
         CompScalars& cs = st->c[c];
+        cs.xstep = cs.active;
         if (!cs.active) continue;
         const double rz_new = acc[c];
         cs.beta = cs.rz != 0.0 ? rz_new / cs.rz : 0.0;
@@ -203,24 +190,29 @@ __global__ void inner_update_kernel(const int* __restrict__ off, const int* __re
 }
 
 template <int NC, typename TS>
-__global__ void inner_dir_kernel(const int* __restrict__ off, const float* __restrict__ r, TS* __restrict__ p,
-                                 const float* __restrict__ dinv, int64_t n, const SolveState* st) {
-  if (st->stop) return;
-  float beta[NC];
-  bool act[NC];
+__global__ void inner_dir_kernel(const int* __restrict__ head, const float* __restrict__ r, TS* __restrict__ p,
+                                 float* __restrict__ x, const float* __restrict__ dinv, int64_t n,
+                                 const SolveState* st, int step) {
+  if (st->step != step) return;  // no update ran in this iteration (the solve had stopped)
+  float alpha[NC], beta[NC];
+  bool xs[NC], act[NC];
 #pragma unroll
   for (int c = 0; c < NC; ++c) {
+    xs[c] = st->c[c].xstep != 0;
     act[c] = st->c[c].active != 0;
+    alpha[c] = float(st->c[c].alpha);
     beta[c] = float(st->c[c].beta);
   }
   for (int64_t g = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; g < n; g += int64_t(gridDim.x) * blockDim.x) {
-    if (__ldg(off + g) < 0) continue;
+    if (__ldg(head + g) == kHeadDirichlet) continue;
     const float di = dinv[g];
 #pragma unroll
     for (int c = 0; c < NC; ++c) {
-      if (!act[c]) continue;
+      if (!xs[c]) continue;
       const size_t i = size_t(g) * NC + c;
-      lp_put(p + i, fmaf(beta[c], lp_get(p + i), di * r[i]));
+      const float pv = lp_get(p + i);
+      x[i] = fmaf(alpha[c], pv, x[i]);
+      if (act[c]) lp_put(p + i, fmaf(beta[c], pv, di * r[i]));
     }
   }
 }
@@ -277,43 +269,25 @@ cudaError_t launch_inner_init(const DeviceMesh& m, int bf16, const double* r64, 
   return cudaGetLastError();
 }
 
-cudaError_t launch_inner_update(const DeviceMesh& m, int bf16, const float* wl, float* x, float* r, const void* p,
-                                const float* dinv, double* partials, SolveState* st, cudaStream_t s) {
-  const int nb = vec_blocks(m.nglobal);
-  if (m.ncomp == 3) {
-    if (bf16)
-      inner_update_kernel<3, __nv_bfloat16><<<nb, 256, 0, s>>>(m.off, m.slots, wl, x, r,
-                                                               static_cast<const __nv_bfloat16*>(p), dinv, m.nglobal,
-                                                               partials, st);
-    else
-      inner_update_kernel<3, float><<<nb, 256, 0, s>>>(m.off, m.slots, wl, x, r, static_cast<const float*>(p), dinv,
-                                                       m.nglobal, partials, st);
-  } else {
-    if (bf16)
-      inner_update_kernel<1, __nv_bfloat16><<<nb, 256, 0, s>>>(m.off, m.slots, wl, x, r,
-                                                               static_cast<const __nv_bfloat16*>(p), dinv, m.nglobal,
-                                                               partials, st);
-    else
-      inner_update_kernel<1, float><<<nb, 256, 0, s>>>(m.off, m.slots, wl, x, r, static_cast<const float*>(p), dinv,
-                                                       m.nglobal, partials, st);
-  }
+cudaError_t launch_inner_update(const DeviceMesh& m, const float* wl, float* r, const float* dinv, double* partials,
+                                SolveState* st, int step, cudaStream_t s) {
+  const int nb = gather_blocks(m.nglobal);
+  if (m.ncomp == 3)
+    inner_update_kernel<3><<<nb, 256, 0, s>>>(m.head, m.slots, wl, r, dinv, m.nglobal, partials, st, step);
+  else
+    inner_update_kernel<1><<<nb, 256, 0, s>>>(m.head, m.slots, wl, r, dinv, m.nglobal, partials, st, step);
   return cudaGetLastError();
 }
 
-cudaError_t launch_inner_dir(const DeviceMesh& m, int bf16, const float* r, void* p, const float* dinv,
-                             const SolveState* st, cudaStream_t s) {
+cudaError_t launch_inner_dir(const DeviceMesh& m, int bf16, const float* r, void* p, float* x, const float* dinv,
+                             const SolveState* st, int step, cudaStream_t s) {
   const int nb = vec_blocks(m.nglobal);
-  if (m.ncomp == 3) {
-    if (bf16)
-      inner_dir_kernel<3, __nv_bfloat16><<<nb, 256, 0, s>>>(m.off, r, static_cast<__nv_bfloat16*>(p), dinv, m.nglobal, st);
-    else
-      inner_dir_kernel<3, float><<<nb, 256, 0, s>>>(m.off, r, static_cast<float*>(p), dinv, m.nglobal, st);
-  } else {
-    if (bf16)
-      inner_dir_kernel<1, __nv_bfloat16><<<nb, 256, 0, s>>>(m.off, r, static_cast<__nv_bfloat16*>(p), dinv, m.nglobal, st);
-    else
-      inner_dir_kernel<1, float><<<nb, 256, 0, s>>>(m.off, r, static_cast<float*>(p), dinv, m.nglobal, st);
-  }
+  auto go = [&](auto* pt) {
+    if (m.ncomp == 3) inner_dir_kernel<3><<<nb, 256, 0, s>>>(m.head, r, pt, x, dinv, m.nglobal, st, step);
+    else inner_dir_kernel<1><<<nb, 256, 0, s>>>(m.head, r, pt, x, dinv, m.nglobal, st, step);
+  };
+  if (bf16) go(static_cast<__nv_bfloat16*>(p));
+  else go(static_cast<float*>(p));
   return cudaGetLastError();
 }
 

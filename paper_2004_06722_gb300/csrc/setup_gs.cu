@@ -12,7 +12,7 @@
 // of w_L[s] -- the action of Q^T in Eq. (21) in a fixed summation order, with
 // no floating-point atomics.  Bit 31 of off[g] flags a Dirichlet node, whose
 // output is zero when masking (the restriction of Algorithm 1).
-#include "common.cuh"
+#include "gather.cuh"
 
 namespace ceedbp {
 
@@ -170,24 +170,47 @@ __global__ void local_diag_kernel(const DeviceMesh m, int kind, const double* __
     for (int k = 0; k < P1; ++k) wl[e * P3 + k * P1 * P1 + ty * P1 + tx] = acc[k];
 }
 
+// every node, Dirichlet rows included (setup, mass operators)
 template <int NC>
-__global__ void gs_kernel(const int* __restrict__ off, const int* __restrict__ slots, const double* __restrict__ wl,
-                          double* __restrict__ w, int64_t n, int mask_out) {
+__global__ void gs_all_kernel(const int* __restrict__ off, const int* __restrict__ slots, const double* __restrict__ wl,
+                              double* __restrict__ w, int64_t n) {
   for (int64_t g = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; g < n; g += int64_t(gridDim.x) * blockDim.x) {
     const int o0 = __ldg(off + g), o1 = __ldg(off + g + 1) & 0x7fffffff;
-    const bool dir = o0 < 0;
     double s[NC];
 #pragma unroll
     for (int c = 0; c < NC; ++c) s[c] = 0.0;
-    if (!(dir && mask_out)) {
-      for (int k = o0 & 0x7fffffff; k < o1; ++k) {
-        const int sl = __ldg(slots + k);
+    for (int k = o0 & 0x7fffffff; k < o1; ++k) {
+      const int sl = __ldg(slots + k) & kSlotMask;
 #pragma unroll
-        for (int c = 0; c < NC; ++c) s[c] += __ldg(wl + size_t(sl) * NC + c);
-      }
+      for (int c = 0; c < NC; ++c) s[c] += __ldg(wl + size_t(sl) * NC + c);
     }
 #pragma unroll
     for (int c = 0; c < NC; ++c) w[g * NC + c] = s[c];
+  }
+}
+
+// Dirichlet rows zero; their values are not read (the element kernels may skip them)
+template <int NC>
+__global__ void __launch_bounds__(256) gs_kernel(const int* __restrict__ head, const int* __restrict__ slots,
+                                                 const double* __restrict__ wl, double* __restrict__ w, int64_t n) {
+  const int64_t stride = int64_t(gridDim.x) * 256;
+  for (int64_t g0 = int64_t(blockIdx.x) * 256 + threadIdx.x; g0 < n; g0 += 2 * stride) {
+    int hd[2];
+    double v[2][NC];
+    gather_nodes<2, NC>(head, slots, wl, g0, stride, n, hd, v);
+#pragma unroll
+    for (int h = 0; h < 2; ++h)
+      if (g0 + h * stride < n)
+#pragma unroll
+        for (int c = 0; c < NC; ++c) w[size_t(g0 + h * stride) * NC + c] = v[h][c];
+  }
+}
+
+__global__ void heads_kernel(const int* __restrict__ off, int* __restrict__ slots, int* __restrict__ head, int64_t n) {
+  for (int64_t g = int64_t(blockIdx.x) * blockDim.x + threadIdx.x; g < n; g += int64_t(gridDim.x) * blockDim.x) {
+    const int raw = off[g], o0 = raw & 0x7fffffff, o1 = off[g + 1] & 0x7fffffff;
+    head[g] = raw < 0 ? kHeadDirichlet : o1 == o0 ? kHeadEmpty : o1 == o0 + 1 ? slots[o0] : -o0 - 2;
+    if (o1 > o0) slots[o1 - 1] |= ~kSlotMask;
   }
 }
 
@@ -263,10 +286,20 @@ int vec_blocks(int64_t n) {
 }
 
 cudaError_t launch_gs(const DeviceMesh& m, const double* wl, double* w, int mask_out, cudaStream_t s) {
-  if (m.ncomp == 3)
-    gs_kernel<3><<<vec_blocks(m.nglobal), 256, 0, s>>>(m.off, m.slots, wl, w, m.nglobal, mask_out);
-  else
-    gs_kernel<1><<<vec_blocks(m.nglobal), 256, 0, s>>>(m.off, m.slots, wl, w, m.nglobal, mask_out);
+  if (mask_out) {
+    const int nb = gather_blocks(m.nglobal);
+    if (m.ncomp == 3) gs_kernel<3><<<nb, 256, 0, s>>>(m.head, m.slots, wl, w, m.nglobal);
+    else gs_kernel<1><<<nb, 256, 0, s>>>(m.head, m.slots, wl, w, m.nglobal);
+  } else {
+    const int nb = vec_blocks(m.nglobal);
+    if (m.ncomp == 3) gs_all_kernel<3><<<nb, 256, 0, s>>>(m.off, m.slots, wl, w, m.nglobal);
+    else gs_all_kernel<1><<<nb, 256, 0, s>>>(m.off, m.slots, wl, w, m.nglobal);
+  }
+  return cudaGetLastError();
+}
+
+cudaError_t launch_heads(const int* off, int* slots, int* head, int64_t n, cudaStream_t s) {
+  heads_kernel<<<vec_blocks(n), 256, 0, s>>>(off, slots, head, n);
   return cudaGetLastError();
 }
 
