@@ -178,10 +178,9 @@ __global__ void __launch_bounds__(FxCoShape<P1>::NT, FxCoShape<P1>::MINB)
     dnext = 0;
 #pragma unroll
     for (int k = 0; k < P1; ++k) {
-      const int gg = g[k] >= 0 ? g[k] : -g[k] - 1;
+      const int gg = g[k] ^ (g[k] >> 31);  // -(g + 1) for Dirichlet nodes
       dnext |= unsigned(g[k] < 0) << k;
-      if (g[k] < 0 && a.mask_in) dst[k * PP] = 0.0;
-      else cp_async8(dst + k * PP, src + size_t(gg) * NC);
+      cp_async8_or_zero(dst + k * PP, src + size_t(gg) * NC, g[k] < 0 && a.mask_in);
     }
   };
   auto prefetch_G = [&](int64_t e) {

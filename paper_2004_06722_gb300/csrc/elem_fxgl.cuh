@@ -232,13 +232,15 @@ __global__ void __launch_bounds__(FxGlShape<P1, KIND>::NT, FxGlShape<P1, KIND>::
   const bool lead = live && (tid & 31) == __ffs(int(lanes)) - 1;
   auto place = [](int idx) { return idx / (P1 * P1) * PS + idx / P1 % P1 * S + idx % P1; };  // of a node in a tile
 
+  // whether the thread has an n-th node (known to the compiler for all but the last)
+  auto has = [&](int n) { return (n + 1) * QQ <= P3 || t + n * QQ < P3; };
   int g[NPT];
   unsigned dnext = 0, dcur = 0;  // Dirichlet bits of the thread's nodes
   auto load_l2g = [&](int it) {
     const int* l2g = m.l2g + elem_of(it) * P3;
 #pragma unroll
     for (int n = 0; n < NPT; ++n)
-      if (t + n * QQ < P3) g[n] = __ldg(l2g + t + n * QQ);
+      if (has(n)) g[n] = __ldg(l2g + t + n * QQ);
   };
   auto fetch_u = [&](int it) {
     double* dst = ubuf + (it % Sh::NU) * P3;
@@ -246,12 +248,10 @@ __global__ void __launch_bounds__(FxGlShape<P1, KIND>::NT, FxGlShape<P1, KIND>::
     dnext = 0;
 #pragma unroll
     for (int n = 0; n < NPT; ++n) {
-      const int idx = t + n * QQ;
-      if (idx >= P3) continue;
-      const int gg = g[n] >= 0 ? g[n] : -g[n] - 1;
+      if (!has(n)) continue;
+      const int gg = g[n] ^ (g[n] >> 31);  // -(g + 1) for Dirichlet nodes
       dnext |= unsigned(g[n] < 0) << n;
-      if (g[n] < 0 && a.mask_in) dst[idx] = 0.0;
-      else cp_async8(dst + idx, src + size_t(gg) * NC);
+      cp_async8_or_zero(dst + t + n * QQ, src + size_t(gg) * NC, g[n] < 0 && a.mask_in);
     }
   };
   auto prefetch_factors = [&](int64_t e) {
@@ -282,7 +282,7 @@ __global__ void __launch_bounds__(FxGlShape<P1, KIND>::NT, FxGlShape<P1, KIND>::
     if (live) {
 #pragma unroll
       for (int n = 0; n < NPT; ++n)
-        if (t + n * QQ < P3) mx = max(mx, unsigned(__double2hiint(su[t + n * QQ])) & 0x7fffffffu);
+        if (has(n)) mx = max(mx, unsigned(__double2hiint(su[t + n * QQ])) & 0x7fffffffu);
       if (it + 1 < nit) load_l2g(it + 1);
     }
     mx = __reduce_max_sync(lanes, mx);
@@ -303,7 +303,7 @@ __global__ void __launch_bounds__(FxGlShape<P1, KIND>::NT, FxGlShape<P1, KIND>::
     if (live && !HELM) {
 #pragma unroll
       for (int n = 0; n < NPT; ++n)
-        if (t + n * QQ < P3) reinterpret_cast<int2*>(tiles)[place(t + n * QQ)] = fx_from_double(su[t + n * QQ], eb);
+        if (has(n)) reinterpret_cast<int2*>(tiles)[place(t + n * QQ)] = fx_from_double(su[t + n * QQ], eb);
     }
     const bool f64 = __syncthreads_or(bad);
     if (!HELM && !f64) {
@@ -343,7 +343,7 @@ __global__ void __launch_bounds__(FxGlShape<P1, KIND>::NT, FxGlShape<P1, KIND>::
       if (live) {
 #pragma unroll
         for (int n = 0; n < NPT; ++n)
-          if (t + n * QQ < P3) tiles[place(t + n * QQ)] = su[t + n * QQ];
+          if (has(n)) tiles[place(t + n * QQ)] = su[t + n * QQ];
       }
       __syncthreads();
       auto done = [](int) {};
@@ -374,8 +374,8 @@ __global__ void __launch_bounds__(FxGlShape<P1, KIND>::NT, FxGlShape<P1, KIND>::
       double acc = 0.0;
 #pragma unroll
       for (int n = 0; n < NPT; ++n) {
+        if (!has(n)) continue;
         const int idx = t + n * QQ;
-        if (idx >= P3) continue;
         const double w = tiles[place(idx)];
         if (!(a.skip_dirichlet_out && ((dcur >> n) & 1u))) wl[size_t(idx) * NC] = w;
         acc += w * su[idx];

@@ -14,6 +14,8 @@
 // go through a private tile.
 #pragma once
 
+#include <algorithm>
+
 #include "elem_lp.cuh"
 
 namespace ceedbp {
@@ -252,11 +254,12 @@ __global__ void __launch_bounds__(256) elem_lpp_kernel(const DeviceMesh m, const
   }
 }
 
-// The shape: two slots per block (one where two do not fit), sequences of 8 elements.
+// The shape: two slots per block (one where two do not fit); sequences of up to 8 elements, as long as one
+// wave of resident blocks covers the mesh (always 8 left 44 of 152 SMs without a block at 12^3 elements).
 template <int P1, int NC>
 struct ElemLppPlan {
   int eb = 0;  // 0: not launchable, use elem_lp_kernel
-  int ns = 8;
+  int resident = 0;  // blocks on the GPU at once
 };
 
 template <int P1, int NC>
@@ -277,7 +280,12 @@ inline ElemLppPlan<P1, NC> elem_lpp_plan() {
               cudaSuccess ||
           nb < 1)
         continue;
+      int dev = 0, sms = 0;
+      if (cudaGetDevice(&dev) != cudaSuccess ||
+          cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+        return p;
       p.eb = eb;
+      p.resident = nb * sms;
       break;
     }
     return p;
@@ -291,9 +299,11 @@ cudaError_t launch_elem_lpp_t(const DeviceMesh& m, const ElemLpArgs& a, cudaStre
   if (p.eb == 0) return launch_elem_lp_t<P1, NC, float>(m, a, s);
   const int nthreads = ((p.eb * P1 * P1 + 31) / 32) * 32;
   const size_t smem = elem_lpp_smem_bytes<P1, NC>(p.eb);
-  const int64_t per_block = int64_t(p.eb) * p.ns;
+  const int64_t full = (m.nelem + p.eb - 1) / p.eb;
+  const int ns = int(std::min<int64_t>(8, (full + p.resident - 1) / p.resident));
+  const int64_t per_block = int64_t(p.eb) * ns;
   const int64_t blocks = (m.nelem + per_block - 1) / per_block;
-  elem_lpp_kernel<P1, NC><<<unsigned(blocks), nthreads, smem, s>>>(m, a, p.eb, p.ns);
+  elem_lpp_kernel<P1, NC><<<unsigned(blocks), nthreads, smem, s>>>(m, a, p.eb, ns);
   return cudaGetLastError();
 }
 

@@ -206,6 +206,12 @@ struct F64Arith {
   __device__ __forceinline__ void take(const FxNorm&, int) {}
 };
 
+// asynchronous copy of one double, or of zero
+__device__ __forceinline__ void cp_async8_or_zero(void* dst, const void* src, bool zero) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;" ::"r"(unsigned(__cvta_generic_to_shared(dst))), "l"(src),
+               "r"(zero ? 0 : 8)
+               : "memory");
+}
 __device__ __forceinline__ void l2_prefetch(const void* p) { asm volatile("prefetch.global.L2 [%0];" ::"l"(p)); }
 
 // Host: blocks of a kernel resident on the GPU (0: it does not fit), and the attribute that lets it use its
