@@ -96,15 +96,16 @@ void release(ceedbp_ctx* c) {
 }
 
 // Fixed-point copies of the stiffness factors and, with Gauss quadrature, the mass factors for the FP64
-// element kernels (elem_fx.cuh, elem_fxgl.cuh): as large as the factors themselves, so they are kept
-// only while they take at most a quarter of the free memory; without them the kernels run in FP64.
+// element kernels (elem_fx.cuh, elem_fxgl.cuh) and the pair arithmetic of BP1/BP3: as large as the factors
+// themselves, so with FP64 arithmetic they are kept only while they take at most a quarter of the free
+// memory; without them the kernels run in FP64.
 ceedbp_status prepare_fx(ceedbp_ctx* c) {
   DeviceMesh& m = c->mesh;
   const size_t nq = size_t(m.nelem) * c->q * c->q * c->q;
   const bool stiff = c->op_kind == kStiff, mass = !c->colloc;
   size_t free_b = 0, total_b = 0;
   CK(c, cudaMemGetInfo(&free_b, &total_b));
-  if (nq * (stiff * 3 * sizeof(int4) + mass * sizeof(int2)) > free_b / 4) return CEEDBP_OK;
+  if (c->arith == CEEDBP_ARITH_FP64 && nq * (stiff * 3 * sizeof(int4) + mass * sizeof(int2)) > free_b / 4) return CEEDBP_OK;
   cudaError_t e = cudaSuccess;
   if (stiff) e = dalloc(&c->d_Gfx, 3 * nq);
   if (stiff && e == cudaSuccess) e = dalloc(&c->d_gexp, size_t(m.nelem));
@@ -236,7 +237,6 @@ ceedbp_status setup_impl(ceedbp_ctx* c, const double* coords, const int64_t* l2g
 
   int nb_apply = elem_blocks(m);
   if (c->colloc) nb_apply = std::max(nb_apply, std::max(int(P.nelem), elem_lp_blocks(m)));
-  else if (P.arith == CEEDBP_ARITH_DF64) nb_apply = std::max(nb_apply, elem_dfgl_blocks(m));
   CK(c, dalloc(&c->d_part_apply, size_t(nb_apply) * nc));
   CK(c, dalloc(&c->d_part_vec, size_t(vec_blocks(n)) * 3 * nc));
 
@@ -271,7 +271,7 @@ ceedbp_status setup_impl(ceedbp_ctx* c, const double* coords, const int64_t* l2g
     if (d_kappa) cudaFree(d_kappa);
     if (e != cudaSuccess) return cuda_fail(c, e, "geometric factors");
   }
-  if (c->arith == CEEDBP_ARITH_FP64 && !recompute && !c->batch_group) {
+  if ((c->arith == CEEDBP_ARITH_FP64 || !c->colloc) && !recompute && !c->batch_group) {
     const ceedbp_status st = prepare_fx(c);
     if (st != CEEDBP_OK) return st;
   }
@@ -320,25 +320,13 @@ ceedbp_status setup_impl(ceedbp_ctx* c, const double* coords, const int64_t* l2g
     }
   }
   if (c->arith == CEEDBP_ARITH_DF64 && !c->colloc) {
-    // BP1 / BP3: pair copies of the factors (G, or the mass factors), of J and Dq, and of dinv;
-    // the kernel sets its splitters from its own line data and the tables' row sums
-    const size_t ng = c->op_kind == kStiff ? size_t(P.nelem) * 6 * Q3 : size_t(P.nelem) * Q3;
-    CK(c, dalloc(&c->d_Gdf, ng));
-    CK(c, dalloc(&c->d_Ddf, size_t(qdef) * p1 + size_t(qdef) * qdef));
+    // BP1 / BP3: the fixed-point kernel with pairs in and out; a pair copy of dinv for the vector kernels
     CK(c, dalloc(&c->d_dinvdf, n));
-    CK(c, launch_f64_to_df(c->op_kind == kStiff ? c->d_G : c->d_Mq, c->d_Gdf, int64_t(ng), s));
     CK(c, launch_f64_to_df(c->d_dinv, c->d_dinvdf, n, s));
-    std::vector<dfloat> hd(size_t(qdef) * p1 + size_t(qdef) * qdef);
-    auto to_pair = [](double d) { const float hi = float(d); return dfloat{hi, float(d - double(hi))}; };
-    for (size_t i = 0; i < basis.J.size(); ++i) hd[i] = to_pair(basis.J[i]);
-    for (size_t i = 0; i < basis.Dq.size(); ++i) hd[basis.J.size() + i] = to_pair(basis.Dq[i]);
-    CK(c, cudaMemcpyAsync(c->d_Ddf, hd.data(), sizeof(dfloat) * hd.size(), cudaMemcpyHostToDevice, s));
-    CK(c, cudaStreamSynchronize(s));
     ElemDfArgs a = {};
     a.u_f64 = c->d_r;
     a.wl = reinterpret_cast<dfloat*>(c->d_wl);
-    a.G = c->d_Gdf;
-    a.D = c->d_Ddf;
+    a.G64 = c->op_kind == kStiff ? c->d_G : c->d_Mq;
     a.mask_in = 1;
     a.fault = &c->d_state->fault;
     CK(c, launch_elem_df(m, a, s));  // one launch outside any capture (attribute setup)
@@ -476,6 +464,7 @@ ElemDfArgs df_args(ceedbp_ctx* c) {
   a.fault = &c->d_state->fault;
   a.first_wait = c->wait_polls;
   a.G = c->d_Gdf;
+  a.G64 = c->op_kind == kStiff ? c->d_G : c->d_Mq;
   a.D = c->d_Ddf;
   a.dnorm_row = c->dnorm_row;
   a.dnorm_col = c->dnorm_col;
@@ -922,10 +911,8 @@ ceedbp_status ceedbp_set_kappa(ceedbp_ctx* c, const double* kappa) {
   m1.ncomp = 1;
   CK(c, launch_gs(m1, c->d_wl, c->d_r, 0, s));
   CK(c, launch_dinv(c->d_off, c->d_r, c->d_dinv, c->prm.nglobal, s));
-  if (c->d_Gdf) {
-    CK(c, launch_f64_to_df(c->d_G, c->d_Gdf, int64_t(ng), s));
-    CK(c, launch_f64_to_df(c->d_dinv, c->d_dinvdf, c->prm.nglobal, s));
-  }
+  if (c->d_Gdf) CK(c, launch_f64_to_df(c->d_G, c->d_Gdf, int64_t(ng), s));
+  if (c->d_dinvdf) CK(c, launch_f64_to_df(c->d_dinv, c->d_dinvdf, c->prm.nglobal, s));
   if (c->d_G32) CK(c, launch_narrow(c->d_G, c->d_G32, int64_t(ng), 0, s));
   if (c->d_Gbf) CK(c, launch_narrow(c->d_G, c->d_Gbf, int64_t(ng), 1, s));
   if (c->d_dinv32) CK(c, launch_narrow(c->d_dinv, c->d_dinv32, c->prm.nglobal, 0, s));

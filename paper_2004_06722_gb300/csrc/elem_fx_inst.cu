@@ -2,6 +2,7 @@
 // BK1..BK4 (elem_fxgl.cuh, instantiated in elem_fxgl_[a-h].cu).
 #include "elem_fx.cuh"
 #include "elem_fxgl.cuh"
+#include "kernel_args.h"
 
 namespace ceedbp {
 
@@ -13,6 +14,7 @@ namespace ceedbp {
   extern template int elem_fx_blocks_t<P, 1>(int64_t);                                          \
   extern template int elem_fx_blocks_t<P, 3>(int64_t); \
   extern template cudaError_t launch_elem_fxgl_t<P>(const DeviceMesh&, int, const ElemArgs&, cudaStream_t); \
+  extern template cudaError_t launch_elem_fxgl_pair_t<P>(const DeviceMesh&, int, const ElemArgs&, cudaStream_t); \
   extern template int elem_fxgl_blocks_any<P>(const DeviceMesh&);
 CEEDBP_FX_P1(X)
 #undef X
@@ -41,6 +43,26 @@ cudaError_t launch_elem_fxgl(const DeviceMesh& m, int kind, const ElemArgs& a, c
   switch (m.p1) {
 #define X(P) \
   case P: return launch_elem_fxgl_t<P>(m, kind, a, s);
+    CEEDBP_FX_P1(X)
+#undef X
+    default: return cudaErrorInvalidValue;
+  }
+}
+
+cudaError_t launch_elem_dfgl(const DeviceMesh& m, const ElemDfArgs& d, cudaStream_t s) {
+  const int kind = m.bp == 1 ? kMass : kStiff;
+  ElemArgs a{};
+  a.u = d.u_f64;
+  a.u_df = d.u_df;
+  a.wl = reinterpret_cast<double*>(d.wl);
+  a.G = d.G64;
+  a.partials = d.partials;
+  a.state = d.state;
+  a.mask_in = d.mask_in;
+  a.skip_dirichlet_out = d.skip_dirichlet_out;
+  switch (m.p1) {
+#define X(P) \
+  case P: return launch_elem_fxgl_pair_t<P>(m, kind, a, s);
     CEEDBP_FX_P1(X)
 #undef X
     default: return cudaErrorInvalidValue;

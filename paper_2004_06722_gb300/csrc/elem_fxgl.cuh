@@ -21,6 +21,10 @@
 // in elem_fx.cuh.  The three directions of Dq^T have a quarter of the range each, so that their sum is
 // in range.
 //
+// The FP32-pair arithmetic of BP1 and BP3 runs this kernel too, with pairs in and out: it is both closer to
+// FP64 and faster than sums of pairs were (BK3, N = 5, 27 x 25 x 23 elements: 261 -> 200 us;
+// BK1, N = 7, 32^3: 782 -> 485 us; one application's error 5 to 100 times smaller).
+//
 // Element sequences, prefetches and the FP64 form of elements off the grid: as in elem_fx.cuh.  With
 // the Helmholtz term (Eq. (17), added at the quadrature points) every element takes the FP64 form.
 #pragma once
@@ -205,7 +209,8 @@ __device__ __forceinline__ void fx_gl_stages(void* tiles, int t, bool live, cons
   __syncthreads();
 }
 
-template <int P1, int NC, int KIND, bool HELM>
+// PAIR: u and w^e are FP32 pairs (df.cuh; u may be FP64 as well), converted in shared memory.
+template <int P1, int NC, int KIND, bool HELM, bool PAIR>
 __global__ void __launch_bounds__(FxGlShape<P1, KIND>::NT, FxGlShape<P1, KIND>::MINB)
     elem_fxgl_kernel(const DeviceMesh m, const ElemArgs a, const __grid_constant__ FxGlTab<P1> tab, const int ns) {
   using Sh = FxGlShape<P1, KIND>;
@@ -244,7 +249,7 @@ __global__ void __launch_bounds__(FxGlShape<P1, KIND>::NT, FxGlShape<P1, KIND>::
   };
   auto fetch_u = [&](int it) {
     double* dst = ubuf + (it % Sh::NU) * P3;
-    const double* src = a.u + (NC == 1 ? 0 : it % NC);
+    const double* src = (PAIR && a.u == nullptr ? reinterpret_cast<const double*>(a.u_df) : a.u) + (NC == 1 ? 0 : it % NC);
     dnext = 0;
 #pragma unroll
     for (int n = 0; n < NPT; ++n) {
@@ -275,9 +280,14 @@ __global__ void __launch_bounds__(FxGlShape<P1, KIND>::NT, FxGlShape<P1, KIND>::
     const int64_t e = elem_of(it);
     const bool store = live && (it / NC) * EB + slot < nblk;
     const int c = NC == 1 ? 0 : it % NC;
-    const double* su = ubuf + (it % Sh::NU) * P3;
+    double* su = ubuf + (it % Sh::NU) * P3;
     cp_async_wait_all();
     dcur = dnext;
+    if (PAIR && a.u == nullptr && live) {
+#pragma unroll
+      for (int n = 0; n < NPT; ++n)
+        if (has(n)) su[t + n * QQ] = df_to_f64(reinterpret_cast<const dfloat*>(su)[t + n * QQ]);
+    }
     unsigned mx = 0;
     if (live) {
 #pragma unroll
@@ -377,7 +387,10 @@ __global__ void __launch_bounds__(FxGlShape<P1, KIND>::NT, FxGlShape<P1, KIND>::
         if (!has(n)) continue;
         const int idx = t + n * QQ;
         const double w = tiles[place(idx)];
-        if (!(a.skip_dirichlet_out && ((dcur >> n) & 1u))) wl[size_t(idx) * NC] = w;
+        if (!(a.skip_dirichlet_out && ((dcur >> n) & 1u))) {
+          if constexpr (PAIR) reinterpret_cast<dfloat*>(wl)[size_t(idx) * NC] = f64_to_df(w);
+          else wl[size_t(idx) * NC] = w;
+        }
         acc += w * su[idx];
       }
 #pragma unroll
@@ -407,17 +420,17 @@ FxGlTab<P1> elem_fxgl_tab(const DeviceMesh& m) {
 
 // Blocks resident on the GPU (0: the kernel does not fit), found once per instantiation; the
 // attribute that lets it use its shared memory is set on the way.
-template <int P1, int NC, int KIND, bool HELM>
+template <int P1, int NC, int KIND, bool HELM, bool PAIR>
 int elem_fxgl_resident() {
   using Sh = FxGlShape<P1, KIND>;
-  static const int n = fx_resident(reinterpret_cast<const void*>(elem_fxgl_kernel<P1, NC, KIND, HELM>), Sh::NT, Sh::SMEM);
+  static const int n = fx_resident(reinterpret_cast<const void*>(elem_fxgl_kernel<P1, NC, KIND, HELM, PAIR>), Sh::NT, Sh::SMEM);
   return n;
 }
 
 // Elements in a slot's sequence: one wave of resident blocks covers the mesh.
 template <int P1, int NC, int KIND>
 int elem_fxgl_seq(int64_t nelem) {
-  return fx_seq(nelem, FxGlShape<P1, KIND>::EB, elem_fxgl_resident<P1, NC, KIND, false>());
+  return fx_seq(nelem, FxGlShape<P1, KIND>::EB, elem_fxgl_resident<P1, NC, KIND, false, false>());
 }
 
 template <int P1, int NC, int KIND>
@@ -426,12 +439,12 @@ int elem_fxgl_blocks_t(int64_t nelem) {
   return int((nelem + per - 1) / per);
 }
 
-template <int P1, int NC, int KIND, bool HELM>
+template <int P1, int NC, int KIND, bool HELM, bool PAIR = false>
 cudaError_t launch_elem_fxgl_h(const DeviceMesh& m, const ElemArgs& a, cudaStream_t s) {
   using Sh = FxGlShape<P1, KIND>;
-  if (elem_fxgl_resident<P1, NC, KIND, HELM>() < 1) return cudaErrorInvalidConfiguration;
+  if (elem_fxgl_resident<P1, NC, KIND, HELM, PAIR>() < 1) return cudaErrorInvalidConfiguration;
   const int ns = elem_fxgl_seq<P1, NC, KIND>(m.nelem), blocks = elem_fxgl_blocks_t<P1, NC, KIND>(m.nelem);
-  elem_fxgl_kernel<P1, NC, KIND, HELM><<<blocks, Sh::NT, Sh::SMEM, s>>>(m, a, elem_fxgl_tab<P1>(m), ns);
+  elem_fxgl_kernel<P1, NC, KIND, HELM, PAIR><<<blocks, Sh::NT, Sh::SMEM, s>>>(m, a, elem_fxgl_tab<P1>(m), ns);
   return cudaGetLastError();
 }
 
@@ -443,6 +456,12 @@ cudaError_t launch_elem_fxgl_t(const DeviceMesh& m, int kind, const ElemArgs& a,
   }
   if (kind == kMass) return launch_elem_fxgl_h<P1, 1, kMass, false>(m, a, s);
   return a.beta != 0.0 ? launch_elem_fxgl_h<P1, 1, kStiff, true>(m, a, s) : launch_elem_fxgl_h<P1, 1, kStiff, false>(m, a, s);
+}
+
+template <int P1>
+cudaError_t launch_elem_fxgl_pair_t(const DeviceMesh& m, int kind, const ElemArgs& a, cudaStream_t s) {
+  return kind == kMass ? launch_elem_fxgl_h<P1, 1, kMass, false, true>(m, a, s)
+                       : launch_elem_fxgl_h<P1, 1, kStiff, false, true>(m, a, s);
 }
 
 // Largest grid of the order's launches with m's elements (room for their partial sums).

@@ -3,7 +3,9 @@
 
 namespace ceedbp {
 template cudaError_t launch_elem_fxgl_t<6>(const DeviceMesh& m, int kind, const ElemArgs& a, cudaStream_t s);
+template cudaError_t launch_elem_fxgl_pair_t<6>(const DeviceMesh& m, int kind, const ElemArgs& a, cudaStream_t s);
 template int elem_fxgl_blocks_any<6>(const DeviceMesh& m);
 template cudaError_t launch_elem_fxgl_t<7>(const DeviceMesh& m, int kind, const ElemArgs& a, cudaStream_t s);
+template cudaError_t launch_elem_fxgl_pair_t<7>(const DeviceMesh& m, int kind, const ElemArgs& a, cudaStream_t s);
 template int elem_fxgl_blocks_any<7>(const DeviceMesh& m);
 }  // namespace ceedbp

@@ -3,7 +3,9 @@
 
 namespace ceedbp {
 template cudaError_t launch_elem_fxgl_t<10>(const DeviceMesh& m, int kind, const ElemArgs& a, cudaStream_t s);
+template cudaError_t launch_elem_fxgl_pair_t<10>(const DeviceMesh& m, int kind, const ElemArgs& a, cudaStream_t s);
 template int elem_fxgl_blocks_any<10>(const DeviceMesh& m);
 template cudaError_t launch_elem_fxgl_t<11>(const DeviceMesh& m, int kind, const ElemArgs& a, cudaStream_t s);
+template cudaError_t launch_elem_fxgl_pair_t<11>(const DeviceMesh& m, int kind, const ElemArgs& a, cudaStream_t s);
 template int elem_fxgl_blocks_any<11>(const DeviceMesh& m);
 }  // namespace ceedbp

@@ -3,5 +3,6 @@
 
 namespace ceedbp {
 template cudaError_t launch_elem_fxgl_t<12>(const DeviceMesh& m, int kind, const ElemArgs& a, cudaStream_t s);
+template cudaError_t launch_elem_fxgl_pair_t<12>(const DeviceMesh& m, int kind, const ElemArgs& a, cudaStream_t s);
 template int elem_fxgl_blocks_any<12>(const DeviceMesh& m);
 }  // namespace ceedbp

@@ -133,8 +133,10 @@ cudaError_t launch_local_diag(const DeviceMesh& m, int kind, const double* G, co
 
 // Element operator: wl = A_L (Q u) or B_L (Q u) for ncomp components, optional
 // per-block dot partials of (Q u, wl); mask_in = read Dirichlet nodes as zero.
+struct dfloat;
 struct ElemArgs {
   const double* u;       // global input [nglobal][ncomp]
+  const dfloat* u_df;    // global input as pairs where u is nullptr (BP1/BP3 pair arithmetic; wl holds pairs then)
   double* wl;            // local output [E p1^3][ncomp]
   const double* G;       // stiffness factors or mass factors
   double* partials;      // [ncomp][nblocks] or nullptr
@@ -178,7 +180,6 @@ cudaError_t launch_dinv(const int* off, const double* diag, double* dinv, int64_
 
 // PCG kernels.
 int vec_blocks(int64_t n);
-inline int gather_blocks(int64_t n) { return vec_blocks((n + 1) / 2); }  // two nodes a thread
 cudaError_t launch_pcg_init(const DeviceMesh& m, const double* b, const double* ax, double* x, double* r, double* p,
                             const double* dinv, double* partials, SolveState* st, double tol,
                             int fixed, cudaStream_t s);
@@ -201,9 +202,7 @@ cudaError_t launch_elem_df(const DeviceMesh& m, const ElemDfArgs& a, cudaStream_
 bool elem_dfeo_supported(const DeviceMesh& m);
 int elem_dfeo_candidates(const DeviceMesh& m, int* eb, int* ns, int cap);
 cudaError_t launch_elem_dfeo(const DeviceMesh& m, const ElemDfArgs& a, cudaStream_t s);
-// BP1/BP3 (Gauss quadrature) on FP32 pairs; a.D holds the pair tables J [q][p1] then Dq [q][q].
-bool elem_dfgl_supported(const DeviceMesh& m);
-int elem_dfgl_blocks(const DeviceMesh& m);
+// BP1/BP3 (Gauss quadrature) with FP32 pairs in and out: the fixed-point kernel of elem_fxgl.cuh.
 cudaError_t launch_elem_dfgl(const DeviceMesh& m, const ElemDfArgs& a, cudaStream_t s);
 cudaError_t launch_init_df(const DeviceMesh& m, const double* b, const double* ax, double* x, dfloat* xd, dfloat* r,
                            dfloat* p, const dfloat* dinv, int x0, double* partials, SolveState* st, double tol,

@@ -14,7 +14,8 @@ struct ElemDfArgs {
   const double* u_f64;   // global input in FP64 (apply), or nullptr
   const dfloat* u_df;    // global input as pairs (CG direction), or nullptr
   dfloat* wl;            // local output [E p1^3][ncomp] pairs
-  const dfloat* G;       // [E][6][p1^3] pairs
+  const dfloat* G;       // [E][6][p1^3] pairs (BP5/BP6)
+  const double* G64;     // FP64 factors (BP1/BP3: elements off the fixed-point grid)
   const dfloat* D;       // [p1][p1] pairs of the GLL derivative matrix
   float dnorm_row;       // max_i sum_n |D_in| (rounded up)
   float dnorm_col;       // max_i sum_n |D_ni| (rounded up)

@@ -92,6 +92,7 @@ extern "C" ceedbp_status ceedbp_apply_noalloc(const ceedbp_ctx* ctx, const doubl
     a.u_f64 = u_dev;
     a.wl = reinterpret_cast<dfloat*>(scratch);
     a.G = ctx->d_Gdf;
+    a.G64 = ctx->op_kind == kStiff ? ctx->d_G : ctx->d_Mq;
     a.D = ctx->d_Ddf;
     a.dnorm_row = ctx->dnorm_row;
     a.dnorm_col = ctx->dnorm_col;

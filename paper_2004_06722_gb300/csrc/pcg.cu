@@ -183,7 +183,7 @@ cudaError_t launch_pcg_init(const DeviceMesh& m, const double* b, const double* 
 
 cudaError_t launch_pcg_update(const DeviceMesh& m, const double* wl, double* r, const double* dinv, double* partials,
                               SolveState* st, int step, cudaStream_t s) {
-  const int nb = gather_blocks(m.nglobal);
+  const int nb = vec_blocks(m.nglobal);
   if (m.ncomp == 3)
     pcg_update_kernel<3><<<nb, 256, 0, s>>>(m.head, m.slots, wl, r, dinv, m.nglobal, partials, st, step);
   else

@@ -216,7 +216,7 @@ cudaError_t launch_init_df(const DeviceMesh& m, const double* b, const double* a
 
 cudaError_t launch_update_df(const DeviceMesh& m, const dfloat* wl, dfloat* r, const dfloat* dinv, double* partials,
                              SolveState* st, int step, cudaStream_t s) {
-  const int nb = gather_blocks(m.nglobal);
+  const int nb = vec_blocks(m.nglobal);
   if (m.ncomp == 3)
     update_df_kernel<3><<<nb, 256, 0, s>>>(m.head, m.slots, wl, r, dinv, m.nglobal, partials, st, step);
   else
@@ -247,9 +247,9 @@ cudaError_t launch_f64_to_df(const double* src, dfloat* dst, int64_t n, cudaStre
 cudaError_t launch_gs_df(const DeviceMesh& m, const dfloat* wl, double* w, int mask_out, cudaStream_t s) {
   if (!mask_out) return cudaErrorInvalidValue;  // the heads know no values of Dirichlet nodes
   if (m.ncomp == 3)
-    gs_df_kernel<3><<<gather_blocks(m.nglobal), 256, 0, s>>>(m.head, m.slots, wl, w, m.nglobal);
+    gs_df_kernel<3><<<vec_blocks(m.nglobal), 256, 0, s>>>(m.head, m.slots, wl, w, m.nglobal);
   else
-    gs_df_kernel<1><<<gather_blocks(m.nglobal), 256, 0, s>>>(m.head, m.slots, wl, w, m.nglobal);
+    gs_df_kernel<1><<<vec_blocks(m.nglobal), 256, 0, s>>>(m.head, m.slots, wl, w, m.nglobal);
   return cudaGetLastError();
 }
 

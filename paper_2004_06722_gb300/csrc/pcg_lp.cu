@@ -271,7 +271,7 @@ cudaError_t launch_inner_init(const DeviceMesh& m, int bf16, const double* r64, 
 
 cudaError_t launch_inner_update(const DeviceMesh& m, const float* wl, float* r, const float* dinv, double* partials,
                                 SolveState* st, int step, cudaStream_t s) {
-  const int nb = gather_blocks(m.nglobal);
+  const int nb = vec_blocks(m.nglobal);
   if (m.ncomp == 3)
     inner_update_kernel<3><<<nb, 256, 0, s>>>(m.head, m.slots, wl, r, dinv, m.nglobal, partials, st, step);
   else

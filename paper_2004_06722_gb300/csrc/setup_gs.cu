@@ -287,7 +287,7 @@ int vec_blocks(int64_t n) {
 
 cudaError_t launch_gs(const DeviceMesh& m, const double* wl, double* w, int mask_out, cudaStream_t s) {
   if (mask_out) {
-    const int nb = gather_blocks(m.nglobal);
+    const int nb = vec_blocks(m.nglobal);
     if (m.ncomp == 3) gs_kernel<3><<<nb, 256, 0, s>>>(m.head, m.slots, wl, w, m.nglobal);
     else gs_kernel<1><<<nb, 256, 0, s>>>(m.head, m.slots, wl, w, m.nglobal);
   } else {
