@@ -64,19 +64,22 @@ __device__ __forceinline__ int2 fx_factor(double g, double w3, double rw3, doubl
 template <int NF>
 __global__ void fx_factors_kernel(const double* __restrict__ G, const double* __restrict__ w, int q, double ch,
                                   double cl, int ce, void* out, int* __restrict__ gexp) {
-  __shared__ double sw[kMaxQ], sred[2][32];
+  __shared__ double sw[kMaxQ], srw[kMaxQ], sred[2][32];
   __shared__ int s_bad;
   const int64_t e = blockIdx.x;
   const int q2 = q * q, q3 = q2 * q, tid = threadIdx.x;
   const double* Ge = G + e * NF * q3;
-  if (tid < q) sw[tid] = w[tid];
+  if (tid < q) {
+    sw[tid] = w[tid];
+    srw[tid] = 1.0 / w[tid];
+  }
   if (tid == 0) s_bad = 0;
   __syncthreads();
   // largest row sum of |G| and smallest point-wise largest entry, both without the weights
   double big = 0.0, small = __longlong_as_double(0x7fefffffffffffffll);
   bool bad = false;
   for (int p = tid; p < q3; p += blockDim.x) {
-    const double rw3 = 1.0 / (sw[p % q] * sw[(p / q) % q] * sw[p / q2]);
+    const double rw3 = srw[p % q] * srw[(p / q) % q] * srw[p / q2];
     double f[NF];
 #pragma unroll
     for (int c = 0; c < NF; ++c) {
@@ -117,7 +120,7 @@ __global__ void fx_factors_kernel(const double* __restrict__ G, const double* __
   if (off) return;
   const double ah = scalbn(ch, 62 - k), al = scalbn(cl, 62 - k);
   for (int p = tid; p < q3; p += blockDim.x) {
-    const double w3 = sw[p % q] * sw[(p / q) % q] * sw[p / q2], rw3 = 1.0 / w3;
+    const double w3 = sw[p % q] * sw[(p / q) % q] * sw[p / q2], rw3 = srw[p % q] * srw[(p / q) % q] * srw[p / q2];
     if constexpr (NF == 6) {
       int2 l[6];
 #pragma unroll
@@ -135,11 +138,12 @@ __global__ void fx_factors_kernel(const double* __restrict__ G, const double* __
 
 cudaError_t launch_fx_factors(const DeviceMesh& m, int kind, const double* G, void* out, int* gexp, cudaStream_t s) {
   const double* w = m.basis + 2 * size_t(m.q) * m.p1 + size_t(m.q) * m.q;
+  const int threads = m.q <= 5 ? 128 : 256;
   int e = 0;
   const long double c = 2.0L * std::frexp(kind == kStiff ? m.fx->chain : m.fx->mchain, &e);  // chain = c 2^(e-1)
   const double ch = double(c), cl = double(c - ch);
-  if (kind == kStiff) fx_factors_kernel<6><<<unsigned(m.nelem), 256, 0, s>>>(G, w, m.q, ch, cl, e - 1, out, gexp);
-  else fx_factors_kernel<1><<<unsigned(m.nelem), 256, 0, s>>>(G, w, m.q, ch, cl, e - 1, out, gexp);
+  if (kind == kStiff) fx_factors_kernel<6><<<unsigned(m.nelem), threads, 0, s>>>(G, w, m.q, ch, cl, e - 1, out, gexp);
+  else fx_factors_kernel<1><<<unsigned(m.nelem), threads, 0, s>>>(G, w, m.q, ch, cl, e - 1, out, gexp);
   return cudaGetLastError();
 }
 
