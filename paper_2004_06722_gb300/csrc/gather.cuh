@@ -15,6 +15,11 @@ namespace ceedbp {
 constexpr int kHeadDirichlet = -1;              // also nodes past the end
 constexpr int kHeadEmpty = int(0x80000000u);    // a node that no element touches
 constexpr int kSlotMask = 0x7fffffff;
+// U, the nodes a thread has in flight: with three components one, whose registers leave room for more blocks
+// (FP64 update, N = 7, 12^3 elements: 43 us, 51 with two); with one component two, unless the grid holds all
+// nodes already, when a second one only costs registers (N = 7: 257 us with two, 371 with one at 2^16 elements,
+// 18.7 and 14.7 us at 8^3)
+inline bool gather_one(int64_t n, int blocks) { return n <= int64_t(blocks) * 256; }
 
 __device__ __forceinline__ void gather_add(double& w, double v) { w += v; }
 __device__ __forceinline__ void gather_add(float& w, float v) { w += v; }

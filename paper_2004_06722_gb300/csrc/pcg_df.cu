@@ -69,7 +69,7 @@ __global__ void init_df_kernel(const int* __restrict__ off, const double* __rest
   }
 }
 
-template <int NC>
+template <int NC, int U>
 __global__ void __launch_bounds__(256) update_df_kernel(const int* __restrict__ head, const int* __restrict__ slots,
                                                         const dfloat* __restrict__ wl, dfloat* __restrict__ r,
                                                         const dfloat* __restrict__ dinv, int64_t n,
@@ -90,19 +90,19 @@ __global__ void __launch_bounds__(256) update_df_kernel(const int* __restrict__ 
 #pragma unroll
   for (int c = 0; c < NC; ++c) rz[c] = rr[c] = dfloat{0.0f, 0.0f};
   const int64_t stride = int64_t(gridDim.x) * 256;
-  for (int64_t g0 = int64_t(blockIdx.x) * 256 + threadIdx.x; g0 < n; g0 += 2 * stride) {
-    int hd[2];
-    dfloat w[2][NC], rv[2][NC], di[2];
+  for (int64_t g0 = int64_t(blockIdx.x) * 256 + threadIdx.x; g0 < n; g0 += U * stride) {
+    int hd[U];
+    dfloat w[U][NC], rv[U][NC], di[U];
 #pragma unroll
-    for (int h = 0; h < 2; ++h) {
+    for (int h = 0; h < U; ++h) {
       const int64_t g = g0 + h * stride < n ? g0 + h * stride : g0;
       di[h] = dinv[g];
 #pragma unroll
       for (int c = 0; c < NC; ++c) rv[h][c] = r[size_t(g) * NC + c];
     }
-    gather_nodes<2, NC>(head, slots, wl, g0, stride, n, hd, w);
+    gather_nodes<U, NC>(head, slots, wl, g0, stride, n, hd, w);
 #pragma unroll
-    for (int h = 0; h < 2; ++h) {
+    for (int h = 0; h < U; ++h) {
       if (hd[h] == kHeadDirichlet) continue;
 #pragma unroll
       for (int c = 0; c < NC; ++c) {
@@ -185,16 +185,16 @@ __global__ void f64_to_df_kernel(const double* __restrict__ src, dfloat* __restr
 }
 
 // mask_out: Dirichlet rows are zero; their values are not read (the element kernels may skip them).
-template <int NC>
+template <int NC, int U>
 __global__ void __launch_bounds__(256) gs_df_kernel(const int* __restrict__ head, const int* __restrict__ slots,
                                                     const dfloat* __restrict__ wl, double* __restrict__ w, int64_t n) {
   const int64_t stride = int64_t(gridDim.x) * 256;
-  for (int64_t g0 = int64_t(blockIdx.x) * 256 + threadIdx.x; g0 < n; g0 += 2 * stride) {
-    int hd[2];
-    dfloat v[2][NC];
-    gather_nodes<2, NC>(head, slots, wl, g0, stride, n, hd, v);
+  for (int64_t g0 = int64_t(blockIdx.x) * 256 + threadIdx.x; g0 < n; g0 += U * stride) {
+    int hd[U];
+    dfloat v[U][NC];
+    gather_nodes<U, NC>(head, slots, wl, g0, stride, n, hd, v);
 #pragma unroll
-    for (int h = 0; h < 2; ++h)
+    for (int h = 0; h < U; ++h)
       if (g0 + h * stride < n)
 #pragma unroll
         for (int c = 0; c < NC; ++c) w[size_t(g0 + h * stride) * NC + c] = df_to_f64(v[h][c]);
@@ -218,9 +218,11 @@ cudaError_t launch_update_df(const DeviceMesh& m, const dfloat* wl, dfloat* r, c
                              SolveState* st, int step, cudaStream_t s) {
   const int nb = vec_blocks(m.nglobal);
   if (m.ncomp == 3)
-    update_df_kernel<3><<<nb, 256, 0, s>>>(m.head, m.slots, wl, r, dinv, m.nglobal, partials, st, step);
+    update_df_kernel<3, 1><<<nb, 256, 0, s>>>(m.head, m.slots, wl, r, dinv, m.nglobal, partials, st, step);
+  else if (gather_one(m.nglobal, nb))
+    update_df_kernel<1, 1><<<nb, 256, 0, s>>>(m.head, m.slots, wl, r, dinv, m.nglobal, partials, st, step);
   else
-    update_df_kernel<1><<<nb, 256, 0, s>>>(m.head, m.slots, wl, r, dinv, m.nglobal, partials, st, step);
+    update_df_kernel<1, 2><<<nb, 256, 0, s>>>(m.head, m.slots, wl, r, dinv, m.nglobal, partials, st, step);
   return cudaGetLastError();
 }
 
@@ -246,10 +248,13 @@ cudaError_t launch_f64_to_df(const double* src, dfloat* dst, int64_t n, cudaStre
 
 cudaError_t launch_gs_df(const DeviceMesh& m, const dfloat* wl, double* w, int mask_out, cudaStream_t s) {
   if (!mask_out) return cudaErrorInvalidValue;  // the heads know no values of Dirichlet nodes
+  const int nb = vec_blocks(m.nglobal);
   if (m.ncomp == 3)
-    gs_df_kernel<3><<<vec_blocks(m.nglobal), 256, 0, s>>>(m.head, m.slots, wl, w, m.nglobal);
+    gs_df_kernel<3, 1><<<nb, 256, 0, s>>>(m.head, m.slots, wl, w, m.nglobal);
+  else if (gather_one(m.nglobal, nb))
+    gs_df_kernel<1, 1><<<nb, 256, 0, s>>>(m.head, m.slots, wl, w, m.nglobal);
   else
-    gs_df_kernel<1><<<vec_blocks(m.nglobal), 256, 0, s>>>(m.head, m.slots, wl, w, m.nglobal);
+    gs_df_kernel<1, 2><<<nb, 256, 0, s>>>(m.head, m.slots, wl, w, m.nglobal);
   return cudaGetLastError();
 }
 

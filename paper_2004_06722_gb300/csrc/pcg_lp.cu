@@ -112,7 +112,7 @@ __global__ void inner_init_kernel(const int* __restrict__ off, const double* __r
   }
 }
 
-template <int NC>
+template <int NC, int U>
 __global__ void __launch_bounds__(256) inner_update_kernel(const int* __restrict__ head, const int* __restrict__ slots,
                                                            const float* __restrict__ wl, float* __restrict__ r,
                                                            const float* __restrict__ dinv, int64_t n,
@@ -133,19 +133,19 @@ __global__ void __launch_bounds__(256) inner_update_kernel(const int* __restrict
 #pragma unroll
   for (int c = 0; c < NC; ++c) rz[c] = rr[c] = dfloat{0.0f, 0.0f};
   const int64_t stride = int64_t(gridDim.x) * 256;
-  for (int64_t g0 = int64_t(blockIdx.x) * 256 + threadIdx.x; g0 < n; g0 += 2 * stride) {
-    int hd[2];
-    float w[2][NC], rv[2][NC], di[2];
+  for (int64_t g0 = int64_t(blockIdx.x) * 256 + threadIdx.x; g0 < n; g0 += U * stride) {
+    int hd[U];
+    float w[U][NC], rv[U][NC], di[U];
 #pragma unroll
-    for (int h = 0; h < 2; ++h) {
+    for (int h = 0; h < U; ++h) {
       const int64_t g = g0 + h * stride < n ? g0 + h * stride : g0;
       di[h] = dinv[g];
 #pragma unroll
       for (int c = 0; c < NC; ++c) rv[h][c] = r[size_t(g) * NC + c];
     }
-    gather_nodes<2, NC>(head, slots, wl, g0, stride, n, hd, w);
+    gather_nodes<U, NC>(head, slots, wl, g0, stride, n, hd, w);
 #pragma unroll
-    for (int h = 0; h < 2; ++h) {
+    for (int h = 0; h < U; ++h) {
       if (hd[h] == kHeadDirichlet) continue;
 #pragma unroll
       for (int c = 0; c < NC; ++c) {
@@ -273,9 +273,11 @@ cudaError_t launch_inner_update(const DeviceMesh& m, const float* wl, float* r, 
                                 SolveState* st, int step, cudaStream_t s) {
   const int nb = vec_blocks(m.nglobal);
   if (m.ncomp == 3)
-    inner_update_kernel<3><<<nb, 256, 0, s>>>(m.head, m.slots, wl, r, dinv, m.nglobal, partials, st, step);
+    inner_update_kernel<3, 1><<<nb, 256, 0, s>>>(m.head, m.slots, wl, r, dinv, m.nglobal, partials, st, step);
+  else if (gather_one(m.nglobal, nb))
+    inner_update_kernel<1, 1><<<nb, 256, 0, s>>>(m.head, m.slots, wl, r, dinv, m.nglobal, partials, st, step);
   else
-    inner_update_kernel<1><<<nb, 256, 0, s>>>(m.head, m.slots, wl, r, dinv, m.nglobal, partials, st, step);
+    inner_update_kernel<1, 2><<<nb, 256, 0, s>>>(m.head, m.slots, wl, r, dinv, m.nglobal, partials, st, step);
   return cudaGetLastError();
 }
 

@@ -221,16 +221,16 @@ __global__ void gs_all_kernel(const int* __restrict__ off, const int* __restrict
 }
 
 // Dirichlet rows zero; their values are not read (the element kernels may skip them)
-template <int NC>
+template <int NC, int U>
 __global__ void __launch_bounds__(256) gs_kernel(const int* __restrict__ head, const int* __restrict__ slots,
                                                  const double* __restrict__ wl, double* __restrict__ w, int64_t n) {
   const int64_t stride = int64_t(gridDim.x) * 256;
-  for (int64_t g0 = int64_t(blockIdx.x) * 256 + threadIdx.x; g0 < n; g0 += 2 * stride) {
-    int hd[2];
-    double v[2][NC];
-    gather_nodes<2, NC>(head, slots, wl, g0, stride, n, hd, v);
+  for (int64_t g0 = int64_t(blockIdx.x) * 256 + threadIdx.x; g0 < n; g0 += U * stride) {
+    int hd[U];
+    double v[U][NC];
+    gather_nodes<U, NC>(head, slots, wl, g0, stride, n, hd, v);
 #pragma unroll
-    for (int h = 0; h < 2; ++h)
+    for (int h = 0; h < U; ++h)
       if (g0 + h * stride < n)
 #pragma unroll
         for (int c = 0; c < NC; ++c) w[size_t(g0 + h * stride) * NC + c] = v[h][c];
@@ -319,8 +319,11 @@ int vec_blocks(int64_t n) {
 cudaError_t launch_gs(const DeviceMesh& m, const double* wl, double* w, int mask_out, cudaStream_t s) {
   if (mask_out) {
     const int nb = vec_blocks(m.nglobal);
-    if (m.ncomp == 3) gs_kernel<3><<<nb, 256, 0, s>>>(m.head, m.slots, wl, w, m.nglobal);
-    else gs_kernel<1><<<nb, 256, 0, s>>>(m.head, m.slots, wl, w, m.nglobal);
+    if (m.ncomp == 3) gs_kernel<3, 1><<<nb, 256, 0, s>>>(m.head, m.slots, wl, w, m.nglobal);
+    else if (gather_one(m.nglobal, nb))
+      gs_kernel<1, 1><<<nb, 256, 0, s>>>(m.head, m.slots, wl, w, m.nglobal);
+    else
+      gs_kernel<1, 2><<<nb, 256, 0, s>>>(m.head, m.slots, wl, w, m.nglobal);
   } else {
     const int nb = vec_blocks(m.nglobal);
     if (m.ncomp == 3) gs_all_kernel<3><<<nb, 256, 0, s>>>(m.off, m.slots, wl, w, m.nglobal);
