@@ -143,7 +143,6 @@ __global__ void __launch_bounds__(FxCoShape<P1>::NT, FxCoShape<P1>::MINB)
   using Sh = FxCoShape<P1>;
   constexpr int PP = Sh::PP, P3 = Sh::P3, EB = Sh::EB, S = Sh::S, PS = P1 * S;
   extern __shared__ __align__(16) double smem_fx[];
-  if (a.state != nullptr && a.state->stop) return;
   double* red = smem_fx;                                  // 32 * NC
   unsigned* smax = reinterpret_cast<unsigned*>(red + 96);  // [u, fluxes][2][EB]
   const int tid = threadIdx.x;
@@ -192,8 +191,9 @@ __global__ void __launch_bounds__(FxCoShape<P1>::NT, FxCoShape<P1>::MINB)
   if (live) {
     load_l2g(0);
     prefetch_G(elem_of(0));
-    fetch_u(0);
   }
+  if (a.state != nullptr && a.state->stop) return;  // read beside the map
+  if (live) fetch_u(0);
   double dot[NC];
 #pragma unroll
   for (int c = 0; c < NC; ++c) dot[c] = 0.0;

@@ -217,7 +217,6 @@ __global__ void __launch_bounds__(FxGlShape<P1, KIND>::NT, FxGlShape<P1, KIND>::
   constexpr int QQ = Sh::QQ, Q3 = Sh::Q3, P3 = Sh::P3, EB = Sh::EB, S = Sh::S, PS = Sh::PS, NPT = Sh::NPT;
   constexpr int NF = KIND == kStiff ? 6 : 1;
   extern __shared__ __align__(16) double smem_fx[];
-  if (a.state != nullptr && a.state->stop) return;
   double* red = smem_fx;                                   // 32 * NC
   unsigned* smax = reinterpret_cast<unsigned*>(red + 96);  // [u, stage 1, 2, 3][2][EB]
   const int tid = threadIdx.x;
@@ -267,8 +266,9 @@ __global__ void __launch_bounds__(FxGlShape<P1, KIND>::NT, FxGlShape<P1, KIND>::
   if (live) {
     load_l2g(0);
     prefetch_factors(elem_of(0));
-    fetch_u(0);
   }
+  if (a.state != nullptr && a.state->stop) return;  // read beside the map
+  if (live) fetch_u(0);
   double dot[NC];
 #pragma unroll
   for (int c = 0; c < NC; ++c) dot[c] = 0.0;
