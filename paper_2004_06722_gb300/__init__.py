@@ -10,6 +10,7 @@ from __future__ import annotations
 
 import ctypes
 import os
+import threading
 
 import numpy as np
 
@@ -160,6 +161,7 @@ class Operator:
         self.device = torch.device("cuda") if device is None else torch.device(device)
         # a dedicated stream: CUDA graphs cannot be captured on the legacy default stream
         self.stream = torch.cuda.Stream(self.device) if stream is None else stream
+        self._events = threading.local()
         self.bp, self.order = bp, order
         self.ncomp = 3 if bp in (2, 4, 6) else 1
         coords = np.ascontiguousarray(coords, dtype=np.float64)
@@ -205,16 +207,24 @@ class Operator:
         shape = (self.nglobal,) if self.ncomp == 1 else (self.nglobal, 3)
         return torch.empty(shape, dtype=torch.float64, device=self.device)
 
+    # The operator's stream waits for the caller's before a call and the caller's for it afterwards, with two
+    # events kept for each calling thread: making two new ones took 2.4 us of a 26 us call on 4^3 elements.
     def _enter(self):
         import torch
         cur = torch.cuda.current_stream(self.device)
         if cur.cuda_stream != self.stream.cuda_stream:
-            self.stream.wait_stream(cur)
+            ev = getattr(self._events, "pair", None)
+            if ev is None:
+                ev = self._events.pair = (torch.cuda.Event(), torch.cuda.Event())
+            ev[0].record(cur)
+            self.stream.wait_event(ev[0])
         return cur
 
     def _leave(self, cur):
         if cur.cuda_stream != self.stream.cuda_stream:
-            cur.wait_stream(self.stream)
+            ev = self._events.pair
+            ev[1].record(self.stream)
+            cur.wait_event(ev[1])
 
     def _call(self, fn, *args):
         cur = self._enter()
