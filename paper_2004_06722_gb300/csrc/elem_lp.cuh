@@ -1,7 +1,7 @@
 // Low-precision BK5/BK6 element kernel for the inner solve of FP64 defect
 // correction: FP32 arithmetic, with the geometric factors and the input
-// direction stored in FP32 or in BF16 (TS).  Same operator and layout as the
-// collocated elem_kernel (Eq. (22) with J = I, factors of Eq. (23)); the local
+// direction stored in FP32 or in BF16 (TS).  The operator of Eq. (22) with J = I
+// and the factors of Eq. (23); thread (i, j) owns the column of nodes (i, j, .); the local
 // output w_L is FP32.  The fused (p, A p) of Algorithm 1 is accumulated as an
 // FP32 pair per thread (two_prod + dw_add) and reduced in FP64, so the CG
 // inner products keep FP64 accuracy while the operator runs in FP32.

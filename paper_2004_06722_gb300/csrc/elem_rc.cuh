@@ -7,7 +7,7 @@
 // operator: dx_d/dr_m = (D_m x_d)(i, j, k), nine contractions of length p1.
 // From it, Eq. (23): G = rho_i rho_j rho_k adj(J) adj(J)^T / |J| (adj(J) =
 // |J| J^{-1}), six symmetric components, and then the operator of Eq. (22)
-// exactly as in elem_kernel.  The element reads 3 coordinates per node
+// in plain FP64.  The element reads 3 coordinates per node
 // (stored [E][3][p1^3]) instead of 6 factors: 24 fewer bytes per node for
 // about 9 p1 + 40 more FMAs per node.
 //
