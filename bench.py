@@ -302,17 +302,15 @@ def measure(pkg, args, mesh, arith, device, rank, world, dist, geom=0):
     if pair_eo:
         name = "df64eo"
     traffic = ncu_traffic(f"bk5_{name}_n{N}.md")
-    if arith == pkg.ARITH_FP64:
+    if rc:
         ach = elem_flops / (elem_ms * 1e-3) / 1e12
-        kname = "elem_rc_kernel (BK5, FP64, factors recomputed)" if rc else "elem_eo_kernel (BK5, FP64, even-odd)"
         roof = {"bound": "alu", "achieved": ach, "peak": fp64_tf, "unit": "TFLOP/s", "frac": ach / fp64_tf,
-                "traffic": traffic, "kernel": kname, "peak_source": fp64_src,
+                "traffic": traffic, "kernel": "elem_rc_kernel (BK5, FP64, factors recomputed)", "peak_source": fp64_src,
                 "peak_derived_tflops": fp64_peak_tflops(peaks)[0],
                 "hbm_frac": (elem_bytes / (elem_ms * 1e-3) / 1e9) / peaks["hbm_gbs"]}
         # the FP64 work the kernel actually executes (ncu thread-instruction counts per element of
         # the same kernel): DFMA counts 2 flops, DADD and DMUL 1
-        name_i = f"bk5_{'fp64rc' if rc else 'fp64'}_n{N}.md"
-        inst = [ncu_value(name_i, k) for k in ("dfma_per_element", "dadd_per_element", "dmul_per_element")]
+        inst = [ncu_value(f"bk5_fp64rc_n{N}.md", k) for k in ("dfma_per_element", "dadd_per_element", "dmul_per_element")]
         if all(v is not None for v in inst):
             E = n_dofs // N ** 3
             exec_flops = (2 * inst[0] + inst[1] + inst[2]) * E
@@ -321,6 +319,16 @@ def measure(pkg, args, mesh, arith, device, rank, world, dist, geom=0):
             roof["executed_flops_per_dof"] = exec_flops / n_dofs
             # FP64 pipe: one DFMA, DADD or DMUL per slot, 2 slots per clock per SM (the peak's rate)
             roof["fp64_pipe_frac"] = sum(inst) * E / (elem_ms * 1e-3) / (fp64_tf * 1e12 / 2)
+    elif arith == pkg.ARITH_FP64:
+        # The contractions run on integers (60-bit values on a grid per element, FP64 in and out), so the
+        # FP64 FMA rate is no bound: bytes against HBM, and the issue share that ncu saw.
+        ach = elem_bytes / (elem_ms * 1e-3) / 1e9
+        roof = {"bound": "hbm", "achieved": ach, "peak": peaks["hbm_gbs"], "unit": "GB/s",
+                "frac": ach / peaks["hbm_gbs"], "traffic": traffic,
+                "kernel": "elem_fx_kernel (BK5, FP64 in and out, contractions in block fixed point)",
+                "peak_source": f"{peak_src} hbm_gbs",
+                "issue_active_pct_ncu": ncu_value(f"bk5_{name}_n{N}.md", "issue_active_pct"),
+                "fp64_equiv_tflops": elem_flops / (elem_ms * 1e-3) / 1e12, "fp64_fma_peak_tflops": fp64_tf}
     else:
         ach = elem_bytes / (elem_ms * 1e-3) / 1e9
         roof = {"bound": "hbm", "achieved": ach, "peak": peaks["hbm_gbs"], "unit": "GB/s",
@@ -397,8 +405,8 @@ def run_ours(args):
         "gpu_launches": head["gpu_launches"], "clocks": head["clocks"], "wall_s_timed": head["wall_s_timed"],
         "solver": head["solver"], "variants": variants,
     }
-    # the HBM-roofline fraction of the iteration in each arithmetic, side by side: native FP64 is
-    # bound by the FP64 pipe; the pair arithmetic carries 47-bit (not 53-bit) significands
+    # the HBM-roofline fraction of the iteration in each arithmetic, side by side; the pair
+    # arithmetic carries 47-bit (not 53-bit) significands
     line["hbm_roofline_by_arith"] = {
         head["dtype"]: head["hbm_roofline"]["frac"],
         **{v["dtype"] + (" recomputed factors" if k == "fp64_recompute" else ""): v["hbm_roofline"]["frac"]
