@@ -64,7 +64,8 @@ typedef enum {
 
 /* Arithmetic of the FP64 operator and solver (ceedbp_params.arith). */
 enum {
-  CEEDBP_ARITH_FP64 = 0, /* native FP64 instructions */
+  CEEDBP_ARITH_FP64 = 0, /* FP64 in and out; contractions on 60-bit integers per element with
+                            the accuracy of FP64 (batched solves: FP64 instructions) */
   CEEDBP_ARITH_DF64 = 1  /* FP64-accurate pairs of FP32 numbers (hi + lo, ~2^-46 relative per
                             value) on the FP32 pipe, which the GB300 issues 63x faster than
                             FP64; BP1, BP3, BP5 and BP6 (EUNSUPPORTED for BP2 and BP4).
