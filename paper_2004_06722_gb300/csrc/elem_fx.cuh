@@ -40,7 +40,10 @@ struct FxCoTab {
   double w[P1];   // GLL weights
 };
 
-template <int P1>
+// W: threads per column of an element: 1, or 3 on small meshes (elem_fx_wide). Three groups of p1^2 threads
+// then take one direction's lines and every third point of the columns each: the same operations in the
+// same order on every value, a shorter chain for one element, more barriers and less reuse for many.
+template <int P1, int W = 1>
 struct FxCoShape {
   static constexpr int PP = P1 * P1, P3 = PP * P1;
   static constexpr int S = P1 | 1;      // odd row length: lines of every direction are free of bank conflicts
@@ -49,8 +52,9 @@ struct FxCoShape {
   // the whole block and lives in uniform registers, and a barrier joins p1^2 threads only (N = 7,
   // E = 2^16: 704 -> 658 us against two elements per block; N = 8, E = 15625: 523 -> 337 us against
   // three).  Several where it would leave lanes idle (p1 = 6: 365 us with seven, 445 us with one, E = 40^3).
-  static constexpr int EB = P1 == 2 ? 32 : P1 == 3 ? 14 : P1 == 4 ? 8 : P1 == 5 ? 5 : P1 == 6 ? 7 : 1;
-  static constexpr int NT = (EB * PP + 31) / 32 * 32;
+  static constexpr int EB = W == 3 ? 1 : P1 == 2 ? 32 : P1 == 3 ? 14 : P1 == 4 ? 8 : P1 == 5 ? 5 : P1 == 6 ? 7 : 1;
+  static constexpr int NT = (EB * W * PP + 31) / 32 * 32;
+  static constexpr int KC = (P1 + W - 1) / W;  // points of a column per thread
   // u buffers: the next element's values land while the current one is computed; from p1 = 13 to 15 one
   // buffer, filled between elements, lets one more block fit on the SM instead
   static constexpr int NU = P1 >= 13 && P1 <= 15 ? 1 : 2;
@@ -63,13 +67,13 @@ struct FxCoShape {
   // Blocks per SM the registers are limited for: what shared memory holds, at 96 registers or more
   // (p1 = 8: eight blocks, 120 registers: 350 us at E = 2^15; ten, 96 registers: 370 us).
   static constexpr int BY_SMEM = int((size_t(227) << 10) / (SMEM + 1024)), BY_REGS = 65536 / (NT * 96);
-  static constexpr int MINB = P1 == 8 ? 8 : BY_SMEM < BY_REGS ? BY_SMEM : BY_REGS;
+  static constexpr int MINB = W == 3 ? 1 : P1 == 8 ? 8 : BY_SMEM < BY_REGS ? BY_SMEM : BY_REGS;
 };
 
 // Per-thread view of one element of a slot.
 template <int P1>
 struct FxCoElem {
-  int t, ti, tj;
+  int t, ti, tj, grp;  // grp: the direction group, 0 with one thread per column
   void* A;           // tiles A, B, C
   const double* su;  // the element's u, [k][t]
 };
@@ -77,10 +81,10 @@ struct FxCoElem {
 // Contractions and factors of one element in arithmetic Ar (FxArith or F64Arith), u in tile A.
 // factors(k, gradient, flux) multiplies by G at point k of the own column; done(shift) comes with the
 // number of bits the fluxes were moved up; out(k, r, s, t) receives the three transposes.
-template <int P1, class Ar, class Tab, class Factors, class Mid, class Done, class Out>
+template <int P1, int W, class Ar, class Tab, class Factors, class Mid, class Done, class Out>
 __device__ __forceinline__ void fx_co_stages(const FxCoElem<P1>& el, const Tab& D, const Tab& DT, bool live,
                                              const FxNorm& norm, Factors&& factors, Mid&& mid, Done&& done, Out&& out) {
-  using Sh = FxCoShape<P1>;
+  using Sh = FxCoShape<P1, W>;
   using L = typename Ar::L;
   using Raw = typename Ar::Raw;
   constexpr int S = Sh::S, PS = P1 * S;
@@ -89,6 +93,21 @@ __device__ __forceinline__ void fx_co_stages(const FxCoElem<P1>& el, const Tab& 
   // lines of thread t: r (j, k), base t S, step 1;  s (i, k), base k P1 S + i, step S;  t (i, j), the own column
   const int rb = el.t * S, sb = el.tj * PS + el.ti, own = el.tj * S + el.ti;
   Ar ar;
+  if constexpr (W == 3) {
+    const int dir = el.grp;
+    const int base = dir == 0 ? rb : dir == 1 ? sb : own, step = dir == 0 ? 1 : dir == 1 ? S : PS;
+    L l[P1];
+    if (live) {
+#pragma unroll
+      for (int n = 0; n < P1; ++n) l[n] = A[base + n * step];
+    }
+    __syncthreads();  // t goes in place
+    if (live) {
+      L* dst = A + (dir == 2 ? 0 : (dir + 1) * Sh::TILE) + base;
+      eo_line<Ar::kBias, P1, P1, true>(D, l, [&](int n, auto y) { dst[n * step] = Ar::limbs(y); });
+    }
+    __syncthreads();
+  } else {
 #pragma unroll Sh::UNROLL
   for (int dir = 0; dir < 3; ++dir) {
     if (dir == 2) __syncthreads();  // r and s have read tile A: t goes in place
@@ -101,10 +120,11 @@ __device__ __forceinline__ void fx_co_stages(const FxCoElem<P1>& el, const Tab& 
       eo_line<Ar::kBias, P1, P1, true>(D, l, [&](int n, auto y) { dst[n * step] = Ar::limbs(y); });
     }
   }
+  }
   mid();
   if (live) {
 #pragma unroll 4
-    for (int k = 0; k < P1; ++k) {
+    for (int k = el.grp; k < P1; k += W) {
       Raw fr, fs, ft;
       factors(k, B[own + k * PS], C[own + k * PS], A[own + k * PS], fr, fs, ft);
       ar.see(fr);
@@ -120,8 +140,8 @@ __device__ __forceinline__ void fx_co_stages(const FxCoElem<P1>& el, const Tab& 
   ar.take(norm, 1);
   done(ar.total);
   if (live) {
-#pragma unroll Sh::UNROLL
-    for (int dir = 0; dir < 3; ++dir) {
+#pragma unroll W == 3 ? 1 : Sh::UNROLL
+    for (int dir = el.grp; dir < 3; dir += W == 3 ? 3 : 1) {
       const int base = dir == 0 ? rb : dir == 1 ? sb : own, step = dir == 0 ? 1 : dir == 1 ? S : PS;
       Raw* dst = Ar_ + (dir == 2 ? 0 : (dir + 1) * Sh::TILE) + base;
       L l[P1];
@@ -133,25 +153,29 @@ __device__ __forceinline__ void fx_co_stages(const FxCoElem<P1>& el, const Tab& 
   __syncthreads();
   if (live) {
 #pragma unroll
-    for (int k = 0; k < P1; ++k) out(k, Br[own + k * PS], Cr[own + k * PS], Ar_[own + k * PS]);
+    for (int h = 0; h < Sh::KC; ++h) {
+      const int k = W * h + el.grp;
+      if (W == 1 || k < P1) out(h, k, Br[own + k * PS], Cr[own + k * PS], Ar_[own + k * PS]);
+    }
   }
 }
 
-template <int P1, int NC, bool HELM>
-__global__ void __launch_bounds__(FxCoShape<P1>::NT, FxCoShape<P1>::MINB)
+template <int P1, int NC, bool HELM, int W>
+__global__ void __launch_bounds__(FxCoShape<P1, W>::NT, FxCoShape<P1, W>::MINB)
     elem_fx_kernel(const DeviceMesh m, const ElemArgs a, const __grid_constant__ FxCoTab<P1> tab, const int ns) {
-  using Sh = FxCoShape<P1>;
-  constexpr int PP = Sh::PP, P3 = Sh::P3, EB = Sh::EB, S = Sh::S, PS = P1 * S;
+  using Sh = FxCoShape<P1, W>;
+  constexpr int PP = Sh::PP, P3 = Sh::P3, EB = Sh::EB, S = Sh::S, PS = P1 * S, KC = Sh::KC;
   extern __shared__ __align__(16) double smem_fx[];
   double* red = smem_fx;                                  // 32 * NC
   unsigned* smax = reinterpret_cast<unsigned*>(red + 96);  // [u, fluxes][2][EB]
   const int tid = threadIdx.x;
-  const int slot = tid / PP;
+  const int slot = tid / (W * PP);
   const bool live = slot < EB;  // threads that pad the block to whole warps only take part in barriers
   char* base = reinterpret_cast<char*>(smem_fx) + Sh::HEAD + size_t(live ? slot : 0) * Sh::SLOT;
   double* ubuf = reinterpret_cast<double*>(base);
   FxCoElem<P1> el;
-  el.t = tid - slot * PP;
+  el.grp = W == 1 ? 0 : tid / PP % W;
+  el.t = tid - (W * slot + el.grp) * PP;
   el.ti = el.t % P1;
   el.tj = el.t / P1;
   el.A = ubuf + Sh::NU * P3;
@@ -164,28 +188,29 @@ __global__ void __launch_bounds__(FxCoShape<P1>::NT, FxCoShape<P1>::MINB)
   const unsigned lanes = __match_any_sync(0xffffffffu, slot);  // the warp's lanes of this slot
   const bool lead = live && (tid & 31) == __ffs(int(lanes)) - 1;
 
-  int g[P1];
+  int g[KC];
   unsigned dnext = 0, dcur = 0;  // Dirichlet bits of the own column
   auto load_l2g = [&](int it) {
     const int* l2g = m.l2g + elem_of(it) * P3 + el.t;
 #pragma unroll
-    for (int k = 0; k < P1; ++k) g[k] = __ldg(l2g + k * PP);
+    for (int h = 0; h < KC; ++h) g[h] = W == 1 || W * h + el.grp < P1 ? __ldg(l2g + (W * h + el.grp) * PP) : 0;
   };
   auto fetch_u = [&](int it) {
     double* dst = ubuf + (it % Sh::NU) * P3 + el.t;
     const double* src = a.u + (NC == 1 ? 0 : it % NC);
     dnext = 0;
 #pragma unroll
-    for (int k = 0; k < P1; ++k) {
-      const int gg = g[k] ^ (g[k] >> 31);  // -(g + 1) for Dirichlet nodes
-      dnext |= unsigned(g[k] < 0) << k;
-      cp_async8_or_zero(dst + k * PP, src + size_t(gg) * NC, g[k] < 0 && a.mask_in);
+    for (int h = 0; h < KC; ++h) {
+      if (W > 1 && W * h + el.grp >= P1) continue;
+      const int gg = g[h] ^ (g[h] >> 31);  // -(g + 1) for Dirichlet nodes
+      dnext |= unsigned(g[h] < 0) << h;
+      cp_async8_or_zero(dst + (W * h + el.grp) * PP, src + size_t(gg) * NC, g[h] < 0 && a.mask_in);
     }
   };
   auto prefetch_G = [&](int64_t e) {
     const char* G = m.Gfx != nullptr ? reinterpret_cast<const char*>(m.Gfx + e * 3 * P3)
                                      : reinterpret_cast<const char*>(a.G + e * 6 * P3);
-    for (int b = el.t * 128; b < 48 * P3; b += PP * 128) l2_prefetch(G + b);
+    for (int b = (el.grp * PP + el.t) * 128; b < 48 * P3; b += W * PP * 128) l2_prefetch(G + b);
   };
   for (int i = tid; i < 4 * EB; i += Sh::NT) smax[i] = 0u;
   if (live) {
@@ -211,7 +236,9 @@ __global__ void __launch_bounds__(FxCoShape<P1>::NT, FxCoShape<P1>::MINB)
     unsigned mx = 0;
     if (live) {
 #pragma unroll
-      for (int k = 0; k < P1; ++k) mx = max(mx, unsigned(__double2hiint(el.su[k * PP])) & 0x7fffffffu);
+      for (int h = 0; h < KC; ++h)
+        if (W == 1 || W * h + el.grp < P1)
+          mx = max(mx, unsigned(__double2hiint(el.su[(W * h + el.grp) * PP])) & 0x7fffffffu);
       if (it + 1 < nit) load_l2g(it + 1);
     }
     mx = __reduce_max_sync(lanes, mx);
@@ -222,14 +249,14 @@ __global__ void __launch_bounds__(FxCoShape<P1>::NT, FxCoShape<P1>::MINB)
     int eb = live ? int(*norm.top >> 20) : 1023;
     const bool bad = live && (ge == kFxNoGrid || (eb != 0 && (eb < 500 || eb > 1500)));
     if (eb == 0) eb = 1023;  // every value is zero (or too small to matter to `bad` blocks): any exponent
-    if (el.t == 0 && live) smax[(~it & 1) * EB + slot] = smax[(2 + (~it & 1)) * EB + slot] = 0u;
+    if (el.t == 0 && el.grp == 0 && live) smax[(~it & 1) * EB + slot] = smax[(2 + (~it & 1)) * EB + slot] = 0u;
     double* wl = a.wl + size_t(e) * P3 * NC + size_t(el.t) * NC + c;
     double acc = 0.0;
-    auto finish = [&](int k, double w) {
+    auto finish = [&](int h, int k, double w) {
       const double u = el.su[k * PP];
       if constexpr (HELM) w += a.beta * __ldg(a.Mq + e * P3 + k * PP + el.t) * u;  // Eq. (17)
       if (store) {
-        if (!(a.skip_dirichlet_out && ((dcur >> k) & 1u))) wl[size_t(k) * PP * NC] = w;
+        if (!(a.skip_dirichlet_out && ((dcur >> h) & 1u))) wl[size_t(k) * PP * NC] = w;
         acc += w * u;
       }
     };
@@ -242,12 +269,13 @@ __global__ void __launch_bounds__(FxCoShape<P1>::NT, FxCoShape<P1>::MINB)
     if (live) {
       int2* A = static_cast<int2*>(el.A) + el.tj * S + el.ti;
 #pragma unroll
-      for (int k = 0; k < P1; ++k) A[k * PS] = fx_from_double(el.su[k * PP], eb);
+      for (int h = 0; h < KC; ++h)
+        if (const int k = W * h + el.grp; W == 1 || k < P1) A[k * PS] = fx_from_double(el.su[k * PP], eb);
     }
     if (!__syncthreads_or(bad)) {
       const int4* G = m.Gfx + e * 3 * P3 + el.t;
       double sc = 0.0;
-      fx_co_stages<P1, FxArith>(
+      fx_co_stages<P1, W, FxArith>(
           el, tab.D, tab.DT, live, norm,
           [&](int k, int2 r, int2 s, int2 t, long long& fr, long long& fs, long long& ft) {
             const int4 g0 = __ldcs(G + (3 * k + 0) * PP), g1 = __ldcs(G + (3 * k + 1) * PP),
@@ -260,18 +288,19 @@ __global__ void __launch_bounds__(FxCoShape<P1>::NT, FxCoShape<P1>::MINB)
           },
           mid,
           [&](int shift) { sc = wij * __hiloint2double((eb + ge - shift - (1082 - 1023)) << 20, 0); },
-          [&](int k, long long r, long long s, long long t) {
-            finish(k, __ll2double_rn(r + s + t) * (tab.w[k] * sc));
+          [&](int h, int k, long long r, long long s, long long t) {
+            finish(h, k, __ll2double_rn(r + s + t) * (tab.w[k] * sc));
           });
     } else {
       if (live) {
         double* A = static_cast<double*>(el.A) + el.tj * S + el.ti;
 #pragma unroll
-        for (int k = 0; k < P1; ++k) A[k * PS] = el.su[k * PP];
+        for (int h = 0; h < KC; ++h)
+          if (const int k = W * h + el.grp; W == 1 || k < P1) A[k * PS] = el.su[k * PP];
       }
       __syncthreads();
       const double* G = a.G + e * 6 * P3 + el.t;
-      fx_co_stages<P1, F64Arith>(
+      fx_co_stages<P1, W, F64Arith>(
           el, tab.D64, tab.DT64, live, norm,
           [&](int k, double r, double s, double t, double& fr, double& fs, double& ft) {
             const double* Gk = G + k * PP;
@@ -281,7 +310,7 @@ __global__ void __launch_bounds__(FxCoShape<P1>::NT, FxCoShape<P1>::MINB)
             fs = g01 * r + g11 * s + g12 * t;
             ft = g02 * r + g12 * s + g22 * t;
           },
-          mid, [](int) {}, [&](int k, double r, double s, double t) { finish(k, r + s + t); });
+          mid, [](int) {}, [&](int h, int k, double r, double s, double t) { finish(h, k, r + s + t); });
     }
     if (Sh::NU == 1 && live && it + 1 < nit) fetch_u(it + 1);  // the own column's values were read last above
 #pragma unroll
@@ -306,11 +335,21 @@ FxCoTab<P1> elem_fx_tab(const DeviceMesh& m) {
 
 // Blocks resident on the GPU (0: the kernel does not fit), found once per instantiation; the
 // attribute that lets it use its shared memory is set on the way.
-template <int P1, int NC, bool HELM>
+template <int P1, int NC, bool HELM, int W = 1>
 int elem_fx_resident() {
-  using Sh = FxCoShape<P1>;
-  static const int n = fx_resident(reinterpret_cast<const void*>(elem_fx_kernel<P1, NC, HELM>), Sh::NT, Sh::SMEM);
+  using Sh = FxCoShape<P1, W>;
+  static const int n = fx_resident(reinterpret_cast<const void*>(elem_fx_kernel<P1, NC, HELM, W>), Sh::NT, Sh::SMEM);
   return n;
+}
+
+// Three threads per column while every element has an SM to itself: the launch then lasts as long as one
+// element does (CG iteration in us, one / three threads: N = 4, E = 64 19.8 / 17.7; N = 5, E = 150 22.5 / 18.0;
+// N = 7, E = 150 22.2 / 19.4; N = 11, E = 64 32.4 / 28.0). With several elements on an SM the warps of one
+// fill the gaps of another and the extra barriers cost (N = 7: E = 256 23.5 / 22.3, 512 28.9 / 31.1, 1728
+// 52 / 60; N = 9, E = 256 33.9 / 37.2). Orders 1 and 2 have too little in a line (N = 1, E = 64 14.6 / 15.4).
+template <int P1, int NC>
+bool elem_fx_wide(int64_t nelem) {
+  return NC == 1 && P1 >= 4 && nelem <= fx_sms();
 }
 
 // Elements in a slot's sequence: one wave of resident blocks covers the mesh.
@@ -321,17 +360,25 @@ int elem_fx_seq(int64_t nelem) {
 
 template <int P1, int NC>
 int elem_fx_blocks_t(int64_t nelem) {
+  if (elem_fx_wide<P1, NC>(nelem)) return int(nelem);  // one element per block
   const int64_t per = int64_t(FxCoShape<P1>::EB) * elem_fx_seq<P1, NC>(nelem);
   return int((nelem + per - 1) / per);
 }
 
+template <int P1, int NC, bool HELM, int W>
+cudaError_t launch_elem_fx_w(const DeviceMesh& m, const ElemArgs& a, int ns, cudaStream_t s) {
+  using Sh = FxCoShape<P1, W>;
+  if (elem_fx_resident<P1, NC, HELM, W>() < 1) return cudaErrorInvalidConfiguration;
+  elem_fx_kernel<P1, NC, HELM, W>
+      <<<elem_fx_blocks_t<P1, NC>(m.nelem), Sh::NT, Sh::SMEM, s>>>(m, a, elem_fx_tab<P1>(m), ns);
+  return cudaGetLastError();
+}
+
 template <int P1, int NC, bool HELM>
 cudaError_t launch_elem_fx_h(const DeviceMesh& m, const ElemArgs& a, cudaStream_t s) {
-  if (elem_fx_resident<P1, NC, HELM>() < 1) return cudaErrorInvalidConfiguration;
-  const int ns = elem_fx_seq<P1, NC>(m.nelem), blocks = elem_fx_blocks_t<P1, NC>(m.nelem);
-  elem_fx_kernel<P1, NC, HELM>
-      <<<blocks, FxCoShape<P1>::NT, FxCoShape<P1>::SMEM, s>>>(m, a, elem_fx_tab<P1>(m), ns);
-  return cudaGetLastError();
+  if constexpr (NC == 1 && P1 >= 4)
+    if (elem_fx_wide<P1, NC>(m.nelem)) return launch_elem_fx_w<P1, NC, HELM, 3>(m, a, 1, s);
+  return launch_elem_fx_w<P1, NC, HELM, 1>(m, a, elem_fx_seq<P1, NC>(m.nelem), s);
 }
 
 template <int P1>

@@ -226,6 +226,18 @@ inline int fx_resident(const void* kernel, int threads, size_t smem) {
   return nb * sms;
 }
 
+// Host: SMs of the GPU, found once.
+inline int fx_sms() {
+  static const int n = [] {
+    int dev = 0, sms = 0;
+    return cudaGetDevice(&dev) == cudaSuccess &&
+                   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess
+               ? sms
+               : 0;
+  }();
+  return n;
+}
+
 // Host: elements in a slot's sequence such that one wave of resident blocks covers the mesh.
 inline int fx_seq(int64_t nelem, int per_block, int resident) {
   const int64_t full = (nelem + per_block - 1) / per_block, res = resident < 1 ? 1 : resident;

@@ -143,3 +143,18 @@ def test_zero_and_sparse_elements(bp, N):
     ref = _local(bp, (3, 1, 1), N, uL)
     assert not w[0].any() and not w[2].any()
     assert np.linalg.norm(w - ref) < 1e-12 * np.linalg.norm(ref)
+
+
+@pytest.mark.parametrize("N", [3, 4, 5, 6, 7, 8, 10, 11, 12])
+@pytest.mark.parametrize("dims", [(6, 5, 5), (6, 6, 5)])
+def test_threads_per_column(N, dims):
+    """Three threads per column while every element has an SM of its own (152: 150 elements), one above
+    (180): the first and the last elements against the oracle, on elements of even proportions."""
+    E = dims[0] * dims[1] * dims[2]
+    op = pkg.Operator.box(5, *dims, N)
+    uL = uniform_pm1(8, np.arange(E * (N + 1) ** 3)).reshape(E, -1)
+    w = _run(op, uL)
+    rule = bp_rule(5, N)
+    for e in (0, 1, E - 2, E - 1):
+        ref = element_matrices(op.coords[e], N, rule, want=("A",))["A"] @ uL[e]
+        assert np.linalg.norm(w[e] - ref) < 1e-12 * np.linalg.norm(ref)
