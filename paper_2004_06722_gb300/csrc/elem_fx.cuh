@@ -233,22 +233,22 @@ __global__ void __launch_bounds__(FxCoShape<P1, W>::NT, FxCoShape<P1, W>::MINB)
     el.su = ubuf + (it % Sh::NU) * P3 + el.t;
     cp_async_wait_all();
     dcur = dnext;
-    unsigned mx = 0;
+    FxTop seen;
     if (live) {
 #pragma unroll
       for (int h = 0; h < KC; ++h)
-        if (W == 1 || W * h + el.grp < P1)
-          mx = max(mx, unsigned(__double2hiint(el.su[(W * h + el.grp) * PP])) & 0x7fffffffu);
+        if (W == 1 || W * h + el.grp < P1) seen.see(el.su[(W * h + el.grp) * PP]);
       if (it + 1 < nit) load_l2g(it + 1);
     }
+    unsigned mx = seen.top();
     mx = __reduce_max_sync(lanes, mx);
     const int ge = live && m.gexp != nullptr ? __ldg(m.gexp + e) : kFxNoGrid;
     const FxNorm norm{lanes, lead, smax + (it & 1) * EB + (live ? slot : 0), 2 * EB};
     if (lead) atomicMax(norm.top, mx);
     __syncthreads();
-    int eb = live ? int(*norm.top >> 20) : 1023;
-    const bool bad = live && (ge == kFxNoGrid || (eb != 0 && (eb < 500 || eb > 1500)));
-    if (eb == 0) eb = 1023;  // every value is zero (or too small to matter to `bad` blocks): any exponent
+    const unsigned top = live ? *norm.top : 0u;
+    const int eb = top == 0u ? 1023 : int(top >> 20);  // every value is zero: any exponent
+    const bool bad = live && (ge == kFxNoGrid || eb < 500 || eb > 1500);
     if (el.t == 0 && el.grp == 0 && live) smax[(~it & 1) * EB + slot] = smax[(2 + (~it & 1)) * EB + slot] = 0u;
     double* wl = a.wl + size_t(e) * P3 * NC + size_t(el.t) * NC + c;
     double acc = 0.0;

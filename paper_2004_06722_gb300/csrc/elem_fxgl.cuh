@@ -288,21 +288,22 @@ __global__ void __launch_bounds__(FxGlShape<P1, KIND>::NT, FxGlShape<P1, KIND>::
       for (int n = 0; n < NPT; ++n)
         if (has(n)) su[t + n * QQ] = df_to_f64(reinterpret_cast<const dfloat*>(su)[t + n * QQ]);
     }
-    unsigned mx = 0;
+    FxTop seen;
     if (live) {
 #pragma unroll
       for (int n = 0; n < NPT; ++n)
-        if (has(n)) mx = max(mx, unsigned(__double2hiint(su[t + n * QQ])) & 0x7fffffffu);
+        if (has(n)) seen.see(su[t + n * QQ]);
       if (it + 1 < nit) load_l2g(it + 1);
     }
+    unsigned mx = seen.top();
     mx = __reduce_max_sync(lanes, mx);
     const int ge = !HELM && live && fxe != nullptr ? __ldg(fxe + e) : kFxNoGrid;
     const FxNorm norm{lanes, lead, smax + (it & 1) * EB + (live ? slot : 0), 2 * EB};
     if (lead) atomicMax(norm.top, mx);
     __syncthreads();
-    int eb = live ? int(*norm.top >> 20) : 1023;
-    const bool bad = live && (ge == kFxNoGrid || (eb != 0 && (eb < 500 || eb > 1500)));
-    if (eb == 0) eb = 1023;  // every value is zero (or too small to matter to `bad` blocks): any exponent
+    const unsigned top = live ? *norm.top : 0u;
+    const int eb = top == 0u ? 1023 : int(top >> 20);  // every value is zero: any exponent
+    const bool bad = live && (ge == kFxNoGrid || eb < 500 || eb > 1500);
     if (t < 4 && live) smax[(2 * t + (~it & 1)) * EB + slot] = 0u;
     auto mid = [&]() {
       if (live && it + 1 < nit) {

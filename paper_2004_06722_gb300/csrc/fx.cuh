@@ -157,6 +157,17 @@ __device__ __forceinline__ long long fx_dot3(int2 a, int2 x, int2 b, int2 y, int
   return fx_join(hh, mm);
 }
 
+// Largest magnitude of FP64 values by upper words; zero only if every value is zero (a subnormal whose upper
+// word is zero counts as one).
+struct FxTop {
+  unsigned hi = 0, lo = 0;
+  __device__ __forceinline__ void see(double v) {
+    hi = max(hi, unsigned(__double2hiint(v)) & 0x7fffffffu);
+    lo |= unsigned(__double2loint(v));
+  }
+  __device__ __forceinline__ unsigned top() const { return max(hi, min(lo, 1u)); }
+};
+
 // Where the threads of an element exchange the largest magnitude of a stage's values: one word for each
 // stage, `step` words apart.
 struct FxNorm {
