@@ -21,8 +21,8 @@
 // the element's actual maximum before the transposes, so that the two derivatives' slack does not add
 // up (fx_limbs_up).  With that the error of one application, against quad-precision references, stays
 // at or below that of the FP64 kernels this arithmetic replaces.  Values a grid cannot hold
-// (infinities, NaN, elements whose factors spread over more than 2^7, exponents near the ends of the
-// FP64 range) take the FP64 form of the same kernel (the double overloads below).
+// (infinities, NaN, elements whose factors spread over more than 2^5 (fx_setup.cu), exponents near the ends
+// of the FP64 range) take the FP64 form of the same kernel (the double overloads below).
 #pragma once
 
 #include "common.cuh"

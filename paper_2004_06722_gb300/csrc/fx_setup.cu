@@ -61,10 +61,22 @@ __device__ __forceinline__ int2 fx_factor(double g, double w3, double rw3, doubl
 // [1, 2) and 2^ce are mantissa and exponent of the tables' scales (their chain): one unit of the element's
 // result is then exactly 2^(k+ce) units of its input. NF = 6: stiffness factors
 // G [e][6][q^3] -> [e][k][3][q^2] pairs of entries (00,01), (02,11), (12,22); NF = 1: mass factors.
+//
+// An element is on the grid while the factors that carry it are within 2^kFxSpread of its largest row sum:
+// one direction's diagonal factors at all points (collocated), the larger ones of each point (Gauss, where
+// interpolation spreads every value over the element), the mass factors. A flux is known to one unit of
+// the largest, and a spread of 2^7 made results up to 5 times worse than FP64's on random values (2^4: equal).
+// D of orders 1 and 2 takes a constant to exact zeros in FP64, so collocated FP64 loses nothing of a function of the
+// weak direction of a thin element, the grid the ratio of the factors: all three directions (all_dirs) have to
+// be within 2^4 there (order 1, thickness 1/100, a function of x: 2e-14 of the result against 3e-17; from order 3
+// on, and with Gauss quadrature, both arithmetics lose the same).
+constexpr int kFxSpread = 5;
+
 template <int NF>
 __global__ void fx_factors_kernel(const double* __restrict__ G, const double* __restrict__ w, int q, double ch,
-                                  double cl, int ce, void* out, int* __restrict__ gexp) {
-  __shared__ double sw[kMaxQ], srw[kMaxQ], sred[2][32];
+                                  double cl, int ce, int colloc, int all_dirs, void* out, int* __restrict__ gexp) {
+  constexpr int NR = NF == 6 ? 5 : 2;  // largest row sum; smallest of each direction and of the points' largest
+  __shared__ double sw[kMaxQ], srw[kMaxQ], sred[NR][32];
   __shared__ int s_bad;
   const int64_t e = blockIdx.x;
   const int q2 = q * q, q3 = q2 * q, tid = threadIdx.x;
@@ -75,8 +87,11 @@ __global__ void fx_factors_kernel(const double* __restrict__ G, const double* __
   }
   if (tid == 0) s_bad = 0;
   __syncthreads();
-  // largest row sum of |G| and smallest point-wise largest entry, both without the weights
-  double big = 0.0, small = __longlong_as_double(0x7fefffffffffffffll);
+  // largest row sum of |G| and smallest diagonal entries, all without the weights
+  double v[NR];
+  v[0] = 0.0;
+#pragma unroll
+  for (int c = 1; c < NR; ++c) v[c] = __longlong_as_double(0x7fefffffffffffffll);
   bool bad = false;
   for (int p = tid; p < q3; p += blockDim.x) {
     const double rw3 = srw[p % q] * srw[(p / q) % q] * srw[p / q2];
@@ -86,36 +101,42 @@ __global__ void fx_factors_kernel(const double* __restrict__ G, const double* __
       f[c] = fabs(Ge[size_t(c) * q3 + p]) * rw3;
       bad |= !isfinite(f[c]);
     }
-    double b, d;
     if constexpr (NF == 6) {
-      b = fmax(f[0] + f[1] + f[2], fmax(f[1] + f[3] + f[4], f[2] + f[4] + f[5]));
-      d = fmax(f[0], fmax(f[3], f[5]));
+      v[0] = fmax(v[0], fmax(f[0] + f[1] + f[2], fmax(f[1] + f[3] + f[4], f[2] + f[4] + f[5])));
+      v[1] = fmin(v[1], f[0]);
+      v[2] = fmin(v[2], f[3]);
+      v[3] = fmin(v[3], f[5]);
+      v[4] = fmin(v[4], fmax(f[0], fmax(f[3], f[5])));
     } else {
-      b = d = f[0];
+      v[0] = fmax(v[0], f[0]);
+      v[1] = fmin(v[1], f[0]);
     }
-    big = fmax(big, b);
-    small = fmin(small, d);
   }
   if (bad) s_bad = 1;
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    big = fmax(big, __shfl_xor_sync(0xffffffffu, big, o));
-    small = fmin(small, __shfl_xor_sync(0xffffffffu, small, o));
-  }
-  if ((tid & 31) == 0) {
-    sred[0][tid >> 5] = big;
-    sred[1][tid >> 5] = small;
+  for (int c = 0; c < NR; ++c) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      const double x = __shfl_xor_sync(0xffffffffu, v[c], o);
+      v[c] = c == 0 ? fmax(v[c], x) : fmin(v[c], x);
+    }
+    if ((tid & 31) == 0) sred[c][tid >> 5] = v[c];
   }
   __syncthreads();
-  for (int i = 0; i < int(blockDim.x) / 32; ++i) {
-    big = fmax(big, sred[0][i]);
-    small = fmin(small, sred[1][i]);
+  for (int i = 0; i < int(blockDim.x) / 32; ++i)
+#pragma unroll
+    for (int c = 0; c < NR; ++c) v[c] = c == 0 ? fmax(v[c], sred[c][i]) : fmin(v[c], sred[c][i]);
+  const double big = v[0];
+  double carry = v[1];
+  if constexpr (NF == 6) {
+    carry = colloc ? fmax(v[1], fmax(v[2], v[3])) : v[4];
+    if (all_dirs && !(fmin(v[1], fmin(v[2], v[3])) * 16.0 >= big)) carry = 0.0;
   }
   // big chain <= 2^k: the rows of alpha G stay within 2^62
   int k = 0;
   frexp(big * ch * (1.0 + 1e-9), &k);
-  // outside the grid: not finite, spread over more than 2^7, or far from 1
-  const bool off = s_bad || !(small * 128.0 >= big) || !(big > 0.0) || k > 200 || k < -200;
+  // outside the grid: not finite, spread too far, or far from 1
+  const bool off = s_bad || !(carry * double(1 << kFxSpread) >= big) || !(big > 0.0) || k > 200 || k < -200;
   if (tid == 0) gexp[e] = off ? kFxNoGrid : k + ce;
   if (off) return;
   const double ah = scalbn(ch, 62 - k), al = scalbn(cl, 62 - k);
@@ -142,8 +163,11 @@ cudaError_t launch_fx_factors(const DeviceMesh& m, int kind, const double* G, vo
   int e = 0;
   const long double c = 2.0L * std::frexp(kind == kStiff ? m.fx->chain : m.fx->mchain, &e);  // chain = c 2^(e-1)
   const double ch = double(c), cl = double(c - ch);
-  if (kind == kStiff) fx_factors_kernel<6><<<unsigned(m.nelem), threads, 0, s>>>(G, w, m.q, ch, cl, e - 1, out, gexp);
-  else fx_factors_kernel<1><<<unsigned(m.nelem), threads, 0, s>>>(G, w, m.q, ch, cl, e - 1, out, gexp);
+  const int all_dirs = m.colloc && m.p1 <= 3;
+  if (kind == kStiff)
+    fx_factors_kernel<6><<<unsigned(m.nelem), threads, 0, s>>>(G, w, m.q, ch, cl, e - 1, m.colloc, all_dirs, out, gexp);
+  else
+    fx_factors_kernel<1><<<unsigned(m.nelem), threads, 0, s>>>(G, w, m.q, ch, cl, e - 1, m.colloc, all_dirs, out, gexp);
   return cudaGetLastError();
 }
 

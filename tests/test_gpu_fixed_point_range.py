@@ -5,8 +5,10 @@ import torch
 
 import paper_2004_06722_gb300 as pkg
 from oracle.element import element_matrices
-from oracle.quadrature import bp_rule
+from oracle.basis import lagrange_derivatives, lagrange_values
+from oracle.quadrature import bp_rule, gll
 from synth import uniform_pm1
+from tensor_reference import Element
 
 pytestmark = pytest.mark.gpu
 
@@ -40,3 +42,62 @@ def test_subnormal_elements(bp, N, k):
     assert not w[1].any()
     got = np.ldexp(w[0], -k)
     assert np.abs(got - ref).max() < (1e-2 if k == -1045 else 1e-6) * np.abs(ref).max()
+
+
+@pytest.mark.parametrize("bp,N", [(5, 1), (5, 2), (6, 1), (6, 2)])
+@pytest.mark.parametrize("aspect", [30.0, 1e2, 1e4])
+def test_thin_elements(bp, N, aspect):
+    """A function of x alone on boxes thin in z: at these orders D takes constants to exact zeros in FP64, so nothing of the small fluxes is lost (A u is a product of 1D sums, about 20 roundings)."""
+    coords, l2g, _ = pkg.mesh_box(2, 1, 1, N, 0.0)
+    coords = coords * np.array([1.0, 1.0, 1.0 / aspect])
+    op = pkg.Operator(bp, N, coords, l2g, None)
+    p1 = N + 1
+    f = np.array([0.7, -0.4, 0.9])[:p1]
+    u = np.tile(f, p1 * p1)
+    uL = np.repeat(u[None], 2, 0)
+    w = _run(op, uL if op.ncomp == 1 else np.repeat(uL[..., None], 3, -1)).reshape(2, p1 ** 3, -1)
+    pts, wq = bp_rule(bp, N)
+    J, D = lagrange_values(gll(N)[0], pts), lagrange_derivatives(gll(N)[0], pts)
+    a = 4.0 * D.T @ (wq * (D @ f))  # hx = 1/2
+    my, mz = 0.5 * J.T @ wq, 0.5 / aspect * J.T @ wq
+    ref = np.einsum("k,j,i->kji", mz, my, a).reshape(-1)
+    assert np.abs(w - ref[None, :, None]).max() < 32 * 2.0 ** -53 * np.abs(ref).max()
+
+
+def _units(bp, N, xe, u, w, kappa=None):
+    """Largest error of an entry of w in units of 2^-53 (|A| |u|)_i."""
+    el = Element(bp, N, xe, kappa)
+    err, scale = np.abs(w - el(u)), el(u, magnitudes=True)
+    assert not err[scale == 0].any()
+    return float((err[scale > 0] / scale[scale > 0]).max()) * 2.0 ** 53
+
+
+def _bound(N):
+    """About 2 p1 + 12 roundings meet on a path through the FP64 form; the 1D tables and the factors of the
+    library and of the reference differ by their own roundings, which the distances of neighbouring
+    nodes amplify (1 / 0.13 at N = 7)."""
+    return 4 * (N + 1) + 64
+
+
+def _peak(N, bits, seed):
+    """One corner value of 1, the others 2^-(bits+1) to 2^-bits with random signs."""
+    r = uniform_pm1(seed, np.arange((N + 1) ** 3))
+    u = np.ldexp(np.copysign(0.5 + 0.5 * np.abs(r), r), -bits)
+    u[0] = 1.0
+    return u
+
+
+@pytest.mark.parametrize("bp,N", [(5, 1), (5, 3), (5, 4), (5, 7), (6, 3)])
+@pytest.mark.parametrize("contrast", [1.0, 100.0, 1e5])
+def test_coefficient_spread(bp, N, contrast):
+    """kappa larger at the corner point where u is: the other entries of A u come from small values and
+    small factors alone. (On a grid of the largest factor and value, 2^-60 of the product of both ratios
+    was about 600 units at contrast 100.)"""
+    op = pkg.Operator.box(bp, 2, 1, 1, N)
+    kappa = np.ones((2, op.nquad ** 3))
+    kappa[:, 0] = contrast
+    op.set_kappa(torch.from_numpy(kappa).cuda())
+    u = np.repeat(_peak(N, 3 if contrast == 1.0 else 6, 10)[None], 2, 0)
+    w = _run(op, u if op.ncomp == 1 else np.repeat(u[..., None], 3, -1)).reshape(u.shape + (-1,))
+    for e in range(2):
+        assert _units(bp, N, op.coords[e], u[e], w[e, :, -1], kappa[e]) < _bound(N)
