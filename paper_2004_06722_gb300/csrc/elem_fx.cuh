@@ -21,7 +21,7 @@
 // current one, its u values are copied to shared memory (cp.async) once the gradient is done, and its
 // factors are prefetched into L2, so that the dependent gather overlaps a whole element's arithmetic.
 //
-// An element whose values or factors do not fit the fixed-point grid (see fx.cuh), and every element
+// An element whose values or factors do not fit the fixed-point grid or are too uneven for it (fx.cuh), and every element
 // when the context holds no fixed-point factors, runs the same stages in FP64 (a.G, with weights).
 #pragma once
 
@@ -65,8 +65,10 @@ struct FxCoShape {
   static constexpr size_t HEAD = 8 * 96 + 16 * size_t(EB);
   static constexpr size_t SMEM = HEAD + EB * SLOT;
   // Blocks per SM the registers are limited for: what shared memory holds, at 96 registers or more
-  // (p1 = 8: eight blocks, 120 registers: 350 us at E = 2^15; ten, 96 registers: 370 us).
-  static constexpr int BY_SMEM = int((size_t(227) << 10) / (SMEM + 1024)), BY_REGS = 65536 / (NT * 96);
+  // (p1 = 8: eight blocks, 120 registers: 350 us at E = 2^15; ten, 96 registers: 370 us), that is five warps
+  // on each of an SM's four partitions (N = 8, 20^3 elements, one iteration: seven blocks of three warps, 80 registers 284 us,
+  // six 272 us).
+  static constexpr int BY_SMEM = int((size_t(227) << 10) / (SMEM + 1024)), BY_REGS = 4 * (512 / 96) / (NT / 32);
   static constexpr int MINB = W == 3 ? 1 : P1 == 8 ? 8 : BY_SMEM < BY_REGS ? BY_SMEM : BY_REGS;
 };
 
@@ -81,8 +83,9 @@ struct FxCoElem {
 // Contractions and factors of one element in arithmetic Ar (FxArith or F64Arith), u in tile A.
 // factors(k, gradient, flux) multiplies by G at point k of the own column; done(shift) comes with the
 // number of bits the fluxes were moved up; out(k, r, s, t) receives the three transposes.
+// False is returned, with only the tiles overwritten, if the element turned out uneven.
 template <int P1, int W, class Ar, class Tab, class Factors, class Mid, class Done, class Out>
-__device__ __forceinline__ void fx_co_stages(const FxCoElem<P1>& el, const Tab& D, const Tab& DT, bool live,
+__device__ __forceinline__ bool fx_co_stages(const FxCoElem<P1>& el, const Tab& D, const Tab& DT, bool live,
                                              const FxNorm& norm, Factors&& factors, Mid&& mid, Done&& done, Out&& out) {
   using Sh = FxCoShape<P1, W>;
   using L = typename Ar::L;
@@ -137,7 +140,7 @@ __device__ __forceinline__ void fx_co_stages(const FxCoElem<P1>& el, const Tab& 
   }
   ar.publish(norm, 1);
   __syncthreads();
-  ar.take(norm, 1);
+  if (ar.take(norm, 1)) return false;
   done(ar.total);
   if (live) {
 #pragma unroll W == 3 ? 1 : Sh::UNROLL
@@ -158,6 +161,7 @@ __device__ __forceinline__ void fx_co_stages(const FxCoElem<P1>& el, const Tab& 
       if (W == 1 || k < P1) out(h, k, Br[own + k * PS], Cr[own + k * PS], Ar_[own + k * PS]);
     }
   }
+  return true;
 }
 
 template <int P1, int NC, bool HELM, int W>
@@ -240,15 +244,15 @@ __global__ void __launch_bounds__(FxCoShape<P1, W>::NT, FxCoShape<P1, W>::MINB)
         if (W == 1 || W * h + el.grp < P1) seen.see(el.su[(W * h + el.grp) * PP]);
       if (it + 1 < nit) load_l2g(it + 1);
     }
-    unsigned mx = seen.top();
-    mx = __reduce_max_sync(lanes, mx);
-    const int ge = live && m.gexp != nullptr ? __ldg(m.gexp + e) : kFxNoGrid;
+    const unsigned mx = __reduce_max_sync(lanes, seen.top());
+    const int code = live && m.gexp != nullptr ? __ldg(m.gexp + e) : kFxNoGrid, ge = code >> kFxReachBits;
     const FxNorm norm{lanes, lead, smax + (it & 1) * EB + (live ? slot : 0), 2 * EB};
     if (lead) atomicMax(norm.top, mx);
     __syncthreads();
     const unsigned top = live ? *norm.top : 0u;
     const int eb = top == 0u ? 1023 : int(top >> 20);  // every value is zero: any exponent
-    const bool bad = live && (ge == kFxNoGrid || eb < 500 || eb > 1500);
+    const bool bad = live && (code == kFxNoGrid || eb < 500 || eb > 1500);
+    const bool weak = live && !bad && int(seen.top()) < fx_reach_word(top, code >> 8 & 15);  // the own column
     if (el.t == 0 && el.grp == 0 && live) smax[(~it & 1) * EB + slot] = smax[(2 + (~it & 1)) * EB + slot] = 0u;
     double* wl = a.wl + size_t(e) * P3 * NC + size_t(el.t) * NC + c;
     double acc = 0.0;
@@ -260,8 +264,10 @@ __global__ void __launch_bounds__(FxCoShape<P1, W>::NT, FxCoShape<P1, W>::MINB)
         acc += w * u;
       }
     };
-    auto mid = [&]() {
-      if (live && it + 1 < nit) {
+    bool ahead = live && it + 1 < nit;
+    auto mid = [&]() {  // once, also if the element changes to FP64
+      if (ahead) {
+        ahead = false;
         if (Sh::NU == 2) fetch_u(it + 1);
         if (NC == 1 || (it + 1) % NC == 0) prefetch_G(elem_of(it + 1));
       }
@@ -272,10 +278,25 @@ __global__ void __launch_bounds__(FxCoShape<P1, W>::NT, FxCoShape<P1, W>::MINB)
       for (int h = 0; h < KC; ++h)
         if (const int k = W * h + el.grp; W == 1 || k < P1) A[k * PS] = fx_from_double(el.su[k * PP], eb);
     }
-    if (!__syncthreads_or(bad)) {
+    bool f64 = __syncthreads_or(bad);
+    if (!f64) {
+      if (weak) {  // its nodes one by one
+        const double* se = el.su - el.t;
+        bool off = false;
+#pragma unroll 1
+        for (int h = 0; h < KC; ++h) {
+          const int k = W * h + el.grp;
+          if ((W > 1 && k >= P1) || (a.skip_dirichlet_out && ((dcur >> h) & 1u))) continue;
+          off |= !fx_line_reaches<P1>(se + k * PP + el.tj * P1, 1, fx_reach_word(top, code & 15)) &&
+                 !fx_line_reaches<P1>(se + k * PP + el.ti, P1, fx_reach_word(top, code >> 4 & 15)) &&
+                 !(W > 1 && fx_line_reaches<P1>(el.su, PP, fx_reach_word(top, code >> 8 & 15)));
+        }
+        if (off)
+          for (int s = 0; s < EB; ++s) atomicMax(smax + (2 + (it & 1)) * EB + s, kFxUneven);
+      }
       const int4* G = m.Gfx + e * 3 * P3 + el.t;
       double sc = 0.0;
-      fx_co_stages<P1, W, FxArith>(
+      f64 = !fx_co_stages<P1, W, FxArith>(
           el, tab.D, tab.DT, live, norm,
           [&](int k, int2 r, int2 s, int2 t, long long& fr, long long& fs, long long& ft) {
             const int4 g0 = __ldcs(G + (3 * k + 0) * PP), g1 = __ldcs(G + (3 * k + 1) * PP),
@@ -291,7 +312,8 @@ __global__ void __launch_bounds__(FxCoShape<P1, W>::NT, FxCoShape<P1, W>::MINB)
           [&](int h, int k, long long r, long long s, long long t) {
             finish(h, k, __ll2double_rn(r + s + t) * (tab.w[k] * sc));
           });
-    } else {
+    }
+    if (f64) {
       if (live) {
         double* A = static_cast<double*>(el.A) + el.tj * S + el.ti;
 #pragma unroll

@@ -68,12 +68,13 @@ struct FxGlShape {
 // One element in arithmetic Ar, u in tile A.  factors: gradient to flux at point z of the own column, or
 // value to value with the mass factors; add(z, v, u) sees the summed transposes (Helmholtz); done(shift)
 // comes with the number of bits the values were moved up; out(i, y) turns the nodal results of line
-// (j, k) = t into FP64, left in tile A.
-template <int P1, int KIND, bool HELM, class Ar, class TJ, class TJT, class TD, class Factors, class Mid, class Add,
-          class Done, class Out>
-__device__ __forceinline__ void fx_gl_stages(void* tiles, int t, bool live, const TJ& J, const TJT& JT, const TD& D,
-                                             const TD& DT, const FxNorm& norm, Factors&& factors, Mid&& mid,
-                                             Add&& add, Done&& done, Out&& out) {
+// (j, k) = t into FP64, left in tile A.  weak(l) sees the values of line (j, k); if it
+// is, uneven() may set the first stage's word to kFxUneven: false is then returned, with only the tiles overwritten.
+template <int P1, int KIND, bool HELM, class Ar, class TJ, class TJT, class TD, class Weak, class Uneven, class Factors,
+          class Mid, class Add, class Done, class Out>
+__device__ __forceinline__ bool fx_gl_stages(void* tiles, int t, bool live, const TJ& J, const TJT& JT, const TD& D,
+                                             const TD& DT, const FxNorm& norm, Weak&& weak, Uneven&& uneven, Factors&& factors,
+                                             Mid&& mid, Add&& add, Done&& done, Out&& out) {
   using Sh = FxGlShape<P1, KIND>;
   using L = typename Ar::L;
   using Raw = typename Ar::Raw;
@@ -86,13 +87,16 @@ __device__ __forceinline__ void fx_gl_stages(void* tiles, int t, bool live, cons
   const int yb = tj * PS + ti;                  // line (q_x, k) = (ti, tj), step S
   const bool xl = live && t < P1 * P1, yl = live && t < Q * P1;
   Ar ar;
+  bool off = false;
   if (xl) {
     L l[P1];
 #pragma unroll
     for (int n = 0; n < P1; ++n) l[n] = A[xb + n];
+    off = weak(l);
     eo_line<Ar::kBias, P1, Q, false>(J, l, [&](int n, auto y) { A[xb + n] = Ar::limbs(y); });
   }
   __syncthreads();
+  if (off) uneven();
   if (yl) {
     L l[P1];
 #pragma unroll
@@ -117,7 +121,7 @@ __device__ __forceinline__ void fx_gl_stages(void* tiles, int t, bool live, cons
     const int rb = tj * PS + ti * S;  // r: line (q_y, z) = (ti, tj), step 1;  s: line (q_x, z) = (ti, tj), step S
     ar.publish(norm, 1);
     __syncthreads();
-    ar.take(norm, 1);
+    if (ar.take(norm, 1)) return false;
 #pragma unroll Sh::UNROLL
     for (int dir = 0; dir < 3; ++dir) {
       if (dir == 2) __syncthreads();  // r and s have read tile A: t goes in place
@@ -183,7 +187,7 @@ __device__ __forceinline__ void fx_gl_stages(void* tiles, int t, bool live, cons
   }
   ar.publish(norm, 3);
   __syncthreads();
-  ar.take(norm, 3);
+  if (ar.take(norm, 3) && KIND == kMass) return false;
   done(ar.total);
   if (live) {
     L l[Q];
@@ -207,6 +211,7 @@ __device__ __forceinline__ void fx_gl_stages(void* tiles, int t, bool live, cons
     eo_line<0, Q, P1, false>(JT, l, [&](int n, auto y) { W[n] = out(n, y); });
   }
   __syncthreads();
+  return true;
 }
 
 // PAIR: u and w^e are FP32 pairs (df.cuh; u may be FP64 as well), converted in shared memory.
@@ -295,18 +300,19 @@ __global__ void __launch_bounds__(FxGlShape<P1, KIND>::NT, FxGlShape<P1, KIND>::
         if (has(n)) seen.see(su[t + n * QQ]);
       if (it + 1 < nit) load_l2g(it + 1);
     }
-    unsigned mx = seen.top();
-    mx = __reduce_max_sync(lanes, mx);
-    const int ge = !HELM && live && fxe != nullptr ? __ldg(fxe + e) : kFxNoGrid;
+    const unsigned mx = __reduce_max_sync(lanes, seen.top());
+    const int code = !HELM && live && fxe != nullptr ? __ldg(fxe + e) : kFxNoGrid, ge = code >> kFxReachBits;
     const FxNorm norm{lanes, lead, smax + (it & 1) * EB + (live ? slot : 0), 2 * EB};
     if (lead) atomicMax(norm.top, mx);
     __syncthreads();
     const unsigned top = live ? *norm.top : 0u;
     const int eb = top == 0u ? 1023 : int(top >> 20);  // every value is zero: any exponent
-    const bool bad = live && (ge == kFxNoGrid || eb < 500 || eb > 1500);
+    const bool bad = live && (code == kFxNoGrid || eb < 500 || eb > 1500);
     if (t < 4 && live) smax[(2 * t + (~it & 1)) * EB + slot] = 0u;
-    auto mid = [&]() {
-      if (live && it + 1 < nit) {
+    bool ahead = live && it + 1 < nit;
+    auto mid = [&]() {  // once, also if the element changes to FP64
+      if (ahead) {
+        ahead = false;
         if (Sh::NU == 2) fetch_u(it + 1);
         if (NC == 1 || (it + 1) % NC == 0) prefetch_factors(elem_of(it + 1));
       }
@@ -316,17 +322,40 @@ __global__ void __launch_bounds__(FxGlShape<P1, KIND>::NT, FxGlShape<P1, KIND>::
       for (int n = 0; n < NPT; ++n)
         if (has(n)) reinterpret_cast<int2*>(tiles)[place(t + n * QQ)] = fx_from_double(su[t + n * QQ], eb);
     }
-    const bool f64 = __syncthreads_or(bad);
-    if (!HELM && !f64) {
-      if constexpr (!HELM) {
+    bool f64 = __syncthreads_or(bad);
+    if constexpr (!HELM) {
+      if (!f64) {
         double sc = 0.0;
+        // a line (j, k) below the limb of the smallest value that reaches, and its nodes one by one. Pairs carry 47
+        // bits: they keep theirs at ratios up to 2^10 larger.
+        const int reach = PAIR ? min((code & 15) + 10, 15) : code & 15;
+        auto weak = [&](const int2(&l)[P1]) {
+          int hi = 0, lo = 0;
+#pragma unroll
+          for (int n = 0; n < P1; ++n) {
+            hi = max(hi, l[n].x);
+            lo = min(lo, l[n].x);
+          }
+          return max(hi, ~lo) < int(((top & 0xfffffu) | 0x100000u) << 8 >> reach);
+        };
+        auto uneven = [&]() {
+          const int j = t % P1, k = t / P1, word = fx_reach_word(top, reach);
+          bool off = false;
+#pragma unroll 1
+          for (int i = 0; i < P1; ++i)
+            off |= !fx_line_reaches<P1>(su + k * P1 * P1 + i, P1, word) &&
+                   !fx_line_reaches<P1>(su + j * P1 + i, P1 * P1, word) &&
+                   !(a.skip_dirichlet_out && __ldg(m.l2g + e * P3 + t * P1 + i) < 0);
+          if (off)
+            for (int s = 0; s < EB; ++s) atomicMax(smax + ((KIND == kStiff ? 2 : 6) + (it & 1)) * EB + s, kFxUneven);
+        };
         auto done = [&](int shift) { sc = wjk * __hiloint2double((eb + ge - shift - (1082 - 1023)) << 20, 0); };
         auto out = [&](int i, long long y) { return __ll2double_rn(y) * (tab.w[i] * sc); };
         auto add = [](int, long long v, double) { return v; };
         if constexpr (KIND == kStiff) {
           const int4* G = m.Gfx + e * 3 * Q3 + t;
-          fx_gl_stages<P1, KIND, false, FxArith>(
-              tiles, t, live, tab.J, tab.JT, tab.D, tab.DT, norm,
+          f64 = !fx_gl_stages<P1, KIND, false, FxArith>(
+              tiles, t, live, tab.J, tab.JT, tab.D, tab.DT, norm, weak, uneven,
               [&](int z, int2 r, int2 s, int2 tt, long long& fr, long long& fs, long long& ft) {
                 const int4 g0 = __ldcs(G + (3 * z + 0) * QQ), g1 = __ldcs(G + (3 * z + 1) * QQ),
                            g2 = __ldcs(G + (3 * z + 2) * QQ);
@@ -339,8 +368,8 @@ __global__ void __launch_bounds__(FxGlShape<P1, KIND>::NT, FxGlShape<P1, KIND>::
               mid, add, done, out);
         } else {
           const int2* M = m.Mfx + e * Q3 + t;
-          fx_gl_stages<P1, KIND, false, FxArith>(
-              tiles, t, live, tab.J, tab.JT, tab.D, tab.DT, norm,
+          f64 = !fx_gl_stages<P1, KIND, false, FxArith>(
+              tiles, t, live, tab.J, tab.JT, tab.D, tab.DT, norm, weak, uneven,
               [&](int z, int2 v) {
                 const int2 f = __ldcs(M + z * QQ);
                 long long mm = fx_mad(f.x, v.y, kFxRound);
@@ -350,7 +379,8 @@ __global__ void __launch_bounds__(FxGlShape<P1, KIND>::NT, FxGlShape<P1, KIND>::
               mid, add, done, out);
         }
       }
-    } else {
+    }
+    if (HELM || f64) {
       if (live) {
 #pragma unroll
         for (int n = 0; n < NPT; ++n)
@@ -360,10 +390,12 @@ __global__ void __launch_bounds__(FxGlShape<P1, KIND>::NT, FxGlShape<P1, KIND>::
       auto done = [](int) {};
       auto add = [&](int z, double v, double u) { return v + a.beta * __ldg(a.Mq + e * Q3 + z * QQ + t) * u; };
       auto out = [](int, double y) { return y; };
+      auto weak = [](const double(&)[P1]) { return false; };
+      auto uneven = []() {};
       const double* G = a.G + e * NF * Q3 + t;
       if constexpr (KIND == kStiff) {
         fx_gl_stages<P1, KIND, HELM, F64Arith>(
-            tiles, t, live, tab.J64, tab.JT64, tab.D64, tab.DT64, norm,
+            tiles, t, live, tab.J64, tab.JT64, tab.D64, tab.DT64, norm, weak, uneven,
             [&](int z, double r, double s, double tt, double& fr, double& fs, double& ft) {
               const double* Gz = G + z * QQ;
               const double g00 = __ldcs(Gz), g01 = __ldcs(Gz + Q3), g02 = __ldcs(Gz + 2 * Q3), g11 = __ldcs(Gz + 3 * Q3),
@@ -375,7 +407,7 @@ __global__ void __launch_bounds__(FxGlShape<P1, KIND>::NT, FxGlShape<P1, KIND>::
             mid, add, done, out);
       } else {
         fx_gl_stages<P1, KIND, HELM, F64Arith>(
-            tiles, t, live, tab.J64, tab.JT64, tab.D64, tab.DT64, norm,
+            tiles, t, live, tab.J64, tab.JT64, tab.D64, tab.DT64, norm, weak, uneven,
             [&](int z, double v) { return __ldcs(G + z * QQ) * v; }, mid, add, done, out);
       }
     }

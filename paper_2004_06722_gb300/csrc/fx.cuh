@@ -168,6 +168,34 @@ struct FxTop {
   __device__ __forceinline__ unsigned top() const { return max(hi, min(lo, 1u)); }
 };
 
+// Uneven elements.  One unit of a stage is 2^-60 of the element's largest values, so a small entry of the
+// result is as accurate as FP64's only while something of that size takes part in it: FP64's error is
+// proportional to (|A| |u|)_i.  Every node is therefore asked for one of the three lines of nodes through it whose
+// largest value reaches 2^-r of the element's (r from its factors, fx_setup.cu); an element with a node
+// that has none (single peaks, values that fall by orders of magnitude) runs in FP64.  Nodes of the Dirichlet boundary
+// whose results nobody reads are not asked.  With that every entry is within a few units of
+// 2^-53 (|A| |u|)_i, as in FP64; without it the error was 2^-60 of the largest entry's scale.
+
+// The word of a stage's largest magnitude that says so: the check needs no barrier of its own.  What it costs
+// elements that are even: 1.4 % of a BP5 iteration at N = 7, 4 % of BP3's.
+constexpr unsigned kFxUneven = 0x80000000u;
+
+// The smallest upper word that reaches (any value of an element of zeros).
+__device__ __forceinline__ int fx_reach_word(unsigned top, int r) {
+  return r == 0 ? 0x7fffffff : max(int(top) - (r << 20), 0);
+}
+
+// Whether one of the N values of a line reaches (the middle one first: most lines are answered by it).
+template <int N>
+__device__ __forceinline__ bool fx_line_reaches(const double* line, int step, int word) {
+  auto at = [&](int n) { return __double2hiint(line[n * step]) & 0x7fffffff; };
+  if (at(N / 2) >= word) return true;
+  int t = 0;
+#pragma unroll 4
+  for (int n = 0; n < N; ++n) t = max(t, at(n));
+  return t >= word;
+}
+
 // Where the threads of an element exchange the largest magnitude of a stage's values: one word for each
 // stage, `step` words apart.
 struct FxNorm {
@@ -179,7 +207,8 @@ struct FxNorm {
 
 // The two arithmetics of the element kernels: L a stage's input, Raw its output.  see() collects the
 // magnitudes (by upper words) of raw values that the next stage reads with load(); publish() before and
-// take() after a barrier turn the element's largest into the shift that moves it up to 2^60.
+// take() after a barrier turn the element's largest into the shift that moves it up to 2^60.  take() is true
+// if the word says that the block's elements are to run in FP64 (kFxUneven, larger than any magnitude).
 struct FxArith {
   using L = int2;
   using Raw = long long;
@@ -199,10 +228,12 @@ struct FxArith {
     if (n.lead) atomicMax(n.top + stage * n.step, t);
     hi = lo = 0;
   }
-  __device__ __forceinline__ void take(const FxNorm& n, int stage) {
-    shift = min(max(__clz(int(n.top[stage * n.step])) - 4, 0), 30);
+  __device__ __forceinline__ bool take(const FxNorm& n, int stage) {
+    const unsigned t = n.top[stage * n.step];
+    shift = min(max(__clz(int(t)) - 4, 0), 30);
     total += shift;
     bias = kFxHalf >> shift;
+    return t >= kFxUneven;
   }
 };
 struct F64Arith {
@@ -214,7 +245,7 @@ struct F64Arith {
   __device__ __forceinline__ L load(Raw y) const { return y; }
   __device__ __forceinline__ void see(Raw) {}
   __device__ __forceinline__ void publish(const FxNorm&, int) {}
-  __device__ __forceinline__ void take(const FxNorm&, int) {}
+  __device__ __forceinline__ bool take(const FxNorm&, int) { return false; }
 };
 
 // asynchronous copy of one double, or of zero

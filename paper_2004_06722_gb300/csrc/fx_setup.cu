@@ -70,11 +70,23 @@ __device__ __forceinline__ int2 fx_factor(double g, double w3, double rw3, doubl
 // weak direction of a thin element, the grid the ratio of the factors: all three directions (all_dirs) have to
 // be within 2^4 there (order 1, thickness 1/100, a function of x: 2e-14 of the result against 3e-17; from order 3
 // on, and with Gauss quadrature, both arithmetics lose the same).
+//
+// reach: a line of nodal values counts as large while it is above 2^-reach of the element's largest value (fx.cuh).
+// The ratio of the factors takes from it; the budget of `reach` bits at ratios below 2 grows at low orders, whose
+// row sums are small (fixed point against FP64, worst entry in units of 2^-53 (|A||u|)_i, one node 2^6
+// above the others: order 1 0.7 / 0.8, 2 2.4 / 0.9, 3 2.6 / 1.9, 5 6.4 / 2.5, 7 8.4 / 5.2, 15 20 / 7.5; 2^4: order 5 and up
+// within 1.1 of FP64).
 constexpr int kFxSpread = 5;
+__device__ __forceinline__ int fx_reach(double big, double small, int budget) {
+  if (!(small * double(1 << kFxSpread) >= big)) return 0;
+  int s = 0;
+  frexp(big / small, &s);  // the ratio is in [2^(s-1), 2^s)
+  return max(budget + 1 - s, 0);
+}
 
 template <int NF>
 __global__ void fx_factors_kernel(const double* __restrict__ G, const double* __restrict__ w, int q, double ch,
-                                  double cl, int ce, int colloc, int all_dirs, void* out, int* __restrict__ gexp) {
+                                  double cl, int ce, int colloc, int all_dirs, int budget, void* out, int* __restrict__ gexp) {
   constexpr int NR = NF == 6 ? 5 : 2;  // largest row sum; smallest of each direction and of the points' largest
   __shared__ double sw[kMaxQ], srw[kMaxQ], sred[NR][32];
   __shared__ int s_bad;
@@ -127,17 +139,20 @@ __global__ void fx_factors_kernel(const double* __restrict__ G, const double* __
 #pragma unroll
     for (int c = 0; c < NR; ++c) v[c] = c == 0 ? fmax(v[c], sred[c][i]) : fmin(v[c], sred[c][i]);
   const double big = v[0];
-  double carry = v[1];
-  if constexpr (NF == 6) {
-    carry = colloc ? fmax(v[1], fmax(v[2], v[3])) : v[4];
-    if (all_dirs && !(fmin(v[1], fmin(v[2], v[3])) * 16.0 >= big)) carry = 0.0;
+  int reach = 0;
+  if (NF == 6 && colloc) {
+    if (!all_dirs || fmin(v[1], fmin(v[2], v[3])) * 16.0 >= big)
+#pragma unroll
+      for (int d = 0; d < 3; ++d) reach |= fx_reach(big, v[1 + d], budget) << 4 * d;
+  } else {
+    reach = fx_reach(big, v[NR - 1], budget);
   }
   // big chain <= 2^k: the rows of alpha G stay within 2^62
   int k = 0;
   frexp(big * ch * (1.0 + 1e-9), &k);
   // outside the grid: not finite, spread too far, or far from 1
-  const bool off = s_bad || !(carry * double(1 << kFxSpread) >= big) || !(big > 0.0) || k > 200 || k < -200;
-  if (tid == 0) gexp[e] = off ? kFxNoGrid : k + ce;
+  const bool off = s_bad || reach == 0 || !(big > 0.0) || k > 200 || k < -200;
+  if (tid == 0) gexp[e] = off ? kFxNoGrid : (k + ce) * (1 << kFxReachBits) + reach;
   if (off) return;
   const double ah = scalbn(ch, 62 - k), al = scalbn(cl, 62 - k);
   for (int p = tid; p < q3; p += blockDim.x) {
@@ -163,11 +178,11 @@ cudaError_t launch_fx_factors(const DeviceMesh& m, int kind, const double* G, vo
   int e = 0;
   const long double c = 2.0L * std::frexp(kind == kStiff ? m.fx->chain : m.fx->mchain, &e);  // chain = c 2^(e-1)
   const double ch = double(c), cl = double(c - ch);
-  const int all_dirs = m.colloc && m.p1 <= 3;
+  const int all_dirs = m.colloc && m.p1 <= 3, budget = m.p1 <= 4 ? 10 - m.p1 : 5;
   if (kind == kStiff)
-    fx_factors_kernel<6><<<unsigned(m.nelem), threads, 0, s>>>(G, w, m.q, ch, cl, e - 1, m.colloc, all_dirs, out, gexp);
+    fx_factors_kernel<6><<<unsigned(m.nelem), threads, 0, s>>>(G, w, m.q, ch, cl, e - 1, m.colloc, all_dirs, budget, out, gexp);
   else
-    fx_factors_kernel<1><<<unsigned(m.nelem), threads, 0, s>>>(G, w, m.q, ch, cl, e - 1, m.colloc, all_dirs, out, gexp);
+    fx_factors_kernel<1><<<unsigned(m.nelem), threads, 0, s>>>(G, w, m.q, ch, cl, e - 1, m.colloc, all_dirs, budget, out, gexp);
   return cudaGetLastError();
 }
 

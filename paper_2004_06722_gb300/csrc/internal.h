@@ -42,9 +42,12 @@ struct FxTables {
   long double chain = 1.0L, mchain = 1.0L;
 };
 
-// Exponent of an element whose factors do not fit the fixed-point grid.
+// Word of an element of fixed-point factors: its exponent above kFxReachBits bits of how far below the
+// element's largest value a line of values may lie (fx_even in fx.cuh), four bits each: collocated one for
+// lines of each direction (0: lines of this direction do not count), Gauss quadrature one for all lines.
+constexpr int kFxReachBits = 12;
+// ... of an element whose factors do not fit the fixed-point grid.
 constexpr int kFxNoGrid = -(1 << 30);
-struct Basis1D;
 void build_fx_tables(const Basis1D& b, FxTables* t);
 
 // Entries behind the last list of `slots` that the gather may read (gather.cuh).
@@ -107,7 +110,7 @@ struct DeviceMesh {
   int tune_ns;          // elements per slot sequence of the pipelined schedule
   const FxTables* fx;   // host: tables of the fixed-point kernels
   const int4* Gfx;      // fixed-point stiffness factors [E][q][3][q^2], or nullptr (FP64 form)
-  const int* gexp;      // [E] exponent of the element's fixed-point result (kFxNoGrid: it runs in FP64)
+  const int* gexp;      // [E] exponent and reaches of the element (kFxNoGrid: it runs in FP64)
   const int2* Mfx;      // fixed-point mass factors [E][q^3] of Gauss quadrature, or nullptr
   const int* mexp;      // [E] as gexp
   const double* X;      // [E][3][p1^3] nodal coordinates when the factors are recomputed, else nullptr

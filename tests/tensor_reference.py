@@ -1,6 +1,7 @@
 """One element's operator by 1D products (interpolate, differentiate, factors, transposes) in a chosen
 precision, and the same with every table, factor and value replaced by its magnitude: the scale
-|A^e| |u| that rounding errors of a componentwise stable evaluation are proportional to."""
+|A^e| |u| that rounding errors of a componentwise stable evaluation are proportional to.  Off-diagonal
+factors are differences of products and known to the rounding of the diagonal ones, which stand in for them."""
 import numpy as np
 
 from oracle.basis import lagrange_derivatives, lagrange_values
@@ -53,6 +54,7 @@ class Element:
             out = f(self.B) * v
         else:
             g = _dx(D, v)
-            flux = [sum(f(self.G[a][b]) * g[b] for b in range(3)) for a in range(3)]
+            G = [[self.G[a][a] + self.G[b][b] if magnitudes and a != b else self.G[a][b] for b in range(3)] for a in range(3)]
+            flux = [sum(f(G[a][b]) * g[b] for b in range(3)) for a in range(3)]
             out = sum(_along(D.T, flux[a], 2 - a) for a in range(3))
         return (out if J is None else _all(J.T, out)).reshape(-1)

@@ -101,3 +101,57 @@ def test_coefficient_spread(bp, N, contrast):
     w = _run(op, u if op.ncomp == 1 else np.repeat(u[..., None], 3, -1)).reshape(u.shape + (-1,))
     for e in range(2):
         assert _units(bp, N, op.coords[e], u[e], w[e, :, -1], kappa[e]) < _bound(N)
+
+
+def _uneven(kind, N, seed):
+    p1 = N + 1
+    k, j, i = np.meshgrid(*[np.arange(p1)] * 3, indexing="ij")
+    if kind.startswith("peak"):
+        return _peak(N, int(kind[4:]), seed)
+    if kind == "inner":  # the peak inside, on the longest list of neighbours
+        u = _peak(N, 24, seed)
+        u[0], u[u.size // 2] = u[1], 1.0
+        return u
+    if kind == "decay":
+        return np.ldexp(1.0 - 0.25 * uniform_pm1(seed, np.arange(p1 ** 3)), -3 * (i + j + k).reshape(-1))
+    if kind == "unit":
+        u = np.zeros(p1 ** 3)
+        u[p1 ** 3 // 3] = 1.0
+        return u
+    if kind == "plane":  # one large plane of nodes: every line across it is large, those along it are not
+        return np.where(j == p1 - 1, 1.0, 2.0 ** -30).reshape(-1) * uniform_pm1(seed, np.arange(p1 ** 3))
+    return uniform_pm1(seed, np.arange(p1 ** 3))
+
+
+@pytest.mark.parametrize("bp,N", [(5, 1), (5, 2), (5, 4), (5, 5), (5, 7), (6, 3), (1, 1), (1, 3), (2, 3), (3, 1), (3, 2), (3, 5),
+                                  (3, 7), (4, 3)])
+@pytest.mark.parametrize("kind", ["random", "peak4", "peak12", "peak40", "inner", "decay", "unit", "plane"])
+def test_uneven_values(bp, N, kind):
+    """Every entry of A u to within a few units of 2^-53 (|A| |u|)_i, however the values of the element are spread."""
+    op = pkg.Operator.box(bp, 3, 1, 1, N)
+    u = np.stack([_uneven(kind, N, 11), uniform_pm1(12, np.arange((N + 1) ** 3)), _uneven(kind, N, 13)])
+    u[2] = np.ldexp(u[2], -40)
+    w = _run(op, u if op.ncomp == 1 else np.stack([u, u[::-1], u], -1)).reshape(u.shape + (-1,))
+    for e in range(3):
+        assert _units(bp, N, op.coords[e], u[e], w[e, :, -1]) < _bound(N)
+
+
+@pytest.mark.parametrize("bp,N", [(5, 3), (5, 7), (5, 11), (3, 4), (6, 5)])
+def test_uneven_values_beside_the_boundary(bp, N):
+    """Rows of A u next to Dirichlet faces, edges and corners, where whole lines are masked to zero."""
+    op = pkg.Operator.box(bp, 2, 2, 2, N)
+    coords, l2g, dirichlet = pkg.mesh_box(2, 2, 2, N, 0.05)
+    n = dirichlet.shape[0]
+    for drop in (0, 30):
+        u = uniform_pm1(14, np.arange(n))
+        u = np.where(np.arange(n) % 3 == 0, u, np.ldexp(u, -drop)) * (1 - dirichlet)
+        w = op.apply(torch.from_numpy(u if op.ncomp == 1 else np.stack([u] * 3, -1)).cuda()).cpu().numpy().reshape(n, -1)[:, -1]
+        ref, scale = np.zeros(n, np.longdouble), np.zeros(n, np.longdouble)
+        for e in range(8):
+            el = Element(bp, N, coords[e])
+            np.add.at(ref, l2g[e], el(u[l2g[e]]))
+            np.add.at(scale, l2g[e], el(u[l2g[e]], magnitudes=True))
+        free = dirichlet == 0
+        assert np.abs(w[free] - ref[free]).max() < 1.0
+        units = float((np.abs(w[free] - ref[free]) / scale[free]).max()) * 2.0 ** 53
+        assert units < _bound(min(N, 7)) * (4 if N > 7 else 1)
