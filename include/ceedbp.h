@@ -64,8 +64,11 @@ typedef enum {
 
 /* Arithmetic of the FP64 operator and solver (ceedbp_params.arith). */
 enum {
-  CEEDBP_ARITH_FP64 = 0, /* FP64 in and out; contractions on 60-bit integers per element with
-                            the accuracy of FP64 (batched solves: FP64 instructions) */
+  CEEDBP_ARITH_FP64 = 0, /* FP64 in and out; contractions on 60-bit integers on a grid of each
+                            element, in FP64 where an element's values or factors are too
+                            uneven for it: every entry of A_e u_e is within a few units of
+                            2^-53 (|A_e| |u_e|)_i either way.  ceedbp_set_fixed_point(ctx, 0)
+                            runs everything in FP64; batched solves always do. */
   CEEDBP_ARITH_DF64 = 1  /* FP64-accurate pairs of FP32 numbers (hi + lo, ~2^-46 relative per
                             value) on the FP32 pipe, which the GB300 issues 63x faster than
                             FP64; BP1, BP3, BP5 and BP6 (EUNSUPPORTED for BP2 and BP4).
@@ -304,6 +307,22 @@ ceedbp_status ceedbp_batch_solve(ceedbp_batch* batch, const double* const* b_dev
                                  const ceedbp_solve_opts* opts, ceedbp_solve_info* infos);
 ceedbp_status ceedbp_batch_destroy(ceedbp_batch* batch);
 const char* ceedbp_batch_last_error(const ceedbp_batch* batch);
+
+/*
+ * Fixed-point factors of CEEDBP_ARITH_FP64 contexts with stored factors, and of
+ * BP1/BP3 with CEEDBP_ARITH_DF64 (CEEDBP_EUNSUPPORTED for other contexts).
+ * Setup makes them, in addition to the factors and as large as those, while
+ * they take at most a quarter of the device's memory (pairs: at any size);
+ * where they do not fit, at setup or beside the memory of a later call, the context goes on without them.
+ * on = 0 gives them back: every element then runs in FP64 instructions (about a
+ * third of the speed).  on = 1 makes them again (CEEDBP_ENOMEM if they do not
+ * fit).  Either synchronises the stream and drops the context's captured
+ * graphs when something changes.
+ */
+ceedbp_status ceedbp_set_fixed_point(ceedbp_ctx* ctx, int on);
+
+/* *on = 1 while the context holds fixed-point factors, else 0. */
+ceedbp_status ceedbp_fixed_point(const ceedbp_ctx* ctx, int* on);
 
 /*
  * Helmholtz operator H = A + beta B of Eq. (17) (the equation of Eq. (4) with

@@ -76,6 +76,8 @@ _SIGS = {
     "ceedbp_bk_apply": (ctypes.c_int, [_P, _P, _P]),
     "ceedbp_set_helmholtz": (ctypes.c_int, [_P, ctypes.c_double]),
     "ceedbp_set_tile": (ctypes.c_int, [_P, ctypes.c_int, ctypes.c_int, ctypes.c_int]),
+    "ceedbp_set_fixed_point": (ctypes.c_int, [_P, ctypes.c_int]),
+    "ceedbp_fixed_point": (ctypes.c_int, [_P, ctypes.POINTER(ctypes.c_int)]),
     "ceedbp_check": (ctypes.c_int, [_P]),
     "ceedbp_fma_peak": (ctypes.c_int, [ctypes.c_int, ctypes.POINTER(ctypes.c_double), ctypes.POINTER(ctypes.c_int)]),
     "ceedbp_mma_peak": (ctypes.c_int, [ctypes.c_int, ctypes.POINTER(ctypes.c_double)]),
@@ -327,6 +329,17 @@ class Operator:
     def set_helmholtz(self, beta: float):
         """Use H = A + beta B (Eq. (17)) in apply, bk_apply and solve; beta = 0 restores A."""
         _check(self._call(self.lib.ceedbp_set_helmholtz, ctypes.c_double(beta)), self.ctx)
+
+    @property
+    def fixed_point(self) -> bool:
+        """Whether the operator holds fixed-point factors; without them every element runs in FP64."""
+        on = ctypes.c_int(0)
+        _check(self.lib.ceedbp_fixed_point(self.ctx, ctypes.byref(on)), self.ctx)
+        return bool(on.value)
+
+    def set_fixed_point(self, on: bool):
+        """Give the fixed-point factors back (and their memory), or make them again."""
+        _check(self._call(self.lib.ceedbp_set_fixed_point, int(bool(on))), self.ctx)
 
     def set_tile(self, elems_per_block: int, schedule: int, seq: int = 1):
         """Pin the pair kernel's shape to one the autotuner times (see tile_info)."""

@@ -95,25 +95,42 @@ void release(ceedbp_ctx* c) {
   c->prof.clear();
 }
 
+// Whether the context's element kernels take fixed-point factors.
+bool fx_context(const ceedbp_ctx* c) {
+  return (c->arith == CEEDBP_ARITH_FP64 || !c->colloc) && c->d_X == nullptr && !c->batch_group;
+}
+
+// Gives the fixed-point factors back: every element then runs in FP64.
+void drop_fx(ceedbp_ctx* c) {
+  DeviceMesh& m = c->mesh;
+  cudaStreamSynchronize(c->stream);
+  for (auto& g : c->graphs) cudaGraphExecDestroy(g.exec);  // captured launches hold the factors
+  c->graphs.clear();
+  void* ptrs[] = {c->d_Gfx, c->d_gexp, c->d_Mfx, c->d_mexp};
+  for (void* p : ptrs)
+    if (p) cudaFree(p);
+  m.Gfx = c->d_Gfx = nullptr;
+  m.gexp = c->d_gexp = nullptr;
+  m.Mfx = c->d_Mfx = nullptr;
+  m.mexp = c->d_mexp = nullptr;
+}
+
 // Fixed-point copies of the stiffness factors and, with Gauss quadrature, the mass factors for the FP64
-// element kernels (elem_fx.cuh, elem_fxgl.cuh) and the pair arithmetic of BP1/BP3: as large as the factors
-// themselves, so with FP64 arithmetic they are kept only while they take at most a quarter of the free
-// memory; without them the kernels run in FP64.
+// element kernels (elem_fx.cuh, elem_fxgl.cuh) and the pair arithmetic of BP1/BP3, as large as the factors
+// themselves. All of them or, with ENOMEM, none.
 ceedbp_status prepare_fx(ceedbp_ctx* c) {
   DeviceMesh& m = c->mesh;
   const size_t nq = size_t(m.nelem) * c->q * c->q * c->q;
   const bool stiff = c->op_kind == kStiff, mass = !c->colloc;
-  size_t free_b = 0, total_b = 0;
-  CK(c, cudaMemGetInfo(&free_b, &total_b));
-  if (c->arith == CEEDBP_ARITH_FP64 && nq * (stiff * 3 * sizeof(int4) + mass * sizeof(int2)) > free_b / 4) return CEEDBP_OK;
   cudaError_t e = cudaSuccess;
   if (stiff) e = dalloc(&c->d_Gfx, 3 * nq);
   if (stiff && e == cudaSuccess) e = dalloc(&c->d_gexp, size_t(m.nelem));
   if (mass && e == cudaSuccess) e = dalloc(&c->d_Mfx, nq);
   if (mass && e == cudaSuccess) e = dalloc(&c->d_mexp, size_t(m.nelem));
   if (e != cudaSuccess) {
-    cudaGetLastError();  // out of memory: run in FP64
-    return CEEDBP_OK;
+    cudaGetLastError();
+    drop_fx(c);
+    return cuda_fail(c, e, "fixed-point factors");
   }
   if (stiff) {
     CK(c, launch_fx_factors(m, kStiff, c->d_G, c->d_Gfx, c->d_gexp, c->stream));
@@ -126,6 +143,34 @@ ceedbp_status prepare_fx(ceedbp_ctx* c) {
     m.mexp = c->d_mexp;
   }
   return CEEDBP_OK;
+}
+
+// Setup keeps fixed-point factors of at most a quarter of the device's memory (pairs: of any size, in the
+// place of pair copies of the factors), whatever else is
+// allocated at the moment, so that equal setups give equal bits; only where they no longer fit does the
+// context run in FP64 (ceedbp_fixed_point tells).
+ceedbp_status setup_fx(ceedbp_ctx* c) {
+  const size_t nq = size_t(c->mesh.nelem) * c->q * c->q * c->q;
+  size_t free_b = 0, total_b = 0;
+  CK(c, cudaMemGetInfo(&free_b, &total_b));
+  const size_t bytes = nq * ((c->op_kind == kStiff) * 3 * sizeof(int4) + !c->colloc * sizeof(int2));
+  if (c->arith == CEEDBP_ARITH_FP64 && bytes > total_b / 4) return CEEDBP_OK;
+  const ceedbp_status st = prepare_fx(c);
+  if (st != CEEDBP_ENOMEM) return st;
+  c->err.clear();
+  return CEEDBP_OK;
+}
+
+// Memory for a call after setup; the fixed-point factors make room for it.
+template <typename T>
+cudaError_t alloc_late(ceedbp_ctx* c, T** p, size_t count) {
+  cudaError_t e = dalloc(p, count);
+  if (e == cudaErrorMemoryAllocation && (c->d_Gfx || c->d_Mfx)) {
+    cudaGetLastError();
+    drop_fx(c);
+    e = dalloc(p, count);
+  }
+  return e;
 }
 
 ceedbp_status setup_impl(ceedbp_ctx* c, const double* coords, const int64_t* l2g, const uint8_t* dirichlet,
@@ -271,8 +316,8 @@ ceedbp_status setup_impl(ceedbp_ctx* c, const double* coords, const int64_t* l2g
     if (d_kappa) cudaFree(d_kappa);
     if (e != cudaSuccess) return cuda_fail(c, e, "geometric factors");
   }
-  if ((c->arith == CEEDBP_ARITH_FP64 || !c->colloc) && !recompute && !c->batch_group) {
-    const ceedbp_status st = prepare_fx(c);
+  if (fx_context(c)) {
+    const ceedbp_status st = setup_fx(c);
     if (st != CEEDBP_OK) return st;
   }
   // ---- Jacobi diagonal: local diag(A^e) (or diag(B^e)), summed by Q^T, inverted
@@ -321,7 +366,7 @@ ceedbp_status setup_impl(ceedbp_ctx* c, const double* coords, const int64_t* l2g
   }
   if (c->arith == CEEDBP_ARITH_DF64 && !c->colloc) {
     // BP1 / BP3: the fixed-point kernel with pairs in and out; a pair copy of dinv for the vector kernels
-    CK(c, dalloc(&c->d_dinvdf, n));
+    CK(c, alloc_late(c, &c->d_dinvdf, n));
     CK(c, launch_f64_to_df(c->d_dinv, c->d_dinvdf, n, s));
     ElemDfArgs a = {};
     a.u_f64 = c->d_r;
@@ -692,20 +737,20 @@ ceedbp_status ceedbp_prepare_mixed(ceedbp_ctx* c, int precision) {
   const int64_t ng = c->prm.nelem * 6 * int64_t(c->q) * c->q * c->q;
   cudaStream_t s = c->stream;
   if (!c->d_xin) {
-    CK(c, dalloc(&c->d_xin, size_t(n * nc)));
-    CK(c, dalloc(&c->d_rin, size_t(n * nc)));
-    CK(c, dalloc(reinterpret_cast<float**>(&c->d_pin), size_t(n * nc)));
-    CK(c, dalloc(&c->d_dinv32, size_t(n)));
-    CK(c, dalloc(&c->d_outer, 3));
+    CK(c, alloc_late(c, &c->d_xin, size_t(n * nc)));
+    CK(c, alloc_late(c, &c->d_rin, size_t(n * nc)));
+    CK(c, alloc_late(c, reinterpret_cast<float**>(&c->d_pin), size_t(n * nc)));
+    CK(c, alloc_late(c, &c->d_dinv32, size_t(n)));
+    CK(c, alloc_late(c, &c->d_outer, 3));
     CK(c, cudaMallocHost(reinterpret_cast<void**>(&c->h_outer), 3 * sizeof(double)));
     CK(c, launch_narrow(c->d_dinv, c->d_dinv32, n, 0, s));
   }
   if (precision != CEEDBP_MIXED_BF16 && !c->d_G32) {
-    CK(c, dalloc(&c->d_G32, size_t(ng)));
+    CK(c, alloc_late(c, &c->d_G32, size_t(ng)));
     CK(c, launch_narrow(c->d_G, c->d_G32, ng, 0, s));
   }
   if (precision == CEEDBP_MIXED_BF16 && !c->d_Gbf) {
-    CK(c, cudaMalloc(&c->d_Gbf, sizeof(uint16_t) * size_t(ng)));
+    CK(c, alloc_late(c, reinterpret_cast<uint16_t**>(&c->d_Gbf), size_t(ng)));
     CK(c, launch_narrow(c->d_G, c->d_Gbf, ng, 1, s));
   }
   // prime the inner element kernel outside any capture (one-time attribute setup)
@@ -900,7 +945,7 @@ ceedbp_status ceedbp_set_kappa(ceedbp_ctx* c, const double* kappa) {
   const int64_t q3 = int64_t(c->q) * c->q * c->q;
   const size_t ng = size_t(c->prm.nelem) * 6 * q3;
   if (!c->d_Ghat) {  // set up with kappa = 1: the current factors are coefficient-free
-    CK(c, dalloc(&c->d_Ghat, ng));
+    CK(c, alloc_late(c, &c->d_Ghat, ng));
     CK(c, cudaMemcpyAsync(c->d_Ghat, c->d_G, sizeof(double) * ng, cudaMemcpyDeviceToDevice, s));
   }
   CK(c, launch_scale_factors(c->d_Ghat, kappa, c->d_G, c->prm.nelem, int(q3), s));
@@ -1006,7 +1051,7 @@ ceedbp_status ceedbp_bk_apply(ceedbp_ctx* c, const double* uL, double* wL) {
   const int64_t nloc = c->prm.nelem * int64_t(c->p1) * c->p1 * c->p1;
   if (!c->d_l2g_id) {
     // the element kernels gather through l2g; the identity map makes them read u_L directly
-    CK(c, dalloc(&c->d_l2g_id, nloc));
+    CK(c, alloc_late(c, &c->d_l2g_id, nloc));
     iota_kernel<<<1216, 256, 0, s>>>(c->d_l2g_id, nloc);
     CK(c, cudaGetLastError());
   }
@@ -1055,6 +1100,27 @@ ceedbp_status ceedbp_set_tile(ceedbp_ctx* c, int eb, int schedule, int seq) {
   a.mask_in = 1;
   CK(c, launch_elem_df(c->mesh, a, s));  // one launch outside any capture (attribute setup)
   CK(c, cudaStreamSynchronize(s));
+  return CEEDBP_OK;
+}
+
+ceedbp_status ceedbp_set_fixed_point(ceedbp_ctx* c, int on) {
+  if (!c) return fail(c, CEEDBP_EINVAL, "null context");
+  if (!fx_context(c))
+    return fail(c, CEEDBP_EUNSUPPORTED, "fixed-point factors belong to FP64 contexts with stored factors and to pairs of BP1 and BP3");
+  const bool have = c->d_Gfx || c->d_Mfx;
+  if (on && !have) {
+    CK(c, cudaStreamSynchronize(c->stream));
+    for (auto& g : c->graphs) cudaGraphExecDestroy(g.exec);  // captured launches hold no factors
+    c->graphs.clear();
+    return prepare_fx(c);
+  }
+  if (!on && have) drop_fx(c);
+  return CEEDBP_OK;
+}
+
+ceedbp_status ceedbp_fixed_point(const ceedbp_ctx* c, int* on) {
+  if (!c || !on) return CEEDBP_EINVAL;
+  *on = c->d_Gfx || c->d_Mfx;
   return CEEDBP_OK;
 }
 
