@@ -25,8 +25,10 @@
 // FP64 and faster than sums of pairs were (BK3, N = 5, 27 x 25 x 23 elements: 261 -> 200 us;
 // BK1, N = 7, 32^3: 782 -> 485 us; one application's error 5 to 100 times smaller).
 //
-// Element sequences, prefetches and the FP64 form of elements off the grid: as in elem_fx.cuh.  With
-// the Helmholtz term (Eq. (17), added at the quadrature points) every element takes the FP64 form.
+// Element sequences, prefetches and the FP64 form of elements off the grid: as in elem_fx.cuh.  The Helmholtz
+// operator (Eq. (17)) is two launches, the second a mass operator that adds beta times its result: both in fixed
+// point (one CG iteration, N = 7, 14^3 elements: 187 us, one FP64 pass that added the term at the quadrature points 458;
+// N = 11, 9^3: 219 against 486; N = 7, 4^3: 40 against 44).
 #pragma once
 
 #include <algorithm>
@@ -66,15 +68,14 @@ struct FxGlShape {
 };
 
 // One element in arithmetic Ar, u in tile A.  factors: gradient to flux at point z of the own column, or
-// value to value with the mass factors; add(z, v, u) sees the summed transposes (Helmholtz); done(shift)
-// comes with the number of bits the values were moved up; out(i, y) turns the nodal results of line
+// value to value with the mass factors; done(shift) comes with the number of bits the values were moved up; out(i, y) turns the nodal results of line
 // (j, k) = t into FP64, left in tile A.  weak(l) sees the values of line (j, k); if it
 // is, uneven() may set the first stage's word to kFxUneven: false is then returned, with only the tiles overwritten.
-template <int P1, int KIND, bool HELM, class Ar, class TJ, class TJT, class TD, class Weak, class Uneven, class Factors,
-          class Mid, class Add, class Done, class Out>
+template <int P1, int KIND, class Ar, class TJ, class TJT, class TD, class Weak, class Uneven, class Factors, class Mid,
+          class Done, class Out>
 __device__ __forceinline__ bool fx_gl_stages(void* tiles, int t, bool live, const TJ& J, const TJT& JT, const TD& D,
                                              const TD& DT, const FxNorm& norm, Weak&& weak, Uneven&& uneven, Factors&& factors,
-                                             Mid&& mid, Add&& add, Done&& done, Out&& out) {
+                                             Mid&& mid, Done&& done, Out&& out) {
   using Sh = FxGlShape<P1, KIND>;
   using L = typename Ar::L;
   using Raw = typename Ar::Raw;
@@ -104,14 +105,12 @@ __device__ __forceinline__ bool fx_gl_stages(void* tiles, int t, bool live, cons
     eo_line<Ar::kBias, P1, Q, false>(J, l, [&](int n, auto y) { A[yb + n * S] = Ar::limbs(y); });
   }
   __syncthreads();
-  double uq[HELM ? Q : 1];  // u at the column's points, FP64 form only
   if constexpr (KIND == kStiff) {
     if (live) {
       L l[P1];
 #pragma unroll
       for (int n = 0; n < P1; ++n) l[n] = A[own + n * PS];
       eo_line<0, P1, Q, false>(J, l, [&](int n, auto y) {
-        if constexpr (HELM) uq[n] = y;
         ar.see(y);
         Ax[own + n * PS] = y;
       });
@@ -166,8 +165,7 @@ __device__ __forceinline__ bool fx_gl_stages(void* tiles, int t, bool live, cons
     if (live) {
 #pragma unroll
       for (int z = 0; z < Q; ++z) {
-        Raw v = Bx[own + z * PS] + Cx[own + z * PS] + Ax[own + z * PS];
-        if constexpr (HELM) v = add(z, v, uq[z]);
+        const Raw v = Bx[own + z * PS] + Cx[own + z * PS] + Ax[own + z * PS];
         ar.see(v);
         Ax[own + z * PS] = v;
       }
@@ -215,7 +213,8 @@ __device__ __forceinline__ bool fx_gl_stages(void* tiles, int t, bool live, cons
 }
 
 // PAIR: u and w^e are FP32 pairs (df.cuh; u may be FP64 as well), converted in shared memory.
-template <int P1, int NC, int KIND, bool HELM, bool PAIR>
+// ADD: a.wl += a.beta w^e.
+template <int P1, int NC, int KIND, bool PAIR, bool ADD>
 __global__ void __launch_bounds__(FxGlShape<P1, KIND>::NT, FxGlShape<P1, KIND>::MINB)
     elem_fxgl_kernel(const DeviceMesh m, const ElemArgs a, const __grid_constant__ FxGlTab<P1> tab, const int ns) {
   using Sh = FxGlShape<P1, KIND>;
@@ -301,7 +300,7 @@ __global__ void __launch_bounds__(FxGlShape<P1, KIND>::NT, FxGlShape<P1, KIND>::
       if (it + 1 < nit) load_l2g(it + 1);
     }
     const unsigned mx = __reduce_max_sync(lanes, seen.top());
-    const int code = !HELM && live && fxe != nullptr ? __ldg(fxe + e) : kFxNoGrid, ge = code >> kFxReachBits;
+    const int code = live && fxe != nullptr ? __ldg(fxe + e) : kFxNoGrid, ge = code >> kFxReachBits;
     const FxNorm norm{lanes, lead, smax + (it & 1) * EB + (live ? slot : 0), 2 * EB};
     if (lead) atomicMax(norm.top, mx);
     __syncthreads();
@@ -317,70 +316,67 @@ __global__ void __launch_bounds__(FxGlShape<P1, KIND>::NT, FxGlShape<P1, KIND>::
         if (NC == 1 || (it + 1) % NC == 0) prefetch_factors(elem_of(it + 1));
       }
     };
-    if (live && !HELM) {
+    if (live) {
 #pragma unroll
       for (int n = 0; n < NPT; ++n)
         if (has(n)) reinterpret_cast<int2*>(tiles)[place(t + n * QQ)] = fx_from_double(su[t + n * QQ], eb);
     }
     bool f64 = __syncthreads_or(bad);
-    if constexpr (!HELM) {
-      if (!f64) {
-        double sc = 0.0;
-        // a line (j, k) below the limb of the smallest value that reaches, and its nodes one by one. Pairs carry 47
-        // bits: they keep theirs at ratios up to 2^10 larger.
-        const int reach = PAIR ? min((code & 15) + 10, 15) : code & 15;
-        auto weak = [&](const int2(&l)[P1]) {
-          int hi = 0, lo = 0;
+    if (!f64) {
+      double sc = 0.0;
+      // a line (j, k) below the limb of the smallest value that reaches, and its nodes one by one. Pairs carry 47
+      // bits: they keep theirs at ratios up to 2^10 larger.
+      const int reach = PAIR ? min((code & 15) + 10, 15) : code & 15;
+      auto weak = [&](const int2(&l)[P1]) {
+        int hi = 0, lo = 0;
 #pragma unroll
-          for (int n = 0; n < P1; ++n) {
-            hi = max(hi, l[n].x);
-            lo = min(lo, l[n].x);
-          }
-          return max(hi, ~lo) < int(((top & 0xfffffu) | 0x100000u) << 8 >> reach);
-        };
-        auto uneven = [&]() {
-          const int j = t % P1, k = t / P1, word = fx_reach_word(top, reach);
-          bool off = false;
-#pragma unroll 1
-          for (int i = 0; i < P1; ++i)
-            off |= !fx_line_reaches<P1>(su + k * P1 * P1 + i, P1, word) &&
-                   !fx_line_reaches<P1>(su + j * P1 + i, P1 * P1, word) &&
-                   !(a.skip_dirichlet_out && __ldg(m.l2g + e * P3 + t * P1 + i) < 0);
-          if (off)
-            for (int s = 0; s < EB; ++s) atomicMax(smax + ((KIND == kStiff ? 2 : 6) + (it & 1)) * EB + s, kFxUneven);
-        };
-        auto done = [&](int shift) { sc = wjk * __hiloint2double((eb + ge - shift - (1082 - 1023)) << 20, 0); };
-        auto out = [&](int i, long long y) { return __ll2double_rn(y) * (tab.w[i] * sc); };
-        auto add = [](int, long long v, double) { return v; };
-        if constexpr (KIND == kStiff) {
-          const int4* G = m.Gfx + e * 3 * Q3 + t;
-          f64 = !fx_gl_stages<P1, KIND, false, FxArith>(
-              tiles, t, live, tab.J, tab.JT, tab.D, tab.DT, norm, weak, uneven,
-              [&](int z, int2 r, int2 s, int2 tt, long long& fr, long long& fs, long long& ft) {
-                const int4 g0 = __ldcs(G + (3 * z + 0) * QQ), g1 = __ldcs(G + (3 * z + 1) * QQ),
-                           g2 = __ldcs(G + (3 * z + 2) * QQ);
-                const int2 g00 = make_int2(g0.x, g0.y), g01 = make_int2(g0.z, g0.w), g02 = make_int2(g1.x, g1.y),
-                           g11 = make_int2(g1.z, g1.w), g12 = make_int2(g2.x, g2.y), g22 = make_int2(g2.z, g2.w);
-                fr = fx_dot3(g00, r, g01, s, g02, tt);
-                fs = fx_dot3(g01, r, g11, s, g12, tt);
-                ft = fx_dot3(g02, r, g12, s, g22, tt);
-              },
-              mid, add, done, out);
-        } else {
-          const int2* M = m.Mfx + e * Q3 + t;
-          f64 = !fx_gl_stages<P1, KIND, false, FxArith>(
-              tiles, t, live, tab.J, tab.JT, tab.D, tab.DT, norm, weak, uneven,
-              [&](int z, int2 v) {
-                const int2 f = __ldcs(M + z * QQ);
-                long long mm = fx_mad(f.x, v.y, kFxRound);
-                mm = fx_mad(f.y, v.x, mm);
-                return fx_join(fx_mad(f.x, v.x, 0), mm);
-              },
-              mid, add, done, out);
+        for (int n = 0; n < P1; ++n) {
+          hi = max(hi, l[n].x);
+          lo = min(lo, l[n].x);
         }
+        return max(hi, ~lo) < int(((top & 0xfffffu) | 0x100000u) << 8 >> reach);
+      };
+      auto uneven = [&]() {
+        const int j = t % P1, k = t / P1, word = fx_reach_word(top, reach);
+        bool off = false;
+#pragma unroll 1
+        for (int i = 0; i < P1; ++i)
+          off |= !fx_line_reaches<P1>(su + k * P1 * P1 + i, P1, word) &&
+                 !fx_line_reaches<P1>(su + j * P1 + i, P1 * P1, word) &&
+                 !(a.skip_dirichlet_out && __ldg(m.l2g + e * P3 + t * P1 + i) < 0);
+        if (off)
+          for (int s = 0; s < EB; ++s) atomicMax(smax + ((KIND == kStiff ? 2 : 6) + (it & 1)) * EB + s, kFxUneven);
+      };
+      auto done = [&](int shift) { sc = wjk * __hiloint2double((eb + ge - shift - (1082 - 1023)) << 20, 0); };
+      auto out = [&](int i, long long y) { return __ll2double_rn(y) * (tab.w[i] * sc); };
+      if constexpr (KIND == kStiff) {
+        const int4* G = m.Gfx + e * 3 * Q3 + t;
+        f64 = !fx_gl_stages<P1, KIND, FxArith>(
+            tiles, t, live, tab.J, tab.JT, tab.D, tab.DT, norm, weak, uneven,
+            [&](int z, int2 r, int2 s, int2 tt, long long& fr, long long& fs, long long& ft) {
+              const int4 g0 = __ldcs(G + (3 * z + 0) * QQ), g1 = __ldcs(G + (3 * z + 1) * QQ),
+                         g2 = __ldcs(G + (3 * z + 2) * QQ);
+              const int2 g00 = make_int2(g0.x, g0.y), g01 = make_int2(g0.z, g0.w), g02 = make_int2(g1.x, g1.y),
+                         g11 = make_int2(g1.z, g1.w), g12 = make_int2(g2.x, g2.y), g22 = make_int2(g2.z, g2.w);
+              fr = fx_dot3(g00, r, g01, s, g02, tt);
+              fs = fx_dot3(g01, r, g11, s, g12, tt);
+              ft = fx_dot3(g02, r, g12, s, g22, tt);
+            },
+            mid, done, out);
+      } else {
+        const int2* M = m.Mfx + e * Q3 + t;
+        f64 = !fx_gl_stages<P1, KIND, FxArith>(
+            tiles, t, live, tab.J, tab.JT, tab.D, tab.DT, norm, weak, uneven,
+            [&](int z, int2 v) {
+              const int2 f = __ldcs(M + z * QQ);
+              long long mm = fx_mad(f.x, v.y, kFxRound);
+              mm = fx_mad(f.y, v.x, mm);
+              return fx_join(fx_mad(f.x, v.x, 0), mm);
+            },
+            mid, done, out);
       }
     }
-    if (HELM || f64) {
+    if (f64) {
       if (live) {
 #pragma unroll
         for (int n = 0; n < NPT; ++n)
@@ -388,13 +384,12 @@ __global__ void __launch_bounds__(FxGlShape<P1, KIND>::NT, FxGlShape<P1, KIND>::
       }
       __syncthreads();
       auto done = [](int) {};
-      auto add = [&](int z, double v, double u) { return v + a.beta * __ldg(a.Mq + e * Q3 + z * QQ + t) * u; };
       auto out = [](int, double y) { return y; };
       auto weak = [](const double(&)[P1]) { return false; };
       auto uneven = []() {};
       const double* G = a.G + e * NF * Q3 + t;
       if constexpr (KIND == kStiff) {
-        fx_gl_stages<P1, KIND, HELM, F64Arith>(
+        fx_gl_stages<P1, KIND, F64Arith>(
             tiles, t, live, tab.J64, tab.JT64, tab.D64, tab.DT64, norm, weak, uneven,
             [&](int z, double r, double s, double tt, double& fr, double& fs, double& ft) {
               const double* Gz = G + z * QQ;
@@ -404,11 +399,11 @@ __global__ void __launch_bounds__(FxGlShape<P1, KIND>::NT, FxGlShape<P1, KIND>::
               fs = g01 * r + g11 * s + g12 * tt;
               ft = g02 * r + g12 * s + g22 * tt;
             },
-            mid, add, done, out);
+            mid, done, out);
       } else {
-        fx_gl_stages<P1, KIND, HELM, F64Arith>(
+        fx_gl_stages<P1, KIND, F64Arith>(
             tiles, t, live, tab.J64, tab.JT64, tab.D64, tab.DT64, norm, weak, uneven,
-            [&](int z, double v) { return __ldcs(G + z * QQ) * v; }, mid, add, done, out);
+            [&](int z, double v) { return __ldcs(G + z * QQ) * v; }, mid, done, out);
       }
     }
     // w^e to the local output (coalesced), (u^e, w^e)
@@ -419,8 +414,9 @@ __global__ void __launch_bounds__(FxGlShape<P1, KIND>::NT, FxGlShape<P1, KIND>::
       for (int n = 0; n < NPT; ++n) {
         if (!has(n)) continue;
         const int idx = t + n * QQ;
-        const double w = tiles[place(idx)];
+        double w = tiles[place(idx)];
         if (!(a.skip_dirichlet_out && ((dcur >> n) & 1u))) {
+          if constexpr (ADD) w = wl[size_t(idx) * NC] + a.beta * w;
           if constexpr (PAIR) reinterpret_cast<dfloat*>(wl)[size_t(idx) * NC] = f64_to_df(w);
           else wl[size_t(idx) * NC] = w;
         }
@@ -453,10 +449,10 @@ FxGlTab<P1> elem_fxgl_tab(const DeviceMesh& m) {
 
 // Blocks resident on the GPU (0: the kernel does not fit), found once per instantiation; the
 // attribute that lets it use its shared memory is set on the way.
-template <int P1, int NC, int KIND, bool HELM, bool PAIR>
+template <int P1, int NC, int KIND, bool PAIR, bool ADD>
 int elem_fxgl_resident() {
   using Sh = FxGlShape<P1, KIND>;
-  static const int n = fx_resident(reinterpret_cast<const void*>(elem_fxgl_kernel<P1, NC, KIND, HELM, PAIR>), Sh::NT, Sh::SMEM);
+  static const int n = fx_resident(reinterpret_cast<const void*>(elem_fxgl_kernel<P1, NC, KIND, PAIR, ADD>), Sh::NT, Sh::SMEM);
   return n;
 }
 
@@ -472,29 +468,35 @@ int elem_fxgl_blocks_t(int64_t nelem) {
   return int((nelem + per - 1) / per);
 }
 
-template <int P1, int NC, int KIND, bool HELM, bool PAIR = false>
-cudaError_t launch_elem_fxgl_h(const DeviceMesh& m, const ElemArgs& a, cudaStream_t s) {
+template <int P1, int NC, int KIND, bool PAIR = false, bool ADD = false>
+cudaError_t launch_elem_fxgl_k(const DeviceMesh& m, const ElemArgs& a, cudaStream_t s) {
   using Sh = FxGlShape<P1, KIND>;
-  if (elem_fxgl_resident<P1, NC, KIND, HELM, PAIR>() < 1) return cudaErrorInvalidConfiguration;
+  if (elem_fxgl_resident<P1, NC, KIND, PAIR, ADD>() < 1) return cudaErrorInvalidConfiguration;
   const int ns = elem_fxgl_seq<P1, NC, KIND>(m.nelem), blocks = elem_fxgl_blocks_t<P1, NC, KIND>(m.nelem);
-  elem_fxgl_kernel<P1, NC, KIND, HELM, PAIR><<<blocks, Sh::NT, Sh::SMEM, s>>>(m, a, elem_fxgl_tab<P1>(m), ns);
+  elem_fxgl_kernel<P1, NC, KIND, PAIR, ADD><<<blocks, Sh::NT, Sh::SMEM, s>>>(m, a, elem_fxgl_tab<P1>(m), ns);
   return cudaGetLastError();
+}
+
+template <int P1, int NC>
+cudaError_t launch_elem_fxgl_n(const DeviceMesh& m, int kind, const ElemArgs& a, cudaStream_t s) {
+  if (kind == kMass) return launch_elem_fxgl_k<P1, NC, kMass>(m, a, s);
+  if (a.beta == 0.0) return launch_elem_fxgl_k<P1, NC, kStiff>(m, a, s);
+  ElemArgs stiff = a, mass = a;  // A u first; the mass pass adds beta B u and sums (u, w) of both
+  stiff.partials = nullptr;
+  mass.G = a.Mq;
+  const cudaError_t e = launch_elem_fxgl_k<P1, NC, kStiff>(m, stiff, s);
+  return e != cudaSuccess ? e : launch_elem_fxgl_k<P1, NC, kMass, false, true>(m, mass, s);
 }
 
 template <int P1>
 cudaError_t launch_elem_fxgl_t(const DeviceMesh& m, int kind, const ElemArgs& a, cudaStream_t s) {
-  if (m.ncomp == 3) {
-    if (kind == kMass) return launch_elem_fxgl_h<P1, 3, kMass, false>(m, a, s);
-    return a.beta != 0.0 ? launch_elem_fxgl_h<P1, 3, kStiff, true>(m, a, s) : launch_elem_fxgl_h<P1, 3, kStiff, false>(m, a, s);
-  }
-  if (kind == kMass) return launch_elem_fxgl_h<P1, 1, kMass, false>(m, a, s);
-  return a.beta != 0.0 ? launch_elem_fxgl_h<P1, 1, kStiff, true>(m, a, s) : launch_elem_fxgl_h<P1, 1, kStiff, false>(m, a, s);
+  return m.ncomp == 3 ? launch_elem_fxgl_n<P1, 3>(m, kind, a, s) : launch_elem_fxgl_n<P1, 1>(m, kind, a, s);
 }
 
 template <int P1>
 cudaError_t launch_elem_fxgl_pair_t(const DeviceMesh& m, int kind, const ElemArgs& a, cudaStream_t s) {
-  return kind == kMass ? launch_elem_fxgl_h<P1, 1, kMass, false, true>(m, a, s)
-                       : launch_elem_fxgl_h<P1, 1, kStiff, false, true>(m, a, s);
+  return kind == kMass ? launch_elem_fxgl_k<P1, 1, kMass, true>(m, a, s)
+                       : launch_elem_fxgl_k<P1, 1, kStiff, true>(m, a, s);
 }
 
 // Largest grid of the order's launches with m's elements (room for their partial sums).

@@ -155,3 +155,19 @@ def test_uneven_values_beside_the_boundary(bp, N):
         assert np.abs(w[free] - ref[free]).max() < 1.0
         units = float((np.abs(w[free] - ref[free]) / scale[free]).max()) * 2.0 ** 53
         assert units < _bound(min(N, 7)) * (4 if N > 7 else 1)
+
+
+@pytest.mark.parametrize("bp,N,E", [(3, 1, 15), (3, 2, 9), (3, 3, 6), (3, 5, 8), (3, 7, 3), (3, 12, 1), (4, 1, 29), (4, 4, 6),
+                                    (4, 6, 2)])
+@pytest.mark.parametrize("beta", [3.0, 1e6])
+def test_helmholtz_is_the_sum_of_two_operators(bp, N, E, beta):
+    """A u + beta B u of BP3/BP4 to two roundings of the sum of BP3's A u and beta times BP1's B u, block
+    remainders and an uneven element included."""
+    coords, l2g, _ = pkg.mesh_box(E, 1, 1, N, 0.05)
+    stiff, mass = pkg.Operator(bp, N, coords, l2g, None), pkg.Operator(1 if bp == 3 else 2, N, coords, l2g, None)
+    shape = (E, (N + 1) ** 3) if bp == 3 else (E, (N + 1) ** 3, 3)
+    u = uniform_pm1(15, np.arange(int(np.prod(shape)))).reshape(shape)
+    u[E // 2].reshape(-1)[1:] *= 1e-9
+    a, b = _run(stiff, u), _run(mass, u)
+    stiff.set_helmholtz(beta)
+    assert (np.abs(_run(stiff, u) - (a + beta * b)) <= 2.0 ** -52 * (np.abs(a) + 2 * beta * np.abs(b))).all()
