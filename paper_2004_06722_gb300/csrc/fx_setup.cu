@@ -50,17 +50,48 @@ long double eo_tables(int NO, int NI, bool anti, const std::vector<long double>&
   }
 }
 
-// (ah + al) g / w3 as limbs (|result| <= 2^62); the errors of the quotient and of the product are put back.
-__device__ __forceinline__ int2 fx_factor(double g, double w3, double rw3, double ah, double al) {
-  const double q = g * rw3, r = __fma_rn(-q, w3, g) * rw3;
-  const double v = q * ah, d = __fma_rn(q, ah, -v) + (r * ah + q * al);
-  return fx_limbs(__double2ll_rn(v) + __double2ll_rn(d) + kFxHalf);
+// Factor of a quadrature point, scale c over its weight, as m 2^(x-63) with 2^63 <= m < 2^64.
+struct FxWeight {
+  unsigned long long m;
+  int x, pad;
+};
+
+// Magnitude of a product g c / w as an upper word of FP64 would order it: 20 bits below the exponent field e,
+// for (1 + fraction) 2^(e-1022); the product's upper bits cut, zeros and subnormal g zero.
+__device__ __forceinline__ int fx_key(double g, FxWeight f) {
+  const int hi = __double2hiint(g), ev = (hi >> 20) & 0x7ff;
+  const unsigned p = __umulhi(unsigned((hi & 0xfffff) | 0x100000) << 11, unsigned(f.m >> 32));
+  const int up = int(p >> 31);  // 2^30 <= p < 2^32
+  return ev == 0 ? 0 : ((ev + f.x - 1 + up) << 20) | int((p >> (10 + up)) & 0xfffffu);
 }
 
-// One block per element: its exponent, then the limbs of alpha G with alpha = 2^(62-k) c, where c = ch + cl in
+// Upper bound of a sum of three magnitudes of at most `top`'s exponent: each is cut by at most 2^-19.
+__device__ __forceinline__ int fx_key_sum(int a, int b, int c, int top) {
+  const int e = top >> 20;
+  auto rel = [&](int k) {
+    const int d = (k >> 20) - e;
+    return d < -60 ? 0.0f : __int_as_float(((127 + d) << 23) | ((k & 0xfffff) << 3));
+  };
+  return (__float_as_int(rel(a) + rel(b) + rel(c)) >> 3) + ((e - 127) << 20) + 8;
+}
+
+// g c / w 2^(62-k) as limbs (|result| <= 2^62), to 2^-62 of itself.
+__device__ __forceinline__ int2 fx_factor(double g, FxWeight f, int k) {
+  const int hi = __double2hiint(g), ev = (hi >> 20) & 0x7ff;
+  const unsigned long long m =
+      ((unsigned long long)(unsigned((hi & 0xfffff) | 0x100000)) << 32 | unsigned(__double2loint(g))) << 11;
+  const int sh = 1023 + k - ev - f.x;  // at least 0 by the choice of k
+  const unsigned long long p = __umul64hi(m, f.m);
+  const long long r = ev == 0 || sh > 64 ? 0ll : sh <= 0 ? (long long)p : (long long)(((p >> (sh - 1)) + 1) >> 1);
+  return fx_limbs((hi < 0 ? -r : r) + kFxHalf);
+}
+
+// One block per element: its exponent, then the limbs of alpha G with alpha = 2^(62-k) c, where c in
 // [1, 2) and 2^ce are mantissa and exponent of the tables' scales (their chain): one unit of the element's
-// result is then exactly 2^(k+ce) units of its input. NF = 6: stiffness factors
-// G [e][6][q^3] -> [e][k][3][q^2] pairs of entries (00,01), (02,11), (12,22); NF = 1: mass factors.
+// result is then exactly 2^(k+ce) units of its input.  The factors come with their quadrature weights, which fw
+// divides out: 64-bit integer products, since some 75 FP64 operations a point took 3.5 ms at N = 7,
+// 32^3 elements (0.4 ms now, of which the bytes are 0.25), and ceedbp_set_kappa pays them on every call.
+// NF = 6: stiffness factors G [e][6][q^3] -> [e][k][3][q^2] pairs of entries (00,01), (02,11), (12,22); NF = 1: mass factors.
 //
 // An element is on the grid while the factors that carry it are within 2^kFxSpread of its largest row sum:
 // one direction's diagonal factors at all points (collocated), the larger ones of each point (Gauss, where
@@ -77,112 +108,113 @@ __device__ __forceinline__ int2 fx_factor(double g, double w3, double rw3, doubl
 // above the others: order 1 0.7 / 0.8, 2 2.4 / 0.9, 3 2.6 / 1.9, 5 6.4 / 2.5, 7 8.4 / 5.2, 15 20 / 7.5; 2^4: order 5 and up
 // within 1.1 of FP64).
 constexpr int kFxSpread = 5;
-__device__ __forceinline__ int fx_reach(double big, double small, int budget) {
-  if (!(small * double(1 << kFxSpread) >= big)) return 0;
-  int s = 0;
-  frexp(big / small, &s);  // the ratio is in [2^(s-1), 2^s)
-  return max(budget + 1 - s, 0);
+__device__ __forceinline__ int fx_ratio_bits(int big, int small) {  // the ratio is below 2^this
+  return (big >> 20) - (small >> 20) + ((big & 0xfffff) >= (small & 0xfffff));
+}
+__device__ __forceinline__ int fx_reach(int big, int small, int budget) {
+  const int s = fx_ratio_bits(big, small);
+  return s > kFxSpread ? 0 : max(budget + 1 - s, 0);
 }
 
 template <int NF>
-__global__ void fx_factors_kernel(const double* __restrict__ G, const double* __restrict__ w, int q, double ch,
-                                  double cl, int ce, int colloc, int all_dirs, int budget, void* out, int* __restrict__ gexp) {
+__global__ void fx_factors_kernel(const double* __restrict__ G, const FxWeight* __restrict__ fw, int q, int ce, int colloc,
+                                  int all_dirs, int budget, void* out, int* __restrict__ gexp) {
   constexpr int NR = NF == 6 ? 5 : 2;  // largest row sum; smallest of each direction and of the points' largest
-  __shared__ double sw[kMaxQ], srw[kMaxQ], sred[NR][32];
-  __shared__ int s_bad;
+  __shared__ int sred[NR][8];
   const int64_t e = blockIdx.x;
   const int q2 = q * q, q3 = q2 * q, tid = threadIdx.x;
   const double* Ge = G + e * NF * q3;
-  if (tid < q) {
-    sw[tid] = w[tid];
-    srw[tid] = 1.0 / w[tid];
-  }
-  if (tid == 0) s_bad = 0;
-  __syncthreads();
-  // largest row sum of |G| and smallest diagonal entries, all without the weights
-  double v[NR];
-  v[0] = 0.0;
+  int v[NR];
+  v[0] = 0;
 #pragma unroll
-  for (int c = 1; c < NR; ++c) v[c] = __longlong_as_double(0x7fefffffffffffffll);
+  for (int c = 1; c < NR; ++c) v[c] = 0x7fffffff;
   bool bad = false;
   for (int p = tid; p < q3; p += blockDim.x) {
-    const double rw3 = srw[p % q] * srw[(p / q) % q] * srw[p / q2];
-    double f[NF];
+    const FxWeight f = fw[p];
+    int y[NF];
 #pragma unroll
     for (int c = 0; c < NF; ++c) {
-      f[c] = fabs(Ge[size_t(c) * q3 + p]) * rw3;
-      bad |= !isfinite(f[c]);
+      const double g = Ge[size_t(c) * q3 + p];
+      bad |= (__double2hiint(g) & 0x7ff00000) == 0x7ff00000;
+      y[c] = fx_key(g, f);
     }
     if constexpr (NF == 6) {
-      v[0] = fmax(v[0], fmax(f[0] + f[1] + f[2], fmax(f[1] + f[3] + f[4], f[2] + f[4] + f[5])));
-      v[1] = fmin(v[1], f[0]);
-      v[2] = fmin(v[2], f[3]);
-      v[3] = fmin(v[3], f[5]);
-      v[4] = fmin(v[4], fmax(f[0], fmax(f[3], f[5])));
+      const int d = max(y[0], max(y[3], y[5])), top = max(d, max(y[1], max(y[2], y[4])));
+      v[0] = max(v[0], max(fx_key_sum(y[0], y[1], y[2], top),
+                           max(fx_key_sum(y[1], y[3], y[4], top), fx_key_sum(y[2], y[4], y[5], top))));
+      v[1] = min(v[1], y[0]);
+      v[2] = min(v[2], y[3]);
+      v[3] = min(v[3], y[5]);
+      v[4] = min(v[4], d);
     } else {
-      v[0] = fmax(v[0], f[0]);
-      v[1] = fmin(v[1], f[0]);
+      v[0] = max(v[0], y[0] + 8);
+      v[1] = min(v[1], y[0]);
     }
   }
-  if (bad) s_bad = 1;
+  bad = __syncthreads_or(bad);
 #pragma unroll
   for (int c = 0; c < NR; ++c) {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      const double x = __shfl_xor_sync(0xffffffffu, v[c], o);
-      v[c] = c == 0 ? fmax(v[c], x) : fmin(v[c], x);
-    }
+    v[c] = c == 0 ? __reduce_max_sync(0xffffffffu, v[c]) : __reduce_min_sync(0xffffffffu, v[c]);
     if ((tid & 31) == 0) sred[c][tid >> 5] = v[c];
   }
   __syncthreads();
   for (int i = 0; i < int(blockDim.x) / 32; ++i)
 #pragma unroll
-    for (int c = 0; c < NR; ++c) v[c] = c == 0 ? fmax(v[c], sred[c][i]) : fmin(v[c], sred[c][i]);
-  const double big = v[0];
+    for (int c = 0; c < NR; ++c) v[c] = c == 0 ? max(v[c], sred[c][i]) : min(v[c], sred[c][i]);
   int reach = 0;
   if (NF == 6 && colloc) {
-    if (!all_dirs || fmin(v[1], fmin(v[2], v[3])) * 16.0 >= big)
+    if (!all_dirs || fx_ratio_bits(v[0], min(v[1], min(v[2], v[3]))) <= 4)
 #pragma unroll
-      for (int d = 0; d < 3; ++d) reach |= fx_reach(big, v[1 + d], budget) << 4 * d;
+      for (int d = 0; d < 3; ++d) reach |= fx_reach(v[0], v[1 + d], budget) << 4 * d;
   } else {
-    reach = fx_reach(big, v[NR - 1], budget);
+    reach = fx_reach(v[0], v[NR - 1], budget);
   }
-  // big chain <= 2^k: the rows of alpha G stay within 2^62
-  int k = 0;
-  frexp(big * ch * (1.0 + 1e-9), &k);
+  const int k = (v[0] >> 20) - 1021;  // the largest row sum is below 2^k: the rows of alpha G stay within 2^62
   // outside the grid: not finite, spread too far, or far from 1
-  const bool off = s_bad || reach == 0 || !(big > 0.0) || k > 200 || k < -200;
+  const bool off = bad || reach == 0 || k > 200 || k < -200;
   if (tid == 0) gexp[e] = off ? kFxNoGrid : (k + ce) * (1 << kFxReachBits) + reach;
   if (off) return;
-  const double ah = scalbn(ch, 62 - k), al = scalbn(cl, 62 - k);
   for (int p = tid; p < q3; p += blockDim.x) {
-    const double w3 = sw[p % q] * sw[(p / q) % q] * sw[p / q2], rw3 = srw[p % q] * srw[(p / q) % q] * srw[p / q2];
+    const FxWeight f = fw[p];
     if constexpr (NF == 6) {
       int2 l[6];
 #pragma unroll
-      for (int c = 0; c < 6; ++c) l[c] = fx_factor(Ge[size_t(c) * q3 + p], w3, rw3, ah, al);
+      for (int c = 0; c < 6; ++c) l[c] = fx_factor(Ge[size_t(c) * q3 + p], f, k);
       int4* o = static_cast<int4*>(out) + e * 3 * q3 + size_t(p / q2) * 3 * q2 + p % q2;
 #pragma unroll
       for (int c = 0; c < 3; ++c) o[size_t(c) * q2] = make_int4(l[2 * c].x, l[2 * c].y, l[2 * c + 1].x, l[2 * c + 1].y);
     } else {
-      static_cast<int2*>(out)[e * q3 + p] = fx_factor(Ge[p], w3, rw3, ah, al);
+      static_cast<int2*>(out)[e * q3 + p] = fx_factor(Ge[p], f, k);
     }
   }
 }
 
 }  // namespace
 
+size_t fx_weight_bytes(int q) { return sizeof(FxWeight) * size_t(q) * q * q; }
+
+// Mantissa c of the chain over the weight of each point; returns the chain's exponent ce.
+int fx_weights(const Basis1D& b, long double chain, void* out) {
+  int ce = 0;
+  const long double c = 2.0L * std::frexp(chain, &ce);  // chain = c 2^(ce-1)
+  FxWeight* f = static_cast<FxWeight*>(out);
+  for (int p = 0; p < b.q * b.q * b.q; ++p) {
+    const long double w = (long double)b.w[p % b.q] * b.w[p / b.q % b.q] * b.w[p / b.q / b.q];
+    int x = 0;
+    const long double m = std::frexp(c / w, &x);  // in [1/2, 1)
+    f[p] = {(unsigned long long)std::ldexp(m, 64), x - 1, 0};
+  }
+  return ce - 1;
+}
+
 cudaError_t launch_fx_factors(const DeviceMesh& m, int kind, const double* G, void* out, int* gexp, cudaStream_t s) {
-  const double* w = m.basis + 2 * size_t(m.q) * m.p1 + size_t(m.q) * m.q;
-  const int threads = m.q <= 5 ? 128 : 256;
-  int e = 0;
-  const long double c = 2.0L * std::frexp(kind == kStiff ? m.fx->chain : m.fx->mchain, &e);  // chain = c 2^(e-1)
-  const double ch = double(c), cl = double(c - ch);
+  const int q3 = m.q * m.q * m.q, threads = q3 >= 256 ? 256 : (q3 + 31) / 32 * 32;
   const int all_dirs = m.colloc && m.p1 <= 3, budget = m.p1 <= 4 ? 10 - m.p1 : 5;
+  const FxWeight* fw = static_cast<const FxWeight*>(kind == kStiff ? m.fxw : m.fxmw);
   if (kind == kStiff)
-    fx_factors_kernel<6><<<unsigned(m.nelem), threads, 0, s>>>(G, w, m.q, ch, cl, e - 1, m.colloc, all_dirs, budget, out, gexp);
+    fx_factors_kernel<6><<<unsigned(m.nelem), threads, 0, s>>>(G, fw, m.q, m.fx->ce, m.colloc, all_dirs, budget, out, gexp);
   else
-    fx_factors_kernel<1><<<unsigned(m.nelem), threads, 0, s>>>(G, w, m.q, ch, cl, e - 1, m.colloc, all_dirs, budget, out, gexp);
+    fx_factors_kernel<1><<<unsigned(m.nelem), threads, 0, s>>>(G, fw, m.q, m.fx->mce, m.colloc, all_dirs, budget, out, gexp);
   return cudaGetLastError();
 }
 
@@ -206,7 +238,11 @@ void build_fx_tables(const Basis1D& b, FxTables* t) {
   eo_tables(q, q, true, MT, 62, &no_limbs, &t->DT64);
   t->w.assign(b.rho.begin(), b.rho.end());
   t->chain = d * dt;
-  if (b.colloc) return;
+  t->weights.resize(fx_weight_bytes(q));
+  if (b.colloc) {
+    t->ce = fx_weights(b, t->chain, t->weights.data());
+    return;
+  }
   std::vector<long double> J(size_t(q) * p), JT(size_t(q) * p);
   for (int j = 0; j < p; ++j) {
     long double sj = 0.0L;
@@ -224,6 +260,9 @@ void build_fx_tables(const Basis1D& b, FxTables* t) {
   eo_tables(p, q, false, JT, 62, &no_limbs, &t->JT64);
   t->mchain = js * js * js * jt * jt * jt;
   t->chain = t->mchain * d * dt;
+  t->ce = fx_weights(b, t->chain, t->weights.data());
+  t->mweights.resize(fx_weight_bytes(q));
+  t->mce = fx_weights(b, t->mchain, t->mweights.data());
 }
 
 }  // namespace ceedbp

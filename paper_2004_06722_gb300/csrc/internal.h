@@ -40,6 +40,9 @@ struct FxTables {
   std::vector<double> D64, DT64, J64, JT64;
   std::vector<double> w;  // weights of the result: GLL, or s of the Gauss tables (elem_fxgl.cuh)
   long double chain = 1.0L, mchain = 1.0L;
+  // a chain's mantissa over the quadrature weight of each point (FxWeight of fx_setup.cu), and its exponent
+  std::vector<unsigned char> weights, mweights;
+  int ce = 0, mce = 0;
 };
 
 // Word of an element of fixed-point factors: its exponent above kFxReachBits bits of how far below the
@@ -109,6 +112,8 @@ struct DeviceMesh {
                         // copy, 2 software-pipelined element sequences (elem_dfp_kernel)
   int tune_ns;          // elements per slot sequence of the pipelined schedule
   const FxTables* fx;   // host: tables of the fixed-point kernels
+  const void* fxw;      // device copies of fx->weights and fx->mweights (only while factors are made and held)
+  const void* fxmw;
   const int4* Gfx;      // fixed-point stiffness factors [E][q][3][q^2], or nullptr (FP64 form)
   const int* gexp;      // [E] exponent and reaches of the element (kFxNoGrid: it runs in FP64)
   const int2* Mfx;      // fixed-point mass factors [E][q^3] of Gauss quadrature, or nullptr
