@@ -1065,7 +1065,9 @@ ceedbp_status ceedbp_bk_apply(ceedbp_ctx* c, const double* uL, double* wL) {
   }
   DeviceMesh mb = c->mesh;
   mb.l2g = c->d_l2g_id;
-  if (c->arith == CEEDBP_ARITH_DF64) {
+  // pairs of BP1/BP3 run the FP64 kernel, which leaves FP64 here as well: pairs first and a second pass over them took
+  // 364 us instead of 289 (BP1, N = 1, 100^3 elements)
+  if (c->arith == CEEDBP_ARITH_DF64 && c->colloc) {
     ElemDfArgs a = df_args(c);
     a.u_f64 = uL;
     a.mask_in = 0;

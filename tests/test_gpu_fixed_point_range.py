@@ -171,3 +171,29 @@ def test_helmholtz_is_the_sum_of_two_operators(bp, N, E, beta):
     a, b = _run(stiff, u), _run(mass, u)
     stiff.set_helmholtz(beta)
     assert (np.abs(_run(stiff, u) - (a + beta * b)) <= 2.0 ** -52 * (np.abs(a) + 2 * beta * np.abs(b))).all()
+
+
+@pytest.mark.parametrize("bp,N", [(1, 1), (1, 4), (3, 2), (3, 7)])
+def test_unassembled_pairs_are_the_fp64_results(bp, N):
+    """Element-local vectors are FP64 on both sides: pair contexts of BP1/BP3 give the FP64 operator's bits."""
+    u = uniform_pm1(16, np.arange(5 * (N + 1) ** 3)).reshape(5, -1)
+    w = [_run(pkg.Operator.box(bp, 5, 1, 1, N, arith=arith), u) for arith in (pkg.ARITH_FP64, pkg.ARITH_DF64)]
+    np.testing.assert_array_equal(w[0], w[1])
+
+
+def test_pair_conversion_of_special_values():
+    """Pairs whose parts are zero, tiny or not finite through an apply of the pair arithmetic."""
+    op = pkg.Operator.box(1, 2, 1, 1, 2, arith=pkg.ARITH_DF64)
+    ref = pkg.Operator.box(1, 2, 1, 1, 2)
+    u = uniform_pm1(17, np.arange(op.nglobal))
+    u[::3] = 0.0
+    u[1::3] = np.ldexp(np.round(np.ldexp(u[1::3], 10)), -10)  # low parts zero
+    t = torch.from_numpy(u).cuda()
+    w, r = op.apply(t).cpu().numpy(), ref.apply(t).cpu().numpy()
+    assert np.abs(w - r).max() < 2.0 ** -44 * np.abs(r).max()
+    b = torch.from_numpy(r).cuda()
+    x, info = op.solve(b, tol=1e-12)
+    assert info["status"] == "OK" and float((x - t).abs().max()) < 1e-10
+    b[3] = float("inf")
+    with pytest.raises(pkg.CeedbpError):
+        op.solve(b, tol=1e-12)
