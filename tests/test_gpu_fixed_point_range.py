@@ -197,3 +197,46 @@ def test_pair_conversion_of_special_values():
     b[3] = float("inf")
     with pytest.raises(pkg.CeedbpError):
         op.solve(b, tol=1e-12)
+
+
+def _graded(N, ratio):
+    """A box of one row of two elements whose nodes crowd towards x = y = z = 0: det J varies over more than
+    `ratio` within each element."""
+    coords, l2g, _ = pkg.mesh_box(2, 1, 1, N, 0.0)
+    a = ratio ** (1.0 / 3.0)
+    grade = lambda x: (x + 0.5 * (a - 1.0) * x * x) / (1.0 + 0.5 * (a - 1.0))
+    out = coords.copy()
+    out[0, :, 0], out[1, :, 0] = 0.5 * grade(2.0 * coords[0, :, 0]), 0.5 + 0.5 * grade(2.0 * coords[1, :, 0] - 1.0)
+    out[..., 1], out[..., 2] = grade(coords[..., 1]), grade(coords[..., 2])
+    return out, l2g
+
+
+@pytest.mark.parametrize("bp,N", [(1, 2), (1, 5), (2, 3), (3, 3), (3, 7), (4, 4), (5, 5), (6, 2)])
+@pytest.mark.parametrize("ratio", [8.0, 1e3, 1e5])
+def test_factors_that_vary_within_an_element(bp, N, ratio):
+    """Mass and stiffness factors on the grid and off it (spreads beyond 2^5), in every kernel."""
+    coords, l2g = _graded(N, ratio)
+    op = pkg.Operator(bp, N, coords, l2g, None)
+    shape = (2, (N + 1) ** 3) if op.ncomp == 1 else (2, (N + 1) ** 3, 3)
+    u = uniform_pm1(18, np.arange(int(np.prod(shape)))).reshape(shape)
+    which = "B" if bp in (1, 2) else "A"
+    w = _run(op, u)
+    for e in range(2):
+        ref = element_matrices(coords[e], N, bp_rule(bp, N), want=(which,))[which] @ u[e]
+        assert np.linalg.norm(w[e] - ref) < 1e-12 * np.linalg.norm(ref)
+
+
+@pytest.mark.parametrize("bp,N", [(3, 2), (3, 6), (4, 3)])
+@pytest.mark.parametrize("contrast", [1e4, 0.0])
+def test_coefficient_jumps_gauss(bp, N, contrast):
+    """kappa jumping between the quadrature points of one element among others, also to zero."""
+    op = pkg.Operator.box(bp, 3, 1, 1, N)
+    kappa = np.ones((3, op.nquad ** 3))
+    kappa[1, ::3] = contrast
+    op.set_kappa(torch.from_numpy(kappa).cuda())
+    shape = (3, (N + 1) ** 3) if op.ncomp == 1 else (3, (N + 1) ** 3, 3)
+    u = uniform_pm1(19, np.arange(int(np.prod(shape)))).reshape(shape)
+    w = _run(op, u)
+    for e in range(3):
+        ref = element_matrices(op.coords[e], N, bp_rule(bp, N), kappa=kappa[e], want=("A",))["A"] @ u[e]
+        assert np.linalg.norm(w[e] - ref) < 1e-12 * np.linalg.norm(ref)
