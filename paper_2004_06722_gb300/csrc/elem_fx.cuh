@@ -252,7 +252,9 @@ __global__ void __launch_bounds__(FxCoShape<P1, W>::NT, FxCoShape<P1, W>::MINB)
     const unsigned top = live ? *norm.top : 0u;
     const int eb = top == 0u ? 1023 : int(top >> 20);  // every value is zero: any exponent
     const bool bad = live && (code == kFxNoGrid || eb < 500 || eb > 1500);
-    const bool weak = live && !bad && int(seen.top()) < fx_reach_word(top, code >> 8 & 15);  // the own column
+    // the own nodes: no large value among them and not all of the Dirichlet boundary
+    const bool weak = live && !bad && int(seen.top()) < fx_reach_word(top, code >> 8 & 15) &&
+                      !(a.skip_dirichlet_out && dcur == (1u << (W == 1 ? P1 : (P1 - el.grp + W - 1) / W)) - 1u);
     if (el.t == 0 && el.grp == 0 && live) smax[(~it & 1) * EB + slot] = smax[(2 + (~it & 1)) * EB + slot] = 0u;
     double* wl = a.wl + size_t(e) * P3 * NC + size_t(el.t) * NC + c;
     double acc = 0.0;

@@ -337,13 +337,18 @@ __global__ void __launch_bounds__(FxGlShape<P1, KIND>::NT, FxGlShape<P1, KIND>::
         return max(hi, ~lo) < int(((top & 0xfffffu) | 0x100000u) << 8 >> reach);
       };
       auto uneven = [&]() {
+        const int* l2g = m.l2g + e * P3 + t * P1;
+        bool free = !a.skip_dirichlet_out;  // lines of the Dirichlet boundary are the usual weak ones
+#pragma unroll
+        for (int i = 0; i < P1; ++i) free |= __ldg(l2g + i) >= 0;
+        if (!free) return;
         const int j = t % P1, k = t / P1, word = fx_reach_word(top, reach);
         bool off = false;
 #pragma unroll 1
         for (int i = 0; i < P1; ++i)
           off |= !fx_line_reaches<P1>(su + k * P1 * P1 + i, P1, word) &&
                  !fx_line_reaches<P1>(su + j * P1 + i, P1 * P1, word) &&
-                 !(a.skip_dirichlet_out && __ldg(m.l2g + e * P3 + t * P1 + i) < 0);
+                 !(a.skip_dirichlet_out && __ldg(l2g + i) < 0);
         if (off)
           for (int s = 0; s < EB; ++s) atomicMax(smax + ((KIND == kStiff ? 2 : 6) + (it & 1)) * EB + s, kFxUneven);
       };

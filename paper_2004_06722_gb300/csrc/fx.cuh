@@ -177,7 +177,9 @@ struct FxTop {
 // 2^-53 (|A| |u|)_i, as in FP64; without it the error was 2^-60 of the largest entry's scale.
 
 // The word of a stage's largest magnitude that says so: the check needs no barrier of its own.  What it costs
-// elements that are even: 1.4 % of a BP5 iteration at N = 7, 4 % of BP3's.
+// where elements are even: 0.8 % of a BP5 iteration at N = 7, 32^3 elements, nothing of BP3's (25^3), 1.3 % of BP1's
+// at N = 3.  At N = 15 the elements along the edges of a Dirichlet boundary are uneven (values fall with the
+// distance of the first node from two faces): 14 % of BP5, 10^3 elements.
 constexpr unsigned kFxUneven = 0x80000000u;
 
 // The smallest upper word that reaches (any value of an element of zeros).
