@@ -83,7 +83,7 @@ void release(ceedbp_ctx* c) {
                   c->d_wl, c->d_r, c->d_p, c->d_ax, c->d_part_apply, c->d_part_vec, c->d_state,
                   c->d_Gdf, c->d_Ddf, c->d_dinvdf, c->d_G32, c->d_Gbf, c->d_dinv32, c->d_xin,
                   c->d_rin, c->d_pin, c->d_outer, c->d_Ghat, c->d_scal, c->d_X, c->d_l2g_id, c->d_Gfx, c->d_gexp, c->d_Mfx,
-                  c->d_mexp, c->d_fxw, c->d_fxmw};
+                  c->d_mexp};
   for (void* p : ptrs)
     if (p) cudaFree(p);
   if (c->h_outer) cudaFreeHost(c->h_outer);
@@ -106,15 +106,13 @@ void drop_fx(ceedbp_ctx* c) {
   cudaStreamSynchronize(c->stream);
   for (auto& g : c->graphs) cudaGraphExecDestroy(g.exec);  // captured launches hold the factors
   c->graphs.clear();
-  void* ptrs[] = {c->d_Gfx, c->d_gexp, c->d_Mfx, c->d_mexp, c->d_fxw, c->d_fxmw};
+  void* ptrs[] = {c->d_Gfx, c->d_gexp, c->d_Mfx, c->d_mexp};
   for (void* p : ptrs)
     if (p) cudaFree(p);
   m.Gfx = c->d_Gfx = nullptr;
   m.gexp = c->d_gexp = nullptr;
   m.Mfx = c->d_Mfx = nullptr;
   m.mexp = c->d_mexp = nullptr;
-  m.fxw = c->d_fxw = nullptr;
-  m.fxmw = c->d_fxmw = nullptr;
 }
 
 // Fixed-point copies of the stiffness factors and, with Gauss quadrature, the mass factors for the FP64
@@ -129,23 +127,17 @@ ceedbp_status prepare_fx(ceedbp_ctx* c) {
   if (stiff && e == cudaSuccess) e = dalloc(&c->d_gexp, size_t(m.nelem));
   if (mass && e == cudaSuccess) e = dalloc(&c->d_Mfx, nq);
   if (mass && e == cudaSuccess) e = dalloc(&c->d_mexp, size_t(m.nelem));
-  if (stiff && e == cudaSuccess) e = dalloc(&c->d_fxw, c->fx.weights.size());
-  if (mass && e == cudaSuccess) e = dalloc(&c->d_fxmw, c->fx.mweights.size());
   if (e != cudaSuccess) {
     cudaGetLastError();
     drop_fx(c);
     return cuda_fail(c, e, "fixed-point factors");
   }
-  m.fxw = c->d_fxw;
-  m.fxmw = c->d_fxmw;
   if (stiff) {
-    CK(c, cudaMemcpyAsync(c->d_fxw, c->fx.weights.data(), c->fx.weights.size(), cudaMemcpyHostToDevice, c->stream));
     CK(c, launch_fx_factors(m, kStiff, c->d_G, c->d_Gfx, c->d_gexp, c->stream));
     m.Gfx = c->d_Gfx;
     m.gexp = c->d_gexp;
   }
   if (mass) {
-    CK(c, cudaMemcpyAsync(c->d_fxmw, c->fx.mweights.data(), c->fx.mweights.size(), cudaMemcpyHostToDevice, c->stream));
     CK(c, launch_fx_factors(m, kMass, c->d_Mq, c->d_Mfx, c->d_mexp, c->stream));
     m.Mfx = c->d_Mfx;
     m.mexp = c->d_mexp;
@@ -241,6 +233,13 @@ ceedbp_status setup_impl(ceedbp_ctx* c, const double* coords, const int64_t* l2g
   std::copy(basis.Dh.begin(), basis.Dh.end(), hb.begin() + size_t(qdef) * p1);
   std::copy(basis.Dq.begin(), basis.Dq.end(), hb.begin() + 2 * size_t(qdef) * p1);
   std::copy(basis.w.begin(), basis.w.end(), hb.begin() + 2 * size_t(qdef) * p1 + size_t(qdef) * qdef);
+  build_fx_tables(basis, &c->fx);
+  // behind them, 16-byte aligned, the weights of the fixed-point factors' conversion
+  const size_t fxw_at = (hb.size() + 1) / 2 * 2, fxmw_at = fxw_at + 2 * c->fx.weights.size();
+  hb.resize(fxmw_at + 2 * c->fx.mweights.size());
+  std::memcpy(hb.data() + fxw_at, c->fx.weights.data(), sizeof(FxWeight) * c->fx.weights.size());
+  if (!c->fx.mweights.empty())
+    std::memcpy(hb.data() + fxmw_at, c->fx.mweights.data(), sizeof(FxWeight) * c->fx.mweights.size());
 
   const int nc = c->ncomp;
   const int64_t n = P.nglobal;
@@ -285,8 +284,9 @@ ceedbp_status setup_impl(ceedbp_ctx* c, const double* coords, const int64_t* l2g
   m.slots = c->d_slots;
   m.head = c->d_head;
   m.basis = c->d_basis;
-  build_fx_tables(basis, &c->fx);
   m.fx = &c->fx;
+  m.fxw = reinterpret_cast<const FxWeight*>(c->d_basis + fxw_at);
+  m.fxmw = reinterpret_cast<const FxWeight*>(c->d_basis + fxmw_at);
 
   int nb_apply = elem_blocks(m);
   if (c->colloc) nb_apply = std::max(nb_apply, std::max(int(P.nelem), elem_lp_blocks(m)));

@@ -32,8 +32,6 @@ struct ceedbp_ctx {
   int* d_gexp = nullptr;
   int2* d_Mfx = nullptr;     // likewise the mass factors of Gauss quadrature
   int* d_mexp = nullptr;
-  unsigned char* d_fxw = nullptr;    // weights of their conversion
-  unsigned char* d_fxmw = nullptr;
   double* d_X = nullptr;  // [E][3][p1^3] coordinates when the factors are recomputed
   int* d_l2g_id = nullptr;  // identity gather map of ceedbp_bk_apply (allocated on its first call)
   double* d_Mq = nullptr;

@@ -32,6 +32,12 @@ struct Basis1D {
 // Device table layout (doubles): J [q*p1] | Dh [q*p1] | Dq [q*q] | w [q]
 inline size_t basis_doubles(int p1, int q) { return size_t(2) * q * p1 + size_t(q) * q + q; }
 
+// A fixed-point table's scale over the quadrature weight of a point, m 2^(x-63) with 2^63 <= m < 2^64.
+struct FxWeight {
+  unsigned long long m;
+  int x, pad;
+};
+
 // Even-odd tables of the block fixed-point kernels (fx.cuh), flattened in the order of EoMat: limb
 // pairs, and the FP64 forms. A scale is the true value of a stage's result over its fixed-point value;
 // chain and mchain are the products over all tables of a stiffness and a mass operator.
@@ -40,8 +46,7 @@ struct FxTables {
   std::vector<double> D64, DT64, J64, JT64;
   std::vector<double> w;  // weights of the result: GLL, or s of the Gauss tables (elem_fxgl.cuh)
   long double chain = 1.0L, mchain = 1.0L;
-  // a chain's mantissa over the quadrature weight of each point (FxWeight of fx_setup.cu), and its exponent
-  std::vector<unsigned char> weights, mweights;
+  std::vector<FxWeight> weights, mweights;  // a chain's mantissa over the weight of each point, and its exponent
   int ce = 0, mce = 0;
 };
 
@@ -112,8 +117,8 @@ struct DeviceMesh {
                         // copy, 2 software-pipelined element sequences (elem_dfp_kernel)
   int tune_ns;          // elements per slot sequence of the pipelined schedule
   const FxTables* fx;   // host: tables of the fixed-point kernels
-  const void* fxw;      // device copies of fx->weights and fx->mweights (only while factors are made and held)
-  const void* fxmw;
+  const FxWeight* fxw;  // device copies of fx->weights and fx->mweights
+  const FxWeight* fxmw;
   const int4* Gfx;      // fixed-point stiffness factors [E][q][3][q^2], or nullptr (FP64 form)
   const int* gexp;      // [E] exponent and reaches of the element (kFxNoGrid: it runs in FP64)
   const int2* Mfx;      // fixed-point mass factors [E][q^3] of Gauss quadrature, or nullptr
