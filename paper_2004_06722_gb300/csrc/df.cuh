@@ -87,14 +87,9 @@ __device__ __forceinline__ dfloat f64_to_df(double x) {
   return r;
 }
 
-// FP32 -> FP64 by its bits: the conversion instruction takes the FP64 pipe 16 cycles a warp.
-__device__ __forceinline__ double f32_to_f64(float x) {
-  const unsigned b = __float_as_uint(x), e = b & 0x7f800000u;
-  if (e - 0x00800000u >= 0x7f000000u) return static_cast<double>(x);  // zero, subnormal, infinity, NaN
-  return __hiloint2double(int((b & 0x80000000u) | (((b & 0x7fffffffu) >> 3) + (896u << 20))), int(b << 29));
+__device__ __forceinline__ double df_to_f64(dfloat v) {
+  return __dadd_rn(static_cast<double>(v.hi), static_cast<double>(v.lo));
 }
-
-__device__ __forceinline__ double df_to_f64(dfloat v) { return __dadd_rn(f32_to_f64(v.hi), f32_to_f64(v.lo)); }
 
 // Smallest power of two >= 2 b (b >= 0), at least 2^-100.
 __device__ __forceinline__ float splitter(float b) {
