@@ -21,8 +21,11 @@
 // current one, its u values are copied to shared memory (cp.async) once the gradient is done, and its
 // factors are prefetched into L2, so that the dependent gather overlaps a whole element's arithmetic.
 //
-// An element whose values or factors do not fit the fixed-point grid or are too uneven for it (fx.cuh), and every element
-// when the context holds no fixed-point factors, runs the same stages in FP64 (a.G, with weights).
+// An element whose values or factors do not fit the fixed-point grid or are too uneven for it (fx.cuh), and
+// every element when the context holds no fixed-point factors, runs the same stages in FP64 (a.G, with weights).
+// That form is not shaped for the FP64 pipe: 0.8 to 1.3 times the FP64 kernels that this one replaced, all
+// elements in it (solves on 1.5e6 DOFs; N = 7 222 -> 246 us an iteration, N = 11 266 -> 340, N = 12 482 -> 390). Blocks of 256 threads
+// of whole elements for it alone gained less than 10 % of that and lost elsewhere.
 #pragma once
 
 #include <algorithm>
@@ -67,7 +70,8 @@ struct FxCoShape {
   // Blocks per SM the registers are limited for: what shared memory holds, at 96 registers or more
   // (p1 = 8: eight blocks, 120 registers: 350 us at E = 2^15; ten, 96 registers: 370 us), that is five warps
   // on each of an SM's four partitions (N = 8, 20^3 elements, one iteration: seven blocks of three warps, 80 registers 284 us,
-  // six 272 us).
+  // six 272 us). From N = 11 on the lines of a thread do not fit these registers: spilled bytes a thread 264 at N = 11,
+  // 1172 at 12 (three blocks, 96 registers), 770-830 at 13 and 14, none at 15 (one block).
   static constexpr int BY_SMEM = int((size_t(227) << 10) / (SMEM + 1024)), BY_REGS = 4 * (512 / 96) / (NT / 32);
   static constexpr int MINB = W == 3 ? 1 : P1 == 8 ? 8 : BY_SMEM < BY_REGS ? BY_SMEM : BY_REGS;
 };
@@ -112,17 +116,17 @@ __device__ __forceinline__ bool fx_co_stages(const FxCoElem<P1>& el, const Tab& 
     __syncthreads();
   } else {
 #pragma unroll Sh::UNROLL
-  for (int dir = 0; dir < 3; ++dir) {
-    if (dir == 2) __syncthreads();  // r and s have read tile A: t goes in place
-    if (live) {
-      const int base = dir == 0 ? rb : dir == 1 ? sb : own, step = dir == 0 ? 1 : dir == 1 ? S : PS;
-      L* dst = A + (dir == 2 ? 0 : (dir + 1) * Sh::TILE) + base;
-      L l[P1];
+    for (int dir = 0; dir < 3; ++dir) {
+      if (dir == 2) __syncthreads();  // r and s have read tile A: t goes in place
+      if (live) {
+        const int base = dir == 0 ? rb : dir == 1 ? sb : own, step = dir == 0 ? 1 : dir == 1 ? S : PS;
+        L* dst = A + (dir == 2 ? 0 : (dir + 1) * Sh::TILE) + base;
+        L l[P1];
 #pragma unroll
-      for (int n = 0; n < P1; ++n) l[n] = A[base + n * step];
-      eo_line<Ar::kBias, P1, P1, true>(D, l, [&](int n, auto y) { dst[n * step] = Ar::limbs(y); });
+        for (int n = 0; n < P1; ++n) l[n] = A[base + n * step];
+        eo_line<Ar::kBias, P1, P1, true>(D, l, [&](int n, auto y) { dst[n * step] = Ar::limbs(y); });
+      }
     }
-  }
   }
   mid();
   if (live) {
@@ -284,15 +288,16 @@ __global__ void __launch_bounds__(FxCoShape<P1, W>::NT, FxCoShape<P1, W>::MINB)
     if (!f64) {
       if (weak) {  // its nodes one by one
         const double* se = el.su - el.t;
+        const int slack = fx_slack(a.state, c);
         bool off = false;
+        if (!fx_line_reaches<P1>(el.su, PP, fx_reach_word(top, code >> 8 & 15, slack)))
 #pragma unroll 1
-        for (int h = 0; h < KC; ++h) {
-          const int k = W * h + el.grp;
-          if ((W > 1 && k >= P1) || (a.skip_dirichlet_out && ((dcur >> h) & 1u))) continue;
-          off |= !fx_line_reaches<P1>(se + k * PP + el.tj * P1, 1, fx_reach_word(top, code & 15)) &&
-                 !fx_line_reaches<P1>(se + k * PP + el.ti, P1, fx_reach_word(top, code >> 4 & 15)) &&
-                 !(W > 1 && fx_line_reaches<P1>(el.su, PP, fx_reach_word(top, code >> 8 & 15)));
-        }
+          for (int h = 0; h < KC; ++h) {
+            const int k = W * h + el.grp;
+            if ((W > 1 && k >= P1) || (a.skip_dirichlet_out && ((dcur >> h) & 1u))) continue;
+            off |= !fx_line_reaches<P1>(se + k * PP + el.tj * P1, 1, fx_reach_word(top, code & 15, slack)) &&
+                   !fx_line_reaches<P1>(se + k * PP + el.ti, P1, fx_reach_word(top, code >> 4 & 15, slack));
+          }
         if (off)
           for (int s = 0; s < EB; ++s) atomicMax(smax + (2 + (it & 1)) * EB + s, kFxUneven);
       }

@@ -63,7 +63,11 @@ struct FxGlShape {
   static constexpr size_t SLOT = 8 * (size_t(NU) * P3 + (KIND == kStiff ? 3 : 1) * size_t(TILE));
   static constexpr size_t HEAD = 8 * 96 + 32 * size_t(EB);
   static constexpr size_t SMEM = HEAD + EB * SLOT;
-  static constexpr int BY_SMEM = int((size_t(227) << 10) / (SMEM + 1024)), BY_REGS = 65536 / (NT * (KIND == kMass || Q <= 7 ? 80 : 96));
+  // Blocks per SM the registers are limited for, as FxCoShape::MINB. Spilled bytes a thread: BK3 40 at N = 7 (seven blocks,
+  // 80 registers; six blocks 714 us against 597, 25^3 elements), 108 at 8, 350-440 at 10, 12 and 13, 250 at 15; BK1 up to 24
+  // to N = 8, 140-160 at 10 to 13, 1150 at 14.
+  static constexpr int BY_SMEM = int((size_t(227) << 10) / (SMEM + 1024)),
+                       BY_REGS = 65536 / (NT * (KIND == kMass || Q <= 7 ? 80 : 96));
   static constexpr int MINB = BY_SMEM < BY_REGS ? BY_SMEM : BY_REGS < 1 ? 1 : BY_REGS;
 };
 
@@ -342,7 +346,8 @@ __global__ void __launch_bounds__(FxGlShape<P1, KIND>::NT, FxGlShape<P1, KIND>::
 #pragma unroll
         for (int i = 0; i < P1; ++i) free |= __ldg(l2g + i) >= 0;
         if (!free) return;
-        const int j = t % P1, k = t / P1, word = fx_reach_word(top, reach);
+        const int slack = fx_slack(a.state, c), word = fx_reach_word(top, reach, slack), j = t % P1, k = t / P1;
+        if (slack > 0 && fx_line_reaches<P1>(su + t * P1, 1, word)) return;
         bool off = false;
 #pragma unroll 1
         for (int i = 0; i < P1; ++i)

@@ -183,8 +183,21 @@ struct FxTop {
 constexpr unsigned kFxUneven = 0x80000000u;
 
 // The smallest upper word that reaches (any value of an element of zeros).
-__device__ __forceinline__ int fx_reach_word(unsigned top, int r) {
-  return r == 0 ? 0x7fffffff : max(int(top) - (r << 20), 0);
+__device__ __forceinline__ int fx_reach_word(unsigned top, int r, int slack = 0) {
+  return r == 0 ? 0x7fffffff : max(int(top) - ((r + slack) << 20), 0);
+}
+
+// More bits that a line may lie below in a CG iteration: those by which the residual has fallen below the right-hand
+// side.  An error of A p counts against b, not against p: CG reaches the same residual while the products'
+// relative error stays below eps norm(b) / norm(r) (inexact Krylov methods: van den Eshof and Sleijpen, SIAM J. Matrix
+// Anal. Appl. 26, 2004; Simoncini and Szyld, SIAM J. Sci. Comput. 25, 2003).  Late directions of BP1 span the
+// quadrature weights: without these bits its solves went over to FP64 from order 9 on (N = 15: 8.0e9 instead of
+// 1.8e10 DOFs/s).  True residuals reached from tolerance 1e-13, right-hand sides of random values, BP1 N = 15: 2.7e-14 as with
+// FP64 kernels; with every direction on the grid 1.5e-13.
+__device__ __forceinline__ int fx_slack(const SolveState* st, int c) {
+  if (st == nullptr) return 0;
+  const int d = (__double2hiint(st->c[c].bb) >> 20) - (__double2hiint(st->c[c].rr) >> 20);  // of squares, not negative
+  return min(max(d >> 1, 0), 12);
 }
 
 // Whether one of the N values of a line reaches (the middle one first: most lines are answered by it).

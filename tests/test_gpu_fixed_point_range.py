@@ -240,3 +240,27 @@ def test_coefficient_jumps_gauss(bp, N, contrast):
     for e in range(3):
         ref = element_matrices(op.coords[e], N, bp_rule(bp, N), kappa=kappa[e], want=("A",))["A"] @ u[e]
         assert np.linalg.norm(w[e] - ref) < 1e-12 * np.linalg.norm(ref)
+
+
+@pytest.mark.parametrize("bp,N,dims", [(1, 7, (4, 3, 3)), (1, 15, (2, 2, 2)), (2, 9, (2, 2, 1)), (3, 11, (2, 2, 2)), (5, 7, (4, 4, 4)),
+                                       (5, 15, (2, 2, 2)), (6, 9, (2, 2, 2))])
+@pytest.mark.parametrize("weighted", [True, False])
+def test_solves_reach_the_residual_of_fp64(bp, N, dims, weighted):
+    """CG takes uneven directions on the grid the later the further the residual has fallen: the same iteration
+    counts and the same true residual as with every element in FP64, for right-hand sides B f and for values that
+    span the quadrature weights from the first direction on."""
+    op = pkg.Operator.box(bp, *dims, N)
+    _, _, d = pkg.mesh_box(*dims, N)
+    f = torch.from_numpy(uniform_pm1(23, np.arange(op.nglobal * op.ncomp)).reshape(tuple(op.empty().shape))).cuda()
+    b = op.mass(f) if weighted else f
+    if bp > 2:
+        free = torch.from_numpy(1.0 - d).cuda()
+        b = b * (free[:, None] if op.ncomp == 3 else free)
+    out = []
+    for on in (False, True):
+        op.set_fixed_point(on)
+        x, info = op.solve(b, tol=1e-12)
+        op.set_fixed_point(False)
+        out.append((info["iters"], float((b - op.apply(x)).norm() / b.norm())))
+    assert all(abs(i - j) <= 1 for i, j in zip(out[0][0], out[1][0]))
+    assert out[1][1] < 2.0 * out[0][1] + 1e-12
