@@ -1,6 +1,6 @@
 // FP64 BK5 element kernel of batched solves at even orders (the column kernel): w^e = A^e u^e for
-// every element, the unassembled product A_L Q u of Eq. (21).  Batched solves keep FP64 arithmetic for the
-// reason given in elem_eo.cuh, which serves the odd orders.
+// every element, the unassembled product A_L Q u of Eq. (21).  elem_eo.cuh serves the
+// odd orders and says why batches run in FP64.
 //
 // Stiffness, Eq. (22) with J = I: w^e = sum_{m,m'} D_m^T G_mm' D_m' u^e with the
 // geometric factors G of Eq. (23) (six symmetric components per point, stored

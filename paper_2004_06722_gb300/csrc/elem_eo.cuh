@@ -1,10 +1,9 @@
 // FP64 BK5 element kernel of batched solves at odd orders, with the even-odd decomposition of the 1D
 // contractions (the symmetry of Eq. (37); Solomonoff 1992, Kopriva 2009).
 //
-// Batched solves keep this FP64 arithmetic although the fixed-point kernel of single solves
-// (elem_fx.cuh) is faster (32 problems of up to 12^3 elements: 50.8 against 88.1 ms): a batch stops each
-// problem at its residual tolerance after up to 400 iterations, where CG has lost orthogonality and
-// carries any other rounding of A p to 1e-9 of the solution at tolerance 1e-8.
+// Batched solves still run in FP64 instructions, here and in elem_col.cuh: the fixed-point kernel of single solves
+// (elem_fx.cuh) has no block tables yet.  The FP64 pipe bounds them, and one solve after the other is faster
+// (64 problems of 2^3 to 16^3 elements, orders 3, 5 and 7, to 1e-8: 0.70 s together, 0.54 s one by one).
 //
 // The GLL derivative matrix D and its transpose are centro-antisymmetric:
 // D[p1-1-i][p1-1-j] = -D[i][j].  With h = p1/2 (even p1), x+_j = x_j + x_{p1-1-j},
