@@ -67,8 +67,10 @@ enum {
   CEEDBP_ARITH_FP64 = 0, /* FP64 in and out; contractions on 60-bit integers on a grid of each
                             element, in FP64 where an element's values or factors are too
                             uneven for it: every entry of A_e u_e is within a few units of
-                            2^-53 (|A_e| |u_e|)_i either way.  ceedbp_set_fixed_point(ctx, 0)
-                            runs everything in FP64; batched solves always do. */
+                            2^-53 (|A_e| |u_e|)_i either way (in a solve up to norm(b) / norm(r)
+                            times that, which CG does not see in its residual).
+                            ceedbp_set_fixed_point(ctx, 0) runs everything in FP64; batched
+                            solves always do. */
   CEEDBP_ARITH_DF64 = 1  /* FP64-accurate pairs of FP32 numbers (hi + lo, ~2^-46 relative per
                             value) on the FP32 pipe, which the GB300 issues 63x faster than
                             FP64; BP1, BP3, BP5 and BP6 (EUNSUPPORTED for BP2 and BP4).

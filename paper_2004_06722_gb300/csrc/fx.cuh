@@ -19,10 +19,10 @@
 // partial sum.  The bound of a derivative (the largest row sum of |D|) can exceed the actual values by
 // 2^8; the gradient keeps enough bits for that, but the fluxes G grad u are moved up to 2^60 again by
 // the element's actual maximum before the transposes, so that the two derivatives' slack does not add
-// up (fx_limbs_up).  With that the error of one application, against quad-precision references, stays
-// at or below that of the FP64 kernels this arithmetic replaces.  Values a grid cannot hold
+// up (fx_limbs_up).  With that the error of one application on even elements, against quad-precision
+// references, is 0.9-1.2 of that of the FP64 kernels this arithmetic replaces.  Values a grid cannot hold
 // (infinities, NaN, elements whose factors spread over more than 2^5 (fx_setup.cu), exponents near the ends
-// of the FP64 range) take the FP64 form of the same kernel (the double overloads below).
+// of the FP64 range) and uneven elements (below) take the FP64 form of the same kernel (the double overloads).
 #pragma once
 
 #include "common.cuh"
@@ -179,7 +179,7 @@ struct FxTop {
 // The word of a stage's largest magnitude that says so: the check needs no barrier of its own.  What it costs
 // where elements are even: 0.8 % of a BP5 iteration at N = 7, 32^3 elements, nothing of BP3's (25^3), 1.3 % of BP1's
 // at N = 3.  At N = 15 the elements along the edges of a Dirichlet boundary are uneven (values fall with the
-// distance of the first node from two faces): 14 % of BP5, 10^3 elements.
+// distance of the first node from two faces): 7 % of BP5, 10^3 elements.
 constexpr unsigned kFxUneven = 0x80000000u;
 
 // The smallest upper word that reaches (any value of an element of zeros).
